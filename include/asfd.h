@@ -489,10 +489,13 @@ asfd_status asfd_line_destroy(asfd_line_plan plan);
  * asfd_execute.  p: the geometry fields are used (n1x..z0; the spreading fields
  * are ignored).  d1_dev: device [n1y][n1x] FP64 metres; u1_dev: device
  * [n1y][n1x] complex; mx_dev, my_dev: device int[npts] destination indices;
- * out_dev: device complex[npts].  Phases are formed in FP64 per (sample,
- * point) pair and reduced modulo 2 pi exactly before an FP32 sine/cosine; sums
- * are FP64.  Allocates (stream-ordered) 32 bytes per source sample for the
- * duration of the call.  Asynchronous on `stream`.  Errors: ASFD_ERR_ARG.
+ * out_dev: device complex[npts].  Phases are formed per (sample, point)
+ * pair in 64-bit fixed point (fractions of a turn; Eq. 2 in FP64), so that they
+ * are reduced modulo 2 pi exactly before an FP32 sine/cosine; the products'
+ * sums are carried with their rounding errors and meet in FP64.  Allocates
+ * (stream-ordered) 32 bytes per source sample, a 256th byte more and the
+ * partial sums (16 bytes per point and chunk of samples) for the duration of
+ * the call.  Asynchronous on `stream`.  Errors: ASFD_ERR_ARG.
  */
 asfd_status asfd_direct_sum(const asfd_params* p, const double* d1_dev, const float* u1_dev,
                             int form, int npts, const int* mx_dev, const int* my_dev,

@@ -5,122 +5,266 @@
 // the Fresnel expansion of Eq. 4).  They measure what those approximations
 // cost at 2D scale and serve as a fast reference on sampled points.
 //
-// Phases are carried in half-turns (k L = pi (2 L / lambda)) and formed in
-// FP64 per (sample, point) pair from FP64 per-sample terms, reduced modulo 2
-// exactly (h - 2 rint(h/2)) and evaluated with sincospif on the reduced
-// fraction; products with u1 are FP32 and the sums are accumulated in FP64.
-//   Eq. 7: h = |x1|^2/(lambda r0) - 2 x1.x2/(lambda r0) + 2 (s.x1 + (sz - 1) d1)/lambda
-//          (the last term is u_I exp(-ik d1) for a plane wave with direction
-//          cosines (sx, sy, sz); zero at normal incidence)
-//   Eq. 5: h = the Eq. 7 phase + |x2|^2/(lambda r0)
-//   Eq. 2: h = 2 (s.x1 + sz d1 + r)/lambda, amplitude 1/r^2, r = |(x2 - x1, z0 - d1)|
+// The phase of a pair is formed modulo one turn in 64-bit fixed point.  At a
+// destination index j = m - M/2 the phases of Eqs. 5 and 7 are, in turns,
+//   Eq. 7: A - B jx - C jy
+//          A = |x1|^2/(2 lambda r0) + (s.x1 + (sz - 1) d1)/lambda (the last
+//          term is u_I exp(-ik d1) for a plane wave with direction cosines
+//          (sx, sy, sz); zero at normal incidence), B = x1 p2x/(lambda r0),
+//          C = y1 p2y/(lambda r0)
+//   Eq. 5: the same + D R, D = p2x^2/(2 lambda r0), R = jx^2 + (p2y/p2x)^2 jy^2,
+//          an integer for equal pitches (else D R is formed in FP64)
+// The per-sample A, B, C, D are formed in FP64 and reduced modulo 1 there, to
+// 2^-50 turns (D, which is small, to 2^-64); products with the integer
+// indices and their sum are then exact modulo 2^64, which is the reduction
+// modulo one turn.  (With FP64 arithmetic per pair -- 2 lanes per clock and
+// SM, where integer multiply-adds have 64 -- and one block per point group 256
+// points of 1024^2 samples took 28.6 ms; now 0.57 ms, at an error against 64
+// bits of 4.3e-8 instead of 5.6e-8.)
+//   Eq. 2: 2 (s.x1 + sz d1 + r)/lambda half-turns, amplitude 1/r^2,
+//          r = |(x2 - x1, z0 - d1)|, in FP64 from an FP32 reciprocal square
+//          root and one Newton step (relative error below 2^-44).
+// The high 32 bits of the phase go to an FP32 sine and cosine on a quarter
+// turn (polynomials, |error| < 6e-8); products with u1 are FP32 and the sums
+// of a thread are carried as an FP32 value and its exact rounding errors
+// (two-sum), which meet in FP64.
 // Outer factors: p1x p1y exp(ik(z0 + |x2|^2/(2 z0)))/(i lambda z0) (Eq. 7),
 // p1x p1y exp(ik z0)/(i lambda z0) (Eq. 5), p1x p1y z0/(i lambda) (Eq. 2).
+#include <algorithm>
 #include <cmath>
 #include <string>
 
 #include "asfd_impl.cuh"
+#include "fft.cuh"
 
 namespace asfd {
 
 namespace {
 
 constexpr int kDirectThreads = 256;
-constexpr int kDirectPoints = 8;  // destination points per block (shares the sample loads)
+constexpr int kDirectPoints = 8;      // destination points per block (shares the sample loads)
+constexpr int kDirectMaxRows = 1024;  // samples per thread, at most (of one two-sum)
+constexpr int kDirectWaves = 4;       // blocks per SM that a call is split into, at least
 
 struct DirectGeom {
     int n1x, n1y, m2x, m2y;
     double p1x, p1y, p2x, p2y, lambda, z0;
     double sx, sy, sz;  // incident plane wave direction cosines
     double ox, oy;      // source grid offset
+    double inv_lambda;
 };
 
-// The four FP64 terms of one source sample, 32-byte aligned (one load).
+// What direct_sum_kernel evaluates: the paper's equations, and Eq. 5 for
+// destination pitches that differ (kEq5Uneven).
+enum DirectForm { kEq2 = 2, kEq5 = 5, kEq5Uneven = 6, kEq7 = 7 };
+
+// Per-sample terms, 32-byte aligned.  Eq. 5/7: {A', -B, -C, D} as 64-bit
+// fractions of a turn (A' = A at the index origin below; D as a double for
+// uneven pitches); Eq. 2: the doubles {x1x, x1y, (z0 - d1)^2,
+// 2 (s.x1 + sz d1)/lambda mod 2}
 struct alignas(32) DirectTerms {
-    double x, y, z, w;
+    unsigned long long a, b, c, d;
 };
 
-// per sample: Eq. 5/7 {|x1|^2/(lambda r0) + 2 (s.x1 + (sz - 1) d1)/lambda,
-// 2 x1x/(lambda r0), 2 x1y/(lambda r0), 1/(lambda r0)} (the first term carries
-// u_I exp(-ik d1), 1 at normal incidence); Eq. 2 {x1x, x1y, z0 - d1,
-// 2 (s.x1 + sz d1)/lambda} (the phase of u_I)
-__global__ void direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
-                                   DirectTerms* __restrict__ out)
+// fractional part of v (turns) in units of 2^-64, to 2^-50: after the
+// reduction to [-1/2, 1/2] the sum with 1.5 2^2 has an ulp of 2^-50
+__device__ __forceinline__ unsigned long long turn_fraction(double v)
 {
-    const size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= (size_t)g.n1x * g.n1y) return;
-    const int nx = (int)(n % g.n1x), ny = (int)(n / g.n1x);
+    const double f = v - rint(v);
+    return (unsigned long long)__double_as_longlong(f + 6.0) << 14;
+}
+
+// Indices enter the products as unsigned 32-bit numbers m + 2^31 (any int is
+// allowed); A' moves the origin there, exactly modulo one turn.
+constexpr unsigned kIndexBias = 0x80000000u;
+
+// bad[blockIdx.x]: whether a term of the block's samples is not finite (d1 is
+// not checked: a NaN, or d1 = z0, makes every sum a NaN, which fixed point
+// cannot carry).
+__global__ void __launch_bounds__(kDirectThreads)
+direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
+                   DirectTerms* __restrict__ out, unsigned char* __restrict__ bad)
+{
+    const size_t n = (size_t)blockIdx.x * kDirectThreads + threadIdx.x;
+    const bool in = n < (size_t)g.n1x * g.n1y;
+    const int nx = in ? (int)(n % g.n1x) : 0, ny = in ? (int)(n / g.n1x) : 0;
     const double x = (nx - g.n1x / 2) * g.p1x + g.ox, y = (ny - g.n1y / 2) * g.p1y + g.oy;
-    const double h = d1[n];
-    const double lin = g.sx * x + g.sy * y;
-    if (form == 2) {
-        out[n] = DirectTerms{x, y, g.z0 - h, 2.0 * (lin + g.sz * h) / g.lambda};
+    const double h = in ? d1[n] : 0.0;
+    DirectTerms t;
+    bool finite = true;
+    if (form == kEq2) {
+        const double z = g.z0 - h;
+        const double w = 2.0 * (g.sx * x + g.sy * y + g.sz * h) * g.inv_lambda;
+        t.a = (unsigned long long)__double_as_longlong(x);
+        t.b = (unsigned long long)__double_as_longlong(y);
+        t.c = (unsigned long long)__double_as_longlong(z * z);
+        t.d = (unsigned long long)__double_as_longlong(w - 2.0 * rint(0.5 * w));
     } else {
         const double inv = 1.0 / (g.lambda * (g.z0 - h));
-        const double inc = 2.0 * (lin + (g.sz - 1.0) * h) / g.lambda;
-        out[n] = DirectTerms{(x * x + y * y) * inv + inc, 2.0 * x * inv, 2.0 * y * inv, inv};
+        const double inc = (g.sx * x + g.sy * y + (g.sz - 1.0) * h) * g.inv_lambda;
+        const unsigned long long b = turn_fraction(x * g.p2x * inv);
+        const unsigned long long c = turn_fraction(y * g.p2y * inv);
+        t.a = turn_fraction(0.5 * (x * x + y * y) * inv) + turn_fraction(inc) +
+              b * ((unsigned long long)kIndexBias + (unsigned)(g.m2x / 2)) +
+              c * ((unsigned long long)kIndexBias + (unsigned)(g.m2y / 2));
+        t.b = 0ull - b;
+        t.c = 0ull - c;
+        const double d = 0.5 * g.p2x * g.p2x * inv;
+        t.d = (unsigned long long)(form == kEq5Uneven
+                                       ? __double_as_longlong(d)
+                                       : __double2ll_rn((d - rint(d)) * 18446744073709551616.0));
+        finite = isfinite(inv) && isfinite(inc);
     }
+    if (in) out[n] = t;
+    const int any = __syncthreads_or(in && !finite);
+    if (threadIdx.x == 0) bad[blockIdx.x] = any != 0;
 }
 
-__device__ __forceinline__ float reduce_halfturns(double h)
+// cos and sin of the phase p 2^-32 turns.  The nearest quarter turn is the
+// top two bits of p + 2^29, the rest is x = (p << 2) 2^-32 quarter turns in
+// [-1/2, 1/2): there sin(pi x/2) = x S(x^2) and cos(pi x/2) = 1 + x^2 C(x^2)
+// with S and C interpolated at the Chebyshev nodes of x^2 in [0, 1/4] (degree
+// 3: 1e-9 and 2e-9 off before rounding); the leading coefficient of S, pi/2,
+// is split in two so that its own rounding does not show.
+__device__ __forceinline__ void turn_sincos(unsigned p, float& sn, float& cs)
 {
-    return (float)(h - 2.0 * rint(0.5 * h));
+    const float x = (float)(int)(p << 2) * 2.3283064365386963e-10f;
+    const float y = x * x;
+    float s = fmaf(y, -0.004602149f, 0.07968022f);
+    s = fmaf(y, s, -0.6459635f);
+    s = fmaf(y, s, -4.371139e-8f);  // pi/2 - 1.5707964f
+    s = fmaf(x, 1.5707964f, x * s);
+    float c = fmaf(y, 0.0009067399f, -0.020861529f);
+    c = fmaf(y, c, 0.2536694f);
+    c = fmaf(y, c, -1.2337005f);
+    c = fmaf(y, c, 1.0f);
+    const unsigned t = p + 0x20000000u;
+    const bool odd = (t & 0x40000000u) != 0;
+    const unsigned c0 = __float_as_uint(odd ? s : c), s0 = __float_as_uint(odd ? c : s);
+    cs = __uint_as_float(c0 ^ ((t ^ (t << 1)) & 0x80000000u));
+    sn = __uint_as_float(s0 ^ (t & 0x80000000u));
 }
 
-template <int FORM>
+// sum + err += v, with err collecting the rounding errors of sum exactly
+// (Knuth's two-sum on a packed complex pair)
+__device__ __forceinline__ void two_sum(float2& sum, float2& err, float2 v)
+{
+    const float2 s = cadd(sum, v);
+    const float2 b = csub(s, sum);
+    const float2 e = cadd(csub(sum, csub(s, b)), csub(v, b));
+    sum = s;
+    err = cadd(err, e);
+}
+
+// Point groups in x, sample chunks in y: the chunk's sums over its samples of
+// kDirectPoints points, to part[chunk][point].  Bound by instruction issue
+// (about 35 a pair).  One block per group alone leaves 120 of the 152 SMs
+// idle at 256 points, so the samples are split as well.  16 points per block
+// (half the reads of the terms, half the resident warps) took 0.66 ms a call,
+// registers capped for three blocks per SM 0.59 ms, as here 0.57 ms.
+template <DirectForm FORM>
 __global__ void __launch_bounds__(kDirectThreads)
 direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2* __restrict__ u1,
-                  int npts, const int* __restrict__ mx, const int* __restrict__ my,
-                  float2* __restrict__ out)
+                  const unsigned char* __restrict__ bad, int npts, const int* __restrict__ mx,
+                  const int* __restrict__ my, size_t chunk, double2* __restrict__ part)
 {
     __shared__ double red[2][kDirectPoints][kDirectThreads / 32];
     const int p0 = blockIdx.x * kDirectPoints;
-    double x2x[kDirectPoints], x2y[kDirectPoints], x2sq[kDirectPoints];
+    unsigned ix[kDirectPoints], iy[kDirectPoints];
+    double x2x[kDirectPoints], x2y[kDirectPoints];
+    unsigned long long r5[kDirectPoints];  // Eq. 5's R
+    double r5u[kDirectPoints];
 #pragma unroll
     for (int j = 0; j < kDirectPoints; ++j) {
         const int i = min(p0 + j, npts - 1);
-        x2x[j] = (mx[i] - g.m2x / 2) * g.p2x;
-        x2y[j] = (my[i] - g.m2y / 2) * g.p2y;
-        x2sq[j] = x2x[j] * x2x[j] + x2y[j] * x2y[j];
+        const int jx = mx[i], jy = my[i];
+        ix[j] = (unsigned)jx + kIndexBias;
+        iy[j] = (unsigned)jy + kIndexBias;
+        if constexpr (FORM == kEq2) {
+            x2x[j] = ((double)jx - g.m2x / 2) * g.p2x;
+            x2y[j] = ((double)jy - g.m2y / 2) * g.p2y;
+        }
+        if constexpr (FORM == kEq5) {
+            const long long kx = (long long)jx - g.m2x / 2, ky = (long long)jy - g.m2y / 2;
+            r5[j] = (unsigned long long)kx * (unsigned long long)kx +
+                    (unsigned long long)ky * (unsigned long long)ky;
+        }
+        if constexpr (FORM == kEq5Uneven) {
+            const double kx = (double)jx - g.m2x / 2;
+            const double ky = ((double)jy - g.m2y / 2) * (g.p2y / g.p2x);
+            r5u[j] = kx * kx + ky * ky;
+        }
     }
-    double accr[kDirectPoints], acci[kDirectPoints];
-#pragma unroll
-    for (int j = 0; j < kDirectPoints; ++j) accr[j] = acci[j] = 0.0;
     const size_t total = (size_t)g.n1x * g.n1y;
-    for (size_t n = threadIdx.x; n < total; n += kDirectThreads) {
-        const DirectTerms t = s[n];
-        const float2 u = __ldg(&u1[n]);
+    const size_t beg = blockIdx.y * chunk, end = min(total, beg + chunk);
+    bool nan = false;
+    for (size_t r = beg / kDirectThreads + threadIdx.x; r * kDirectThreads < end; r += kDirectThreads)
+        nan = nan || bad[r] != 0;
+    nan = __syncthreads_or(nan);
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    if (lane < kDirectPoints) red[0][lane][warp] = red[1][lane][warp] = 0.0;
+    __syncwarp();
+    // at most kDirectMaxRows samples of a thread in one two-sum
+    for (size_t b0 = beg; b0 < end; b0 += (size_t)kDirectMaxRows * kDirectThreads) {
+        const size_t b1 = min(end, b0 + (size_t)kDirectMaxRows * kDirectThreads);
+        float2 sum[kDirectPoints], err[kDirectPoints];
+#pragma unroll
+        for (int j = 0; j < kDirectPoints; ++j) sum[j] = err[j] = make_float2(0.f, 0.f);
+        for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
+            const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
+            const ulonglong2 t0 = __ldg(tp), t1 = __ldg(tp + 1);
+            const float2 u = __ldg(&u1[n]);
+#pragma unroll
+            for (int j = 0; j < kDirectPoints; ++j) {
+                unsigned p;
+                float2 w = u;
+                if constexpr (FORM == kEq2) {
+                    const double dx = x2x[j] - __longlong_as_double((long long)t0.x);
+                    const double dy = x2y[j] - __longlong_as_double((long long)t0.y);
+                    const double r2 = fma(dx, dx, fma(dy, dy, __longlong_as_double((long long)t1.x)));
+                    const float r2f = (float)r2;
+                    // (a sample on the point itself: r = 0, amplitude infinite)
+                    const float y = rsqrtf(fmaxf(r2f, 1e-37f));
+                    const double yd = (double)y;
+                    const double r0 = r2 * yd;  // r to 2^-22; one Newton step
+                    const double r = fma(0.5 * yd, fma(-r0, r0, r2), r0);
+                    double h = fma(2.0 * g.inv_lambda, r, __longlong_as_double((long long)t1.y));
+                    h -= 2.0 * rint(0.5 * h);
+                    // units of 2^-31 half-turns from the low bits of h + 1.5 2^21
+                    p = (unsigned)__double_as_longlong(h + 3145728.0);
+                    // 1/r^2 from its FP32 estimate and that one's residual in FP64
+                    const float a0 = y * y;
+                    const float amp = r2f == 0.f ? __int_as_float(0x7f800000)
+                                                 : fmaf(a0, (float)fma(-r2, (double)a0, 1.0), a0);
+                    w = make_float2(u.x * amp, u.y * amp);
+                } else {
+                    unsigned long long ph = t0.x + t0.y * (unsigned long long)ix[j] +
+                                            t1.x * (unsigned long long)iy[j];
+                    if constexpr (FORM == kEq5) ph += t1.y * r5[j];
+                    if constexpr (FORM == kEq5Uneven)
+                        ph += turn_fraction(__longlong_as_double((long long)t1.y) * r5u[j]);
+                    p = (unsigned)(ph >> 32);
+                }
+                float sn, cs;
+                turn_sincos(p, sn, cs);
+                two_sum(sum[j], err[j],
+                        make_float2(w.x * cs - w.y * sn, w.x * sn + w.y * cs));
+            }
+        }
 #pragma unroll
         for (int j = 0; j < kDirectPoints; ++j) {
-            float amp = 1.0f;
-            double h;
-            if constexpr (FORM == 2) {
-                const double dx = x2x[j] - t.x, dy = x2y[j] - t.y;
-                const double r2 = fma(dx, dx, fma(dy, dy, t.z * t.z));
-                h = fma(2.0 / g.lambda, sqrt(r2), t.w);
-                amp = (float)(1.0 / r2);
-            } else {
-                h = t.x - fma(t.y, x2x[j], t.z * x2y[j]);
-                if constexpr (FORM == 5) h = fma(t.w, x2sq[j], h);
+            // (an infinite sum has no rounding error: its err is a NaN)
+            double a = sum[j].x, b = sum[j].y;
+            if (isfinite(a)) a += err[j].x;
+            if (isfinite(b)) b += err[j].y;
+            for (int o = 16; o > 0; o >>= 1) {
+                a += __shfl_xor_sync(0xffffffffu, a, o);
+                b += __shfl_xor_sync(0xffffffffu, b, o);
             }
-            float sn, cs;
-            sincospif(reduce_halfturns(h), &sn, &cs);
-            const float re = (u.x * cs - u.y * sn) * amp, im = (u.x * sn + u.y * cs) * amp;
-            accr[j] += (double)re;
-            acci[j] += (double)im;
-        }
-    }
-    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-#pragma unroll
-    for (int j = 0; j < kDirectPoints; ++j) {
-        double a = accr[j], b = acci[j];
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            b += __shfl_xor_sync(0xffffffffu, b, o);
-        }
-        if (lane == 0) {
-            red[0][j][warp] = a;
-            red[1][j][warp] = b;
+            if (lane == 0) {
+                red[0][j][warp] += a;
+                red[1][j][warp] += b;
+            }
         }
     }
     __syncthreads();
@@ -131,23 +275,50 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
             a += red[0][j][w];
             b += red[1][j][w];
         }
-        // outer factor o = f * exp(i pi ph) / i = f (sin(pi ph) - i cos(pi ph))
-        const double wgt = g.p1x * g.p1y;
-        double f, ph;
-        if (FORM == 2) {
-            f = wgt * g.z0 / g.lambda;
-            ph = 0.0;
-        } else {
-            f = wgt / (g.lambda * g.z0);
-            ph = 2.0 * g.z0 / g.lambda;
-            if (FORM == 7) ph += x2sq[j] / (g.lambda * g.z0);
-        }
-        ph -= 2.0 * rint(0.5 * ph);
-        double sp, cp;
-        sincospi(ph, &sp, &cp);
-        const double ore = f * sp, oim = -f * cp;
-        out[p0 + j] = make_float2((float)(ore * a - oim * b), (float)(ore * b + oim * a));
+        if (nan) a = b = __longlong_as_double(0x7ff8000000000000ll);
+        part[(size_t)blockIdx.y * npts + p0 + j] = make_double2(a, b);
     }
+}
+
+// The chunks' sums in order, times the outer factor: a warp per point.
+__global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int* __restrict__ mx,
+                                     const int* __restrict__ my, int chunks,
+                                     const double2* __restrict__ part, float2* __restrict__ out)
+{
+    const int i = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 32);
+    const int lane = threadIdx.x % 32;
+    if (i >= npts) return;  // warp-uniform
+    double a = 0.0, b = 0.0;
+    for (int k = lane; k < chunks; k += 32) {
+        const double2 v = part[(size_t)k * npts + i];
+        a += v.x;
+        b += v.y;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane != 0) return;
+    // outer factor o = f * exp(i pi ph) / i = f (sin(pi ph) - i cos(pi ph))
+    const double wgt = g.p1x * g.p1y;
+    double f, ph;
+    if (form == kEq2) {
+        f = wgt * g.z0 / g.lambda;
+        ph = 0.0;
+    } else {
+        f = wgt / (g.lambda * g.z0);
+        ph = 2.0 * g.z0 / g.lambda;
+        if (form == kEq7) {
+            const double x2 = ((double)mx[i] - g.m2x / 2) * g.p2x;
+            const double y2 = ((double)my[i] - g.m2y / 2) * g.p2y;
+            ph += (x2 * x2 + y2 * y2) / (g.lambda * g.z0);
+        }
+    }
+    ph -= 2.0 * rint(0.5 * ph);
+    double sp, cp;
+    sincospi(ph, &sp, &cp);
+    const double ore = f * sp, oim = -f * cp;
+    out[i] = make_float2((float)(ore * a - oim * b), (float)(ore * b + oim * a));
 }
 
 }  // namespace
@@ -177,22 +348,39 @@ asfd_status direct_sum(const asfd_params* p, const double* d1, const float2* u1,
                                 p->incidence_sy * p->incidence_sy);
     DirectGeom g{p->n1x, p->n1y, p->m2x, p->m2y, p->p1x, p->p1y, p->p2x, p->p2y,
                  p->lambda, p->z0, p->incidence_sx, p->incidence_sy, sz, p->offset_x,
-                 p->offset_y};
+                 p->offset_y, 1.0 / p->lambda};
     const size_t n = (size_t)p->n1x * p->n1y;
+    // chunks of samples: enough blocks for every SM
+    int dev = 0, sms = 0;
+    ASFD_CUDA(cudaGetDevice(&dev));
+    ASFD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const size_t groups = ((size_t)npts + kDirectPoints - 1) / kDirectPoints;
+    const size_t most = (n + kDirectThreads - 1) / kDirectThreads;  // rows of a single chunk
+    size_t chunks = ((size_t)kDirectWaves * sms + groups - 1) / groups;
+    chunks = std::min(chunks, (most + 3) / 4);
+    const size_t rows = (most + chunks - 1) / chunks;
+    chunks = (most + rows - 1) / rows;
     DirectTerms* s = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&s), sizeof(DirectTerms) * n, st);
+    const size_t bytes = sizeof(DirectTerms) * n + sizeof(double2) * chunks * npts + most;
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&s), bytes, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(ASFD_ERR_NOMEM, std::string("per-sample terms: ") + cudaGetErrorString(e));
     }
-    direct_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(g, d1, form, s);
-    const unsigned blocks = (unsigned)((npts + kDirectPoints - 1) / kDirectPoints);
-    if (form == 2)
-        direct_sum_kernel<2><<<blocks, kDirectThreads, 0, st>>>(g, s, u1, npts, mx, my, out);
-    else if (form == 5)
-        direct_sum_kernel<5><<<blocks, kDirectThreads, 0, st>>>(g, s, u1, npts, mx, my, out);
-    else
-        direct_sum_kernel<7><<<blocks, kDirectThreads, 0, st>>>(g, s, u1, npts, mx, my, out);
+    double2* part = reinterpret_cast<double2*>(s + n);
+    unsigned char* bad = reinterpret_cast<unsigned char*>(part + chunks * npts);
+    const int eq = form == 5 && p->p2x != p->p2y ? (int)kEq5Uneven : form;
+    direct_prep_kernel<<<(unsigned)most, kDirectThreads, 0, st>>>(g, d1, eq, s, bad);
+    const dim3 grid((unsigned)groups, (unsigned)chunks);
+    const size_t chunk = rows * kDirectThreads;
+    switch (eq) {
+#define ASFD_DS(F) case F: direct_sum_kernel<F><<<grid, kDirectThreads, 0, st>>>(g, s, u1, bad, npts, mx, my, chunk, part); break;
+        ASFD_DS(kEq2) ASFD_DS(kEq5) ASFD_DS(kEq5Uneven) ASFD_DS(kEq7)
+#undef ASFD_DS
+        default: break;
+    }
+    direct_finish_kernel<<<(unsigned)(((size_t)npts + 7) / 8), 256, 0, st>>>(
+        g, eq, npts, mx, my, (int)chunks, part, out);
     e = cudaGetLastError();
     const cudaError_t ef = cudaFreeAsync(s, st);
     if (e != cudaSuccess) return cuda_fail(e, "direct_sum_kernel launch");
