@@ -19,8 +19,8 @@
 // indices and their sum are then exact modulo 2^64, which is the reduction
 // modulo one turn.  (With FP64 arithmetic per pair -- 2 lanes per clock and
 // SM, where integer multiply-adds have 64 -- and one block per point group 256
-// points of 1024^2 samples took 28.6 ms; now 0.57 ms, at an error against 64
-// bits of 4.3e-8 instead of 5.6e-8.)
+// points of 1024^2 samples took 28.6 ms; now 0.45 ms, at an error against 64
+// bits of 5.1e-8 instead of 6.2e-8.)
 //   Eq. 2: 2 (s.x1 + sz d1 + r)/lambda half-turns, amplitude 1/r^2,
 //          r = |(x2 - x1, z0 - d1)|, in FP64 from an FP32 reciprocal square
 //          root and one Newton step (relative error below 2^-44).
@@ -43,8 +43,8 @@ namespace {
 
 constexpr int kDirectThreads = 256;
 constexpr int kDirectPoints = 8;      // destination points per block (shares the sample loads)
+constexpr int kDirectBlocks = 4;      // blocks per SM that the samples are split into
 constexpr int kDirectMaxRows = 1024;  // samples per thread, at most (of one two-sum)
-constexpr int kDirectWaves = 4;       // blocks per SM that a call is split into, at least
 
 struct DirectGeom {
     int n1x, n1y, m2x, m2y;
@@ -78,66 +78,75 @@ __device__ __forceinline__ unsigned long long turn_fraction(double v)
 // allowed); A' moves the origin there, exactly modulo one turn.
 constexpr unsigned kIndexBias = 0x80000000u;
 
-// bad[blockIdx.x]: whether a term of the block's samples is not finite (d1 is
-// not checked: a NaN, or d1 = z0, makes every sum a NaN, which fixed point
-// cannot carry).
-__global__ void __launch_bounds__(kDirectThreads)
+// A block takes 256 columns x kPrepRows rows: a thread's column terms serve its
+// rows, the rows' terms are formed once per block (FP64 is 2 lanes per clock
+// and SM: 45 FP64 operations per sample in a thread each took 90 us at 1024^2).
+// *bad is set when a term is not finite (d1 is not checked: a NaN, or d1 =
+// z0, makes every sum a NaN, which fixed point cannot carry).
+constexpr int kPrepRows = 8;
+
+__global__ void __launch_bounds__(256)
 direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
-                   DirectTerms* __restrict__ out, unsigned char* __restrict__ bad)
+                   DirectTerms* __restrict__ out, unsigned* __restrict__ bad)
 {
-    const size_t n = (size_t)blockIdx.x * kDirectThreads + threadIdx.x;
-    const bool in = n < (size_t)g.n1x * g.n1y;
-    const int nx = in ? (int)(n % g.n1x) : 0, ny = in ? (int)(n / g.n1x) : 0;
-    const double x = (nx - g.n1x / 2) * g.p1x + g.ox, y = (ny - g.n1y / 2) * g.p1y + g.oy;
-    const double h = in ? d1[n] : 0.0;
-    DirectTerms t;
-    bool finite = true;
-    if (form == kEq2) {
-        const double z = g.z0 - h;
-        const double w = 2.0 * (g.sx * x + g.sy * y + g.sz * h) * g.inv_lambda;
-        t.a = (unsigned long long)__double_as_longlong(x);
-        t.b = (unsigned long long)__double_as_longlong(y);
-        t.c = (unsigned long long)__double_as_longlong(z * z);
-        t.d = (unsigned long long)__double_as_longlong(w - 2.0 * rint(0.5 * w));
-    } else {
-        const double inv = 1.0 / (g.lambda * (g.z0 - h));
-        const double inc = (g.sx * x + g.sy * y + (g.sz - 1.0) * h) * g.inv_lambda;
-        const unsigned long long b = turn_fraction(x * g.p2x * inv);
-        const unsigned long long c = turn_fraction(y * g.p2y * inv);
-        t.a = turn_fraction(0.5 * (x * x + y * y) * inv) + turn_fraction(inc) +
-              b * ((unsigned long long)kIndexBias + (unsigned)(g.m2x / 2)) +
-              c * ((unsigned long long)kIndexBias + (unsigned)(g.m2y / 2));
-        t.b = 0ull - b;
-        t.c = 0ull - c;
-        const double d = 0.5 * g.p2x * g.p2x * inv;
-        t.d = (unsigned long long)(form == kEq5Uneven
-                                       ? __double_as_longlong(d)
-                                       : __double2ll_rn((d - rint(d)) * 18446744073709551616.0));
-        finite = isfinite(inv) && isfinite(inc);
+    __shared__ double ys[kPrepRows];
+    const int nx = blockIdx.x * 256 + threadIdx.x, ny0 = blockIdx.y * kPrepRows;
+    if (threadIdx.x < kPrepRows)
+        ys[threadIdx.x] = (ny0 + (int)threadIdx.x - g.n1y / 2) * g.p1y + g.oy;
+    __syncthreads();
+    if (nx >= g.n1x) return;
+    const double x = (nx - g.n1x / 2) * g.p1x + g.ox;
+    const double xx = x * x, xp = x * g.p2x, half_pp = 0.5 * g.p2x * g.p2x;
+    const bool tilted = g.sx != 0.0 || g.sy != 0.0;
+    const int rows = min(kPrepRows, g.n1y - ny0);
+    for (int r = 0; r < rows; ++r) {
+        const size_t n = (size_t)(ny0 + r) * g.n1x + nx;
+        const double y = ys[r], h = d1[n];
+        DirectTerms t;
+        if (form == kEq2) {
+            const double z = g.z0 - h;
+            const double w = 2.0 * (g.sx * x + g.sy * y + g.sz * h) * g.inv_lambda;
+            t.a = (unsigned long long)__double_as_longlong(x);
+            t.b = (unsigned long long)__double_as_longlong(y);
+            t.c = (unsigned long long)__double_as_longlong(z * z);
+            t.d = (unsigned long long)__double_as_longlong(w - 2.0 * rint(0.5 * w));
+        } else {
+            const double inv = 1.0 / (g.lambda * (g.z0 - h));
+            const unsigned long long b = turn_fraction(xp * inv);
+            const unsigned long long c = turn_fraction(y * g.p2y * inv);
+            t.a = turn_fraction(0.5 * (xx + y * y) * inv) +
+                  b * ((unsigned long long)kIndexBias + (unsigned)(g.m2x / 2)) +
+                  c * ((unsigned long long)kIndexBias + (unsigned)(g.m2y / 2));
+            if (tilted)
+                t.a += turn_fraction((g.sx * x + g.sy * y + (g.sz - 1.0) * h) * g.inv_lambda);
+            t.b = 0ull - b;
+            t.c = 0ull - c;
+            const double d = half_pp * inv;
+            t.d = 0;
+            if (form == kEq5Uneven)
+                t.d = (unsigned long long)__double_as_longlong(d);
+            else if (form == kEq5)
+                t.d = (unsigned long long)__double2ll_rn((d - rint(d)) * 18446744073709551616.0);
+            if (!isfinite(inv)) atomicOr(bad, 1u);
+        }
+        out[n] = t;
     }
-    if (in) out[n] = t;
-    const int any = __syncthreads_or(in && !finite);
-    if (threadIdx.x == 0) bad[blockIdx.x] = any != 0;
 }
 
-// cos and sin of the phase p 2^-32 turns.  The nearest quarter turn is the
+// cos and sin of two phases p 2^-32 turns.  The nearest quarter turn is the
 // top two bits of p + 2^29, the rest is x = (p << 2) 2^-32 quarter turns in
-// [-1/2, 1/2): there sin(pi x/2) = x S(x^2) and cos(pi x/2) = 1 + x^2 C(x^2)
+// [-1/2, 1/2): there sin(pi x/2) = x S(x^2) and cos(pi x/2) = 1 + x^2 C(x^2),
 // with S and C interpolated at the Chebyshev nodes of x^2 in [0, 1/4] (degree
-// 3: 1e-9 and 2e-9 off before rounding); the leading coefficient of S, pi/2,
-// is split in two so that its own rounding does not show.
-__device__ __forceinline__ void turn_sincos(unsigned p, float& sn, float& cs)
+// 3); the leading coefficient of S, pi/2, is split in two so that its own
+// rounding does not show (rms error 2.4e-8 of a unit vector; 2.1e-8 is the
+// rounding to FP32 alone).  Two points at a time: the polynomials run in
+// packed FP32x2, the choice of the quadrant on the integer pipe.  (Half
+// turns, with longer polynomials and one sign to choose, are no faster and
+// less exact, 3.7e-8: x^2 of a larger x is rounded.)
+__device__ __forceinline__ float2 pair2(float v) { return make_float2(v, v); }
+
+__device__ __forceinline__ void to_quadrant(unsigned p, float s, float c, float& sn, float& cs)
 {
-    const float x = (float)(int)(p << 2) * 2.3283064365386963e-10f;
-    const float y = x * x;
-    float s = fmaf(y, -0.004602149f, 0.07968022f);
-    s = fmaf(y, s, -0.6459635f);
-    s = fmaf(y, s, -4.371139e-8f);  // pi/2 - 1.5707964f
-    s = fmaf(x, 1.5707964f, x * s);
-    float c = fmaf(y, 0.0009067399f, -0.020861529f);
-    c = fmaf(y, c, 0.2536694f);
-    c = fmaf(y, c, -1.2337005f);
-    c = fmaf(y, c, 1.0f);
     const unsigned t = p + 0x20000000u;
     const bool odd = (t & 0x40000000u) != 0;
     const unsigned c0 = __float_as_uint(odd ? s : c), s0 = __float_as_uint(odd ? c : s);
@@ -145,37 +154,62 @@ __device__ __forceinline__ void turn_sincos(unsigned p, float& sn, float& cs)
     sn = __uint_as_float(s0 ^ (t & 0x80000000u));
 }
 
-// sum + err += v, with err collecting the rounding errors of sum exactly
-// (Knuth's two-sum on a packed complex pair)
-__device__ __forceinline__ void two_sum(float2& sum, float2& err, float2 v)
+__device__ __forceinline__ void turn_sincos2(unsigned p0, unsigned p1, float2& sn, float2& cs)
 {
-    const float2 s = cadd(sum, v);
-    const float2 b = csub(s, sum);
-    const float2 e = cadd(csub(sum, csub(s, b)), csub(v, b));
-    sum = s;
-    err = cadd(err, e);
+    const float2 x = mul_f2(make_float2((float)(int)(p0 << 2), (float)(int)(p1 << 2)),
+                            pair2(2.3283064365386963e-10f));
+    const float2 y = mul_f2(x, x);
+    float2 s = fma_f2(y, pair2(-0.004602149f), pair2(0.07968022f));
+    s = fma_f2(y, s, pair2(-0.6459635f));
+    s = fma_f2(y, s, pair2(-4.371139e-8f));  // pi/2 - 1.5707964f
+    s = fma_f2(x, pair2(1.5707964f), mul_f2(x, s));
+    float2 c = fma_f2(y, pair2(0.0009067399f), pair2(-0.020861529f));
+    c = fma_f2(y, c, pair2(0.2536694f));
+    c = fma_f2(y, c, pair2(-1.2337005f));
+    c = fma_f2(y, c, pair2(1.0f));
+    to_quadrant(p0, s.x, c.x, sn.x, cs.x);
+    to_quadrant(p1, s.y, c.y, sn.y, cs.y);
+}
+
+// sum += v on a pair, with the low part of the sum in -low (Kahan)
+__device__ __forceinline__ void kahan_add(float2& sum, float2& low, float2 v)
+{
+    const float2 y = csub(v, low);
+    const float2 t = cadd(sum, y);
+    low = csub(csub(t, sum), y);
+    sum = t;
+}
+
+// Resident blocks per SM (three need Eq. 7's 80 registers)
+__host__ __device__ constexpr int direct_blocks_per_sm(int form)
+{
+    return form == kEq7 ? 3 : 2;
 }
 
 // Point groups in x, sample chunks in y: the chunk's sums over its samples of
-// kDirectPoints points, to part[chunk][point].  Bound by instruction issue
-// (about 35 a pair).  One block per group alone leaves 120 of the 152 SMs
-// idle at 256 points, so the samples are split as well.  16 points per block
-// (half the reads of the terms, half the resident warps) took 0.66 ms a call,
-// registers capped for three blocks per SM 0.59 ms, as here 0.57 ms.
+// kDirectPoints points, to part[chunk][point].  Bound by the FMA pipe and
+// instruction issue together (69 and 55 % busy: 12 packed operations, 4
+// integer multiply-adds and 10 integer operations a pair), so more resident
+// warps, a sample's loads one iteration ahead and one exact wave of blocks
+// made no difference (0.39-0.42 ms against 0.385 ms at 256 points of 1024^2
+// samples).  One block per group alone leaves 120 of the 152 SMs idle there,
+// so the samples are split as well.
 template <DirectForm FORM>
-__global__ void __launch_bounds__(kDirectThreads)
+__global__ void __launch_bounds__(kDirectThreads, direct_blocks_per_sm(FORM))
 direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2* __restrict__ u1,
-                  const unsigned char* __restrict__ bad, int npts, const int* __restrict__ mx,
-                  const int* __restrict__ my, size_t chunk, double2* __restrict__ part)
+                  int npts, const int* __restrict__ mx, const int* __restrict__ my, size_t chunk,
+                  double2* __restrict__ part)
 {
-    __shared__ double red[2][kDirectPoints][kDirectThreads / 32];
-    const int p0 = blockIdx.x * kDirectPoints;
-    unsigned ix[kDirectPoints], iy[kDirectPoints];
-    double x2x[kDirectPoints], x2y[kDirectPoints];
-    unsigned long long r5[kDirectPoints];  // Eq. 5's R
-    double r5u[kDirectPoints];
+    constexpr int P = kDirectPoints;
+    static_assert(P % 2 == 0 && P <= 32, "points in pairs, a lane each for the sums");
+    __shared__ double red[2][P][kDirectThreads / 32];
+    const int p0 = blockIdx.x * P;
+    unsigned ix[P], iy[P];
+    double x2x[P], x2y[P];
+    unsigned long long r5[P];  // Eq. 5's R
+    double r5u[P];
 #pragma unroll
-    for (int j = 0; j < kDirectPoints; ++j) {
+    for (int j = 0; j < P; ++j) {
         const int i = min(p0 + j, npts - 1);
         const int jx = mx[i], jy = my[i];
         ix[j] = (unsigned)jx + kIndexBias;
@@ -195,87 +229,122 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
             r5u[j] = kx * kx + ky * ky;
         }
     }
+    // phase (2^-32 turns) and amplitude of the sample's terms t at point j
+    auto phase = [&](const ulonglong2& t0, const ulonglong2& t1, int j, float& amp) -> unsigned {
+        if constexpr (FORM == kEq2) {
+            const double dx = x2x[j] - __longlong_as_double((long long)t0.x);
+            const double dy = x2y[j] - __longlong_as_double((long long)t0.y);
+            const double r2 = fma(dx, dx, fma(dy, dy, __longlong_as_double((long long)t1.x)));
+            const float r2f = (float)r2;
+            // (a sample on the point itself: r = 0, amplitude infinite)
+            const float y = rsqrtf(fmaxf(r2f, 1e-37f));
+            const double yd = (double)y;
+            const double ra = r2 * yd;  // r to 2^-22; one Newton step
+            const double r = fma(0.5 * yd, fma(-ra, ra, r2), ra);
+            double h = fma(2.0 * g.inv_lambda, r, __longlong_as_double((long long)t1.y));
+            h -= 2.0 * rint(0.5 * h);
+            // 1/r^2 from its FP32 estimate and that one's residual in FP64
+            const float a0 = y * y;
+            amp = r2f == 0.f ? __int_as_float(0x7f800000)
+                             : fmaf(a0, (float)fma(-r2, (double)a0, 1.0), a0);
+            // units of 2^-31 half-turns from the low bits of h + 1.5 2^21
+            return (unsigned)__double_as_longlong(h + 3145728.0);
+        } else {
+            unsigned long long ph = t0.x + t0.y * (unsigned long long)ix[j] +
+                                    t1.x * (unsigned long long)iy[j];
+            if constexpr (FORM == kEq5) ph += t1.y * r5[j];
+            if constexpr (FORM == kEq5Uneven)
+                ph += turn_fraction(__longlong_as_double((long long)t1.y) * r5u[j]);
+            return (unsigned)(ph >> 32);
+        }
+    };
+    // products u exp(2 pi i phase) amp of points j and j + 1
+    auto products = [&](const ulonglong2& t0, const ulonglong2& t1, float2 u, int j, float2& re,
+                        float2& im) {
+        float2 amp = pair2(1.f), sn, cs;
+        const unsigned pa = phase(t0, t1, j, amp.x), pb = phase(t0, t1, j + 1, amp.y);
+        turn_sincos2(pa, pb, sn, cs);
+        float2 ux = pair2(u.x), uy = pair2(u.y);
+        if constexpr (FORM == kEq2) {
+            ux = mul_f2(ux, amp);
+            uy = mul_f2(uy, amp);
+        }
+        re = fma_f2(cs, ux, mul_f2(sn, make_float2(-uy.x, -uy.y)));
+        im = fma_f2(cs, uy, mul_f2(sn, ux));
+    };
     const size_t total = (size_t)g.n1x * g.n1y;
     const size_t beg = blockIdx.y * chunk, end = min(total, beg + chunk);
-    bool nan = false;
-    for (size_t r = beg / kDirectThreads + threadIdx.x; r * kDirectThreads < end; r += kDirectThreads)
-        nan = nan || bad[r] != 0;
-    nan = __syncthreads_or(nan);
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-    if (lane < kDirectPoints) red[0][lane][warp] = red[1][lane][warp] = 0.0;
+    if (lane < P) red[0][lane][warp] = red[1][lane][warp] = 0.0;
     __syncwarp();
-    // at most kDirectMaxRows samples of a thread in one two-sum
+    // at most kDirectMaxRows samples of a thread in one compensated sum
     for (size_t b0 = beg; b0 < end; b0 += (size_t)kDirectMaxRows * kDirectThreads) {
         const size_t b1 = min(end, b0 + (size_t)kDirectMaxRows * kDirectThreads);
-        float2 sum[kDirectPoints], err[kDirectPoints];
+        float2 sr[P / 2], lr[P / 2], si[P / 2], li[P / 2];  // of points 2k and 2k + 1
 #pragma unroll
-        for (int j = 0; j < kDirectPoints; ++j) sum[j] = err[j] = make_float2(0.f, 0.f);
+        for (int k = 0; k < P / 2; ++k) sr[k] = lr[k] = si[k] = li[k] = pair2(0.f);
         for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
             const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
             const ulonglong2 t0 = __ldg(tp), t1 = __ldg(tp + 1);
             const float2 u = __ldg(&u1[n]);
 #pragma unroll
-            for (int j = 0; j < kDirectPoints; ++j) {
-                unsigned p;
-                float2 w = u;
-                if constexpr (FORM == kEq2) {
-                    const double dx = x2x[j] - __longlong_as_double((long long)t0.x);
-                    const double dy = x2y[j] - __longlong_as_double((long long)t0.y);
-                    const double r2 = fma(dx, dx, fma(dy, dy, __longlong_as_double((long long)t1.x)));
-                    const float r2f = (float)r2;
-                    // (a sample on the point itself: r = 0, amplitude infinite)
-                    const float y = rsqrtf(fmaxf(r2f, 1e-37f));
-                    const double yd = (double)y;
-                    const double r0 = r2 * yd;  // r to 2^-22; one Newton step
-                    const double r = fma(0.5 * yd, fma(-r0, r0, r2), r0);
-                    double h = fma(2.0 * g.inv_lambda, r, __longlong_as_double((long long)t1.y));
-                    h -= 2.0 * rint(0.5 * h);
-                    // units of 2^-31 half-turns from the low bits of h + 1.5 2^21
-                    p = (unsigned)__double_as_longlong(h + 3145728.0);
-                    // 1/r^2 from its FP32 estimate and that one's residual in FP64
-                    const float a0 = y * y;
-                    const float amp = r2f == 0.f ? __int_as_float(0x7f800000)
-                                                 : fmaf(a0, (float)fma(-r2, (double)a0, 1.0), a0);
-                    w = make_float2(u.x * amp, u.y * amp);
-                } else {
-                    unsigned long long ph = t0.x + t0.y * (unsigned long long)ix[j] +
-                                            t1.x * (unsigned long long)iy[j];
-                    if constexpr (FORM == kEq5) ph += t1.y * r5[j];
-                    if constexpr (FORM == kEq5Uneven)
-                        ph += turn_fraction(__longlong_as_double((long long)t1.y) * r5u[j]);
-                    p = (unsigned)(ph >> 32);
-                }
-                float sn, cs;
-                turn_sincos(p, sn, cs);
-                two_sum(sum[j], err[j],
-                        make_float2(w.x * cs - w.y * sn, w.x * sn + w.y * cs));
+            for (int k = 0; k < P / 2; ++k) {
+                float2 re, im;
+                products(t0, t1, u, 2 * k, re, im);
+                kahan_add(sr[k], lr[k], re);
+                kahan_add(si[k], li[k], im);
             }
         }
+        double vs[2 * P];  // re and im of each point
 #pragma unroll
-        for (int j = 0; j < kDirectPoints; ++j) {
-            // (an infinite sum has no rounding error: its err is a NaN)
-            double a = sum[j].x, b = sum[j].y;
-            if (isfinite(a)) a += err[j].x;
-            if (isfinite(b)) b += err[j].y;
-            for (int o = 16; o > 0; o >>= 1) {
-                a += __shfl_xor_sync(0xffffffffu, a, o);
-                b += __shfl_xor_sync(0xffffffffu, b, o);
+        for (int k = 0; k < P / 2; ++k) {
+            double v[4] = {(double)sr[k].x - lr[k].x, (double)si[k].x - li[k].x,
+                           (double)sr[k].y - lr[k].y, (double)si[k].y - li[k].y};
+            // overflow of an FP32 sum (or infinite fields): the sums in FP64
+            if (!(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3]))) {
+                v[0] = v[1] = v[2] = v[3] = 0.0;
+                for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
+                    const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
+                    float2 re, im;
+                    products(__ldg(tp), __ldg(tp + 1), __ldg(&u1[n]), 2 * k, re, im);
+                    v[0] += re.x;
+                    v[1] += im.x;
+                    v[2] += re.y;
+                    v[3] += im.y;
+                }
             }
-            if (lane == 0) {
-                red[0][j][warp] += a;
-                red[1][j][warp] += b;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) vs[4 * k + c] = v[c];
+        }
+        // the warp's 2 P sums by recursive halving: at offset o a lane keeps
+        // the half of its values that its bit o selects (16 FP64 additions
+        // instead of 80 for a shuffle tree per value)
+        static_assert(2 * P == 16, "16 values, then one exchange between half warps");
+#pragma unroll
+        for (int lvl = 0; lvl < 4; ++lvl) {
+            const int o = 1 << lvl, half = P >> lvl;
+            const bool upper = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < half; ++i) {
+                const double send = upper ? vs[i] : vs[i + half];
+                const double keep = upper ? vs[i + half] : vs[i];
+                vs[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
             }
+        }
+        vs[0] += __shfl_xor_sync(0xffffffffu, vs[0], 16);
+        if (lane < 16) {  // lane bits 0..3 chose value bits 3..0
+            const int i = ((lane & 1) << 3) | ((lane & 2) << 1) | ((lane & 4) >> 1) | (lane >> 3);
+            red[i % 2][i / 2][warp] += vs[0];
         }
     }
     __syncthreads();
-    if (threadIdx.x < kDirectPoints && p0 + (int)threadIdx.x < npts) {
+    if (threadIdx.x < P && p0 + (int)threadIdx.x < npts) {
         const int j = threadIdx.x;
         double a = 0.0, b = 0.0;
         for (int w = 0; w < kDirectThreads / 32; ++w) {
             a += red[0][j][w];
             b += red[1][j][w];
         }
-        if (nan) a = b = __longlong_as_double(0x7ff8000000000000ll);
         part[(size_t)blockIdx.y * npts + p0 + j] = make_double2(a, b);
     }
 }
@@ -283,7 +352,8 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
 // The chunks' sums in order, times the outer factor: a warp per point.
 __global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int* __restrict__ mx,
                                      const int* __restrict__ my, int chunks,
-                                     const double2* __restrict__ part, float2* __restrict__ out)
+                                     const double2* __restrict__ part,
+                                     const unsigned* __restrict__ bad, float2* __restrict__ out)
 {
     const int i = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 32);
     const int lane = threadIdx.x % 32;
@@ -299,6 +369,7 @@ __global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int
         b += __shfl_xor_sync(0xffffffffu, b, o);
     }
     if (lane != 0) return;
+    if (*bad) a = b = __longlong_as_double(0x7ff8000000000000ll);
     // outer factor o = f * exp(i pi ph) / i = f (sin(pi ph) - i cos(pi ph))
     const double wgt = g.p1x * g.p1y;
     double f, ph;
@@ -354,34 +425,37 @@ asfd_status direct_sum(const asfd_params* p, const double* d1, const float2* u1,
     int dev = 0, sms = 0;
     ASFD_CUDA(cudaGetDevice(&dev));
     ASFD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int eq = form == 5 && p->p2x != p->p2y ? (int)kEq5Uneven : form;
     const size_t groups = ((size_t)npts + kDirectPoints - 1) / kDirectPoints;
     const size_t most = (n + kDirectThreads - 1) / kDirectThreads;  // rows of a single chunk
-    size_t chunks = ((size_t)kDirectWaves * sms + groups - 1) / groups;
+    size_t chunks = ((size_t)kDirectBlocks * sms + groups - 1) / groups;
     chunks = std::min(chunks, (most + 3) / 4);
     const size_t rows = (most + chunks - 1) / chunks;
     chunks = (most + rows - 1) / rows;
     DirectTerms* s = nullptr;
-    const size_t bytes = sizeof(DirectTerms) * n + sizeof(double2) * chunks * npts + most;
+    const size_t bytes = sizeof(DirectTerms) * n + sizeof(double2) * chunks * npts + sizeof(unsigned);
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&s), bytes, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(ASFD_ERR_NOMEM, std::string("per-sample terms: ") + cudaGetErrorString(e));
     }
     double2* part = reinterpret_cast<double2*>(s + n);
-    unsigned char* bad = reinterpret_cast<unsigned char*>(part + chunks * npts);
-    const int eq = form == 5 && p->p2x != p->p2y ? (int)kEq5Uneven : form;
-    direct_prep_kernel<<<(unsigned)most, kDirectThreads, 0, st>>>(g, d1, eq, s, bad);
+    unsigned* bad = reinterpret_cast<unsigned*>(part + chunks * npts);
+    e = cudaMemsetAsync(bad, 0, sizeof(unsigned), st);
+    direct_prep_kernel<<<dim3((unsigned)((p->n1x + 255) / 256),
+                              (unsigned)((p->n1y + kPrepRows - 1) / kPrepRows)),
+                         256, 0, st>>>(g, d1, eq, s, bad);
     const dim3 grid((unsigned)groups, (unsigned)chunks);
     const size_t chunk = rows * kDirectThreads;
     switch (eq) {
-#define ASFD_DS(F) case F: direct_sum_kernel<F><<<grid, kDirectThreads, 0, st>>>(g, s, u1, bad, npts, mx, my, chunk, part); break;
+#define ASFD_DS(F) case F: direct_sum_kernel<F><<<grid, kDirectThreads, 0, st>>>(g, s, u1, npts, mx, my, chunk, part); break;
         ASFD_DS(kEq2) ASFD_DS(kEq5) ASFD_DS(kEq5Uneven) ASFD_DS(kEq7)
 #undef ASFD_DS
         default: break;
     }
     direct_finish_kernel<<<(unsigned)(((size_t)npts + 7) / 8), 256, 0, st>>>(
-        g, eq, npts, mx, my, (int)chunks, part, out);
-    e = cudaGetLastError();
+        g, eq, npts, mx, my, (int)chunks, part, bad, out);
+    if (e == cudaSuccess) e = cudaGetLastError();
     const cudaError_t ef = cudaFreeAsync(s, st);
     if (e != cudaSuccess) return cuda_fail(e, "direct_sum_kernel launch");
     if (ef != cudaSuccess) return cuda_fail(ef, "cudaFreeAsync");
