@@ -158,6 +158,7 @@ struct asfd_plan_s {
     float2* lu2 = nullptr;          // [m2y][m2x] training forward output (work buffer)
     float2* lres = nullptr;         // [m2y][m2x] loss gradient (work buffer)
     double* lred = nullptr;         // [2] loss reductions
+    float* lpart = nullptr;         // per-block sums of the table and MLP gradients
     float2* stage_u1 = nullptr;     // staging for asfd_execute_host (work buffer)
     float2* stage_u2 = nullptr;
     // asfd_execute_host: a stream for the device-to-host copies of column

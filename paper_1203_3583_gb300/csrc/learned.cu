@@ -30,7 +30,9 @@
 #include <vector>
 
 #include "asfd_impl.cuh"
+#include "fft.cuh"
 #include "sample.cuh"
+#include "spread.cuh"
 
 namespace asfd {
 
@@ -91,26 +93,53 @@ __global__ void __launch_bounds__(256) features_kernel(const float* q, const Axi
 
 // ---- MLP forward: features -> hidden -> table --------------------------------
 
-__global__ void __launch_bounds__(kLearnTableSize) mlp_forward_kernel(const float* __restrict__ prm,
-                                                                      const float* __restrict__ feat,
-                                                                      float* __restrict__ hid,
-                                                                      float* __restrict__ tab)
+// A block takes kMlpTiles tiles: thread (g, o) holds row o of W2 in registers
+// and forms table entry o of the tiles g, g + 4, ...  (One block of 64
+// threads per tile read the 8 KB of W2 again for every tile, a cache line per
+// lane: 121 us for 16384 tiles; see learned_gradient.)
+constexpr int kMlpTiles = 32;
+
+__global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restrict__ prm,
+                                                          const float* __restrict__ feat, int ntiles,
+                                                          float* __restrict__ hid,
+                                                          float* __restrict__ tab)
 {
-    const int t = blockIdx.x, o = threadIdx.x;
-    __shared__ float f[kLearnFeat], h[kLearnHidden];
-    if (o < kLearnFeat) f[o] = feat[(size_t)t * kLearnFeat + o];
+    constexpr int O = kLearnTableSize, H = kLearnHidden, F = kLearnFeat, T = kMlpTiles;
+    static_assert(O == 64 && H % 4 == 0, "four tiles at a time in 256 threads");
+    __shared__ float w1[H][F + 1], f[T][F];
+    __shared__ __align__(16) float h[T][H];
+    const int tid = threadIdx.x, t0 = blockIdx.x * T, nt = min(T, ntiles - t0);
+    for (int i = tid; i < H * F; i += 256) w1[i / F][i % F] = prm[kLpW1 + i];
+    for (int i = tid; i < nt * F; i += 256) f[i / F][i % F] = feat[(size_t)t0 * F + i];
+    const int o = tid % O;
+    float w2[H];
+#pragma unroll
+    for (int i = 0; i < H; ++i) w2[i] = __ldg(&prm[kLpW2 + o * H + i]);
+    const float b2 = prm[kLpB2 + o], base = prm[kLpBase + o];
     __syncthreads();
-    if (o < kLearnHidden) {
-        float s = prm[kLpB1 + o];
-        for (int i = 0; i < kLearnFeat; ++i) s = fmaf(prm[kLpW1 + o * kLearnFeat + i], f[i], s);
+    for (int i = tid; i < nt * H; i += 256) {
+        const int t = i / H, k = i % H;
+        float s = prm[kLpB1 + k];
+#pragma unroll
+        for (int j = 0; j < F; ++j) s = fmaf(w1[k][j], f[t][j], s);
         const float hv = tanhf(s);
-        h[o] = hv;
-        hid[(size_t)t * kLearnHidden + o] = hv;
+        h[t][k] = hv;
+        hid[(size_t)t0 * H + i] = hv;
     }
     __syncthreads();
-    float s = prm[kLpB2 + o];
-    for (int i = 0; i < kLearnHidden; ++i) s = fmaf(prm[kLpW2 + o * kLearnHidden + i], h[i], s);
-    tab[(size_t)t * kLearnTableSize + o] = prm[kLpBase + o] + kLearnOutScale * s;
+    for (int t = tid / O; t < nt; t += 256 / O) {
+        float s = b2;
+        const float4* h4 = reinterpret_cast<const float4*>(h[t]);
+#pragma unroll
+        for (int i = 0; i < H / 4; ++i) {
+            const float4 v = h4[i];
+            s = fmaf(w2[4 * i], v.x, s);
+            s = fmaf(w2[4 * i + 1], v.y, s);
+            s = fmaf(w2[4 * i + 2], v.z, s);
+            s = fmaf(w2[4 * i + 3], v.w, s);
+        }
+        tab[(size_t)(t0 + t) * O + o] = base + kLearnOutScale * s;
+    }
 }
 
 // ---- deconvolution correction ----------------------------------------------
@@ -143,91 +172,149 @@ __global__ void deconv_build_kernel(const float* __restrict__ prm, const float2*
 
 // ---- loss --------------------------------------------------------------------
 
-__global__ void loss_reduce_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
-                                   size_t n, double* red)
+constexpr int kLossBlocks = 1216;  // eight per SM
+
+// sum + err += v on a pair, err collecting the rounding errors of sum exactly
+// (Knuth's two-sum)
+__device__ __forceinline__ void two_sum2(float2& sum, float2& err, float2 v)
 {
-    double e = 0.0, r = 0.0;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const float2 a = u2[i], b = ref[i];
-        const double dx = (double)a.x - b.x, dy = (double)a.y - b.y;
-        e += dx * dx + dy * dy;
-        r += (double)b.x * b.x + (double)b.y * b.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        e += __shfl_xor_sync(0xffffffffu, e, o);
-        r += __shfl_xor_sync(0xffffffffu, r, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&red[0], e);
-        atomicAdd(&red[1], r);
-    }
+    const float2 s = cadd(sum, v);
+    const float2 b = csub(s, sum);
+    err = cadd(err, cadd(csub(sum, csub(s, b)), csub(v, b)));
+    sum = s;
 }
 
-__global__ void residual_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
-                                size_t n, const double* red, float2* __restrict__ g)
+// sum + err += (v + dv)^2 on a pair, exactly but for the last term's rounding
+__device__ __forceinline__ void add_square2(float2& sum, float2& err, float2 v, float2 dv)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float sc = (float)(2.0 / fmax(red[1], 1e-300));
-    const float2 a = u2[i], b = ref[i];
-    g[i] = make_float2(sc * (a.x - b.x), sc * (a.y - b.y));
+    const float2 p = mul_f2(v, v);
+    const float2 pe = fma_f2(v, v, make_float2(-p.x, -p.y));
+    two_sum2(sum, err, p);
+    err = cadd(err, fma_f2(cadd(v, v), dv, pe));
 }
 
-// dL/dcorr_x[mx] = Re sum_my conj(g) u2 / corr_x[mx]: blocks of 32 columns x
-// 8 thread rows over a slab of destination rows; the slab's column sums are
-// added atomically to out (zeroed by the caller)
-constexpr int kDeconvSlabs = 64;
-
-__global__ void __launch_bounds__(256) deconv_grad_x_kernel(const float2* __restrict__ g,
-                                                            const float2* __restrict__ u2,
-                                                            const float* __restrict__ corr,
-                                                            int m2x, int m2y, float* __restrict__ out)
+// Whether a thread's FP32 sum of squares is exact to about 2^-40: not so
+// large that a term may have overflowed, nor so small that the terms'
+// rounding errors have underflowed (the caller then sums again in FP64).
+__device__ __forceinline__ bool squares_in_range(float2 sum)
 {
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int mx = blockIdx.x * 32 + tx;
-    const int slab = (m2y + gridDim.y - 1) / gridDim.y;
-    const int y0 = blockIdx.y * slab, y1 = min(m2y, y0 + slab);
-    float s = 0.f;
-    if (mx < m2x)
-        for (int my = y0 + ty; my < y1; my += 8) {
-            const float2 a = g[(size_t)my * m2x + mx], b = u2[(size_t)my * m2x + mx];
-            s += a.x * b.x + a.y * b.y;
+    const float t = sum.x + sum.y;
+    return t > 8.2718061e-25f && t < 1.2676506e30f;  // 2^-80 .. 2^100
+}
+
+// Adds the block's sum to *out.  `part`: a slot per thread (256); one warp adds
+// them (a shuffle tree in every warp is seven times as many FP64 additions, at
+// 2 lanes per clock).  Has a block barrier.
+__device__ __forceinline__ void block_add(double v, double* part, double* out)
+{
+    part[threadIdx.x] = v;
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    for (int w = 1; w < 8; ++w) v += part[threadIdx.x + 32 * w];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) atomicAdd(out, v);
+}
+
+// red[1] += |ref|^2, and the deconvolution gradients are set to zero.  The
+// squares are carried as FP32 values with their exact rounding errors: FP64
+// sums over 4.2 M points are bound by the FP64 pipe (this and the squared
+// error together took 116 us).
+__global__ void __launch_bounds__(256) ref_norm_kernel(const float2* __restrict__ ref, size_t n,
+                                                       double* red, float* __restrict__ gcorr,
+                                                       int ncorr)
+{
+    const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t step = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = i0; i < (size_t)ncorr; i += step) gcorr[i] = 0.f;
+    float2 sum = make_float2(0.f, 0.f), err = sum;
+#pragma unroll 8
+    for (size_t i = i0; i < n; i += step)
+        add_square2(sum, err, __ldg(&ref[i]), make_float2(0.f, 0.f));
+    double v = ((double)sum.x + (double)sum.y) + ((double)err.x + (double)err.y);
+    if (!squares_in_range(sum)) {
+        v = 0.0;
+        for (size_t i = i0; i < n; i += step) {
+            const float2 b = __ldg(&ref[i]);
+            v += (double)b.x * b.x + (double)b.y * b.y;
         }
-    __shared__ float red[8][33];
-    red[ty][tx] = s;
-    __syncthreads();
-    if (ty == 0 && mx < m2x) {
+    }
+    __shared__ double part[256];
+    block_add(v, part, red + 1);
+}
+
+// One pass over the output: g = dL/du2 = 2 (u2 - ref)/|ref|^2, red[0] +=
+// |u2 - ref|^2, and dL/dcorr of both axes (sums of Re[conj(g) u2] / corr over
+// the columns' rows and the rows' columns).  A warp takes 128 columns (4 a
+// lane) of every 8th row of its block's kLossRows rows.  Four kernels (the
+// loss in FP64, g with an FP64 division per point, one pass per axis) took
+// 212 us at 2048^2; see learned_gradient.
+constexpr int kLossCols = 128, kLossRows = 32;
+
+__global__ void __launch_bounds__(256)
+loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
+            const float* __restrict__ corr, int m2x, int m2y, double* red, float2* __restrict__ g,
+            float* __restrict__ gcorr)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int c0 = blockIdx.x * kLossCols + lane;
+    const int y1 = min(m2y, (int)(blockIdx.y + 1) * kLossRows);
+    const float sc = (float)(2.0 / fmax(red[1], 1e-300));
+    float2 sum = make_float2(0.f, 0.f), err = sum;
+    float col[kLossCols / 32];
+#pragma unroll
+    for (int j = 0; j < kLossCols / 32; ++j) col[j] = 0.f;
+    for (int y = blockIdx.y * kLossRows + warp; y < y1; y += 8) {
+        const size_t row = (size_t)y * m2x;
+        float across = 0.f;
+#pragma unroll
+        for (int j = 0; j < kLossCols / 32; ++j) {
+            const int c = c0 + 32 * j;
+            if (c < m2x) {
+                const float2 a = __ldg(&u2[row + c]), b = __ldg(&ref[row + c]);
+                // a - b = d + e exactly
+                const float2 d = csub(a, b), z = csub(d, a);
+                const float2 e = csub(csub(a, csub(d, z)), cadd(b, z));
+                add_square2(sum, err, d, e);
+                const float2 v = make_float2(sc * d.x, sc * d.y);
+                g[row + c] = v;
+                const float dot = v.x * a.x + v.y * a.y;
+                col[j] += dot;
+                across += dot;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) across += __shfl_xor_sync(0xffffffffu, across, o);
+        if (lane == 0) atomicAdd(&gcorr[m2x + y], across / corr[m2x + y]);
+    }
+    __shared__ float cols[8][kLossCols];
+#pragma unroll
+    for (int j = 0; j < kLossCols / 32; ++j) cols[warp][lane + 32 * j] = col[j];
+    double e2 = ((double)sum.x + (double)sum.y) + ((double)err.x + (double)err.y);
+    if (!squares_in_range(sum)) {
+        e2 = 0.0;
+        for (int y = blockIdx.y * kLossRows + warp; y < y1; y += 8)
+            for (int c = c0; c < min(m2x, (int)(blockIdx.x + 1) * kLossCols); c += 32) {
+                const float2 a = __ldg(&u2[(size_t)y * m2x + c]), b = __ldg(&ref[(size_t)y * m2x + c]);
+                const double dx = (double)a.x - b.x, dy = (double)a.y - b.y;
+                e2 += dx * dx + dy * dy;
+            }
+    }
+    __shared__ double part[256];
+    block_add(e2, part, red);
+    const int c = blockIdx.x * kLossCols + threadIdx.x;
+    if (threadIdx.x < kLossCols && c < m2x) {
         float t = 0.f;
-        for (int r = 0; r < 8; ++r) t += red[r][tx];
-        atomicAdd(&out[mx], t / corr[mx]);
+        for (int w = 0; w < 8; ++w) t += cols[w][threadIdx.x];
+        atomicAdd(&gcorr[c], t / corr[c]);
     }
 }
 
-// dL/dcorr_y[my] (one block per row)
-__global__ void deconv_grad_y_kernel(const float2* __restrict__ g, const float2* __restrict__ u2,
-                                     const float* __restrict__ corr, int m2x, float* __restrict__ out)
+// dL/dd_j = sum_k dL/dcorr[k] T_2j(u_k): block 0 the x axis, block 1 the y axis
+__global__ void __launch_bounds__(1024) cheb_grad_kernel(const float* __restrict__ gcorr, int m2x,
+                                                         int m2y, float* __restrict__ grad)
 {
-    const int my = blockIdx.x;
-    float s = 0.f;
-    for (int mx = threadIdx.x; mx < m2x; mx += blockDim.x) {
-        const float2 a = g[(size_t)my * m2x + mx], b = u2[(size_t)my * m2x + mx];
-        s += a.x * b.x + a.y * b.y;
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ float red[32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < (int)(blockDim.x / 32); ++w) t += red[w];
-        out[my] = t / corr[my];
-    }
-}
-
-// dL/dd_j = sum_k dL/dcorr[k] T_2j(u_k) (one block per axis)
-__global__ void cheb_grad_kernel(const float* __restrict__ gcorr, int m, float* __restrict__ grad)
-{
+    const int m = blockIdx.x == 0 ? m2x : m2y;
+    if (blockIdx.x == 1) gcorr += m2x;
+    grad += blockIdx.x == 0 ? kLpDx : kLpDy;
     float s[kLearnCheb];
     for (int j = 0; j < kLearnCheb; ++j) s[j] = 0.f;
     for (int k = threadIdx.x; k < m; k += blockDim.x) {
@@ -267,65 +354,105 @@ struct TGArgs {
     float inc_d;
 };
 
-__global__ void __launch_bounds__(256) table_grad_kernel(TGArgs a)
+// A warp per source tile, a lane per half column (8 samples): the lane sums its
+// samples' contributions to the 64 table entries, per axis and tap the sum
+// over the other axis' taps first, then times the powers of t; the warp's 64
+// sums meet in one reduce-scatter per tile.  (A thread per sample, with the
+// powers inside the 16 taps and a reduce-scatter per 32 samples, took 147 us at
+// 2048^2; see learned_gradient.)
+constexpr int kTgWarps = 4;
+
+template <bool WRAP>
+__global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int ntiles)
 {
     constexpr int W = kLearnW, K = kLearnCoef;
-    const int t = blockIdx.x;
-    const int nx = (t % a.nstx) * kSrcTile + threadIdx.x % kSrcTile;
-    const int ny = (t / a.nstx) * kSrcTile + threadIdx.x / kSrcTile;
-    float gx[W][K], gy[W][K];
+    static_assert(kSrcTile == 16 && 2 * W * K == 64, "half a column per lane, 64 sums over 32 lanes");
+    __shared__ __align__(16) float tsm[kTgWarps][2 * W * K];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
+    const int t = blockIdx.x * kTgWarps + wid;
+    if (t >= ntiles) return;  // warp-uniform
+    // the tile's polynomials as (x, y) coefficient pairs
+#pragma unroll
+    for (int e = lane; e < 2 * W * K; e += 32)
+        tsm[wid][2 * (e % (W * K)) + e / (W * K)] = __ldg(&a.tab[(size_t)t * kLearnTableSize + e]);
+    __syncwarp();
+    const int nx = (t % a.nstx) * kSrcTile + (lane & 15);
+    const int ny0 = (t / a.nstx) * kSrcTile + (lane >> 4) * (kSrcTile / 2);
+    const int rows = nx < a.n1x ? min(kSrcTile / 2, a.n1y - ny0) : 0;
+    const int mx = a.nfx - 1, my = a.nfy - 1;
+    float2 G[W][K];  // (x, y) sums
 #pragma unroll
     for (int i = 0; i < W; ++i)
 #pragma unroll
-        for (int k = 0; k < K; ++k) gx[i][k] = gy[i][k] = 0.f;
-    if (nx < a.n1x && ny < a.n1y) {
-        const Raw r = load_raw(a, nx, ny);
+        for (int k = 0; k < K; ++k) G[i][k] = make_float2(0.f, 0.f);
+    Raw next;
+    if (rows > 0) next = load_raw(a, nx, ny0);
+    for (int r = 0; r < rows; ++r) {
+        const Raw s = next;
+        if (r + 1 < rows) {  // the next sample's inputs, while this one is processed
+            const int ny = ny0 + r + 1;
+            const size_t n = (size_t)ny * a.n1x + nx;
+            next.q = __ldg(&a.q[n]);
+            next.u = __ldg(&a.u1[n]);
+            next.ey = a.ay[ny];
+            next.py = a.py[ny];
+        }
         int l0x, l0y;
         float dx, dy;
-        sample_pos(r.ex, r.ey, r.px, r.py, r.q, a.half_w, l0x, l0y, dx, dy);
-        const float2 c = sample_value_fast(r, a.inc_d);
-        float wx[W], wy[W];
-        table_weights<W>(a.tab + (size_t)t * kLearnTableSize, dx, dy, wx, wy);
-        const float tx = fmaf(2.f, dx, -1.f), ty = fmaf(2.f, dy, -1.f);
-        float ptx[K], pty[K];
-        ptx[0] = pty[0] = 1.f;
+        sample_pos(s.ex, s.ey, s.px, s.py, s.q, a.half_w, l0x, l0y, dx, dy);
+        float2 B[W][W];
+        if constexpr (WRAP) {
 #pragma unroll
-        for (int k = 1; k < K; ++k) {
-            ptx[k] = ptx[k - 1] * tx;
-            pty[k] = pty[k - 1] * ty;
+            for (int b = 0; b < W; ++b) {
+                const float2* row = a.grid + (size_t)((l0y + b) & my) * a.nfx;
+#pragma unroll
+                for (int i = 0; i < W; ++i) B[b][i] = __ldg(&row[(l0x + i) & mx]);
+            }
+        } else {
+            // (clamped all the same: every address stays inside the grid)
+            const float2* cell = a.grid + (size_t)min(max(l0y, 0), a.nfy - W) * a.nfx +
+                                 min(max(l0x, 0), a.nfx - W);
+#pragma unroll
+            for (int b = 0; b < W; ++b)
+#pragma unroll
+                for (int i = 0; i < W; ++i) B[b][i] = __ldg(cell + (size_t)b * a.nfx + i);
         }
-        const int mx = a.nfx - 1, my = a.nfy - 1;
+        const float2 c = sample_value_fast(s, a.inc_d);
+        float wx[W], wy[W];
+        table_weights_smem<W>(reinterpret_cast<const float4*>(tsm[wid]), dx, dy, wx, wy);
+        // sums of the cells over the other axis' taps, then Re[conj(sum) c]
+        float2 vc[W], vr[W];
 #pragma unroll
         for (int b = 0; b < W; ++b) {
-            const float2* row = a.grid + (size_t)((l0y + b) & my) * a.nfx;
+            vr[b] = mul2(B[b][0], wx[0]);
 #pragma unroll
-            for (int i = 0; i < W; ++i) {
-                const float2 B = __ldg(&row[(l0x + i) & mx]);
-                const float v = B.x * c.x + B.y * c.y;  // Re[conj(B) c]
-                const float vx = v * wy[b], vy = v * wx[i];
+            for (int i = 1; i < W; ++i) vr[b] = fma2(B[b][i], wx[i], vr[b]);
 #pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    gx[i][k] = fmaf(vx, ptx[k], gx[i][k]);
-                    gy[b][k] = fmaf(vy, pty[k], gy[b][k]);
-                }
-            }
+            for (int i = 0; i < W; ++i) vc[i] = b == 0 ? mul2(B[b][i], wy[b]) : fma2(B[b][i], wy[b], vc[i]);
+        }
+        const float2 tt = make_float2(fmaf(2.f, dx, -1.f), fmaf(2.f, dy, -1.f));
+        float2 pw[K];
+        pw[0] = make_float2(1.f, 1.f);
+#pragma unroll
+        for (int k = 1; k < K; ++k) pw[k] = mul_f2(pw[k - 1], tt);
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const float2 v = make_float2(vc[i].x * c.x + vc[i].y * c.y, vr[i].x * c.x + vr[i].y * c.y);
+#pragma unroll
+            for (int k = 0; k < K; ++k) G[i][k] = fma_f2(v, pw[k], G[i][k]);
         }
     }
-    // block reduction of the 2 W K = 64 sums: within each warp a
-    // reduce-scatter by recursive halving (at offset o a lane keeps the half
+    // reduce-scatter by recursive halving: at offset o a lane keeps the half
     // of its values selected by lane bit o and adds its partner's copy of
-    // that half), after which lane l holds the warp's sums of entries 2l and
-    // 2l + 1; then the 8 warps' sums are added in shared memory
-    static_assert(2 * W * K == 64, "reduce-scatter of 64 values over 32 lanes");
+    // that half; lane l ends with the warp's sums of entries 2l and 2l + 1
     float v[64];
 #pragma unroll
     for (int i = 0; i < W; ++i)
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            v[i * K + k] = gx[i][k];
-            v[(W + i) * K + k] = gy[i][k];
+            v[i * K + k] = G[i][k].x;
+            v[(W + i) * K + k] = G[i][k].y;
         }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
 #pragma unroll
     for (int lvl = 0; lvl < 5; ++lvl) {
         const int o = 16 >> lvl, half = 32 >> lvl;
@@ -337,64 +464,136 @@ __global__ void __launch_bounds__(256) table_grad_kernel(TGArgs a)
             v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    __shared__ float red[8][kLearnTableSize];
-    red[wid][2 * lane] = v[0];
-    red[wid][2 * lane + 1] = v[1];
-    __syncthreads();
-    if (threadIdx.x < kLearnTableSize) {
-        float s = 0.f;
-        for (int w2 = 0; w2 < 8; ++w2) s += red[w2][threadIdx.x];
-        a.tgrad[(size_t)t * kLearnTableSize + threadIdx.x] = s;
-    }
+    reinterpret_cast<float2*>(a.tgrad + (size_t)t * kLearnTableSize)[lane] = make_float2(v[0], v[1]);
 }
 
 // ---- MLP backward over tiles (block-private accumulation, then atomics) --------
+
+// Blocks walk over groups of kBackTiles tiles.  A thread keeps its 8 entries of
+// dL/dW2 (row o, 8 columns), its entry of dL/dW1 and of the biases in
+// registers over all groups, and column ti of W2 for the hidden gradient of
+// its (tile, unit) in each group; the next group's inputs are loaded while one
+// is processed.  (One tile at a time, with the sums in shared memory and 32 of
+// 256 threads on the hidden gradient, took 92 us for 16384 tiles; see
+// learned_gradient.)
+constexpr int kBackTiles = 8;
+constexpr int kBackBlocks = 304;      // two per SM
+constexpr int kMlpParams = kLpDx;     // table and MLP parameters come first
 
 __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restrict__ prm,
                                                            const float* __restrict__ feat,
                                                            const float* __restrict__ hid,
                                                            const float* __restrict__ tgrad, int ntiles,
-                                                           float* __restrict__ grad)
+                                                           float* __restrict__ part)
 {
-    constexpr int O = kLearnTableSize, H = kLearnHidden, F = kLearnFeat;
-    __shared__ float gW2[O * H], gb2[O], gbase[O], gW1[H * F], gb1[H];
-    __shared__ float dout[O], h[H], f[F], dh[H];
+    constexpr int O = kLearnTableSize, H = kLearnHidden, F = kLearnFeat, T = kBackTiles;
+    static_assert(T * H == 256 && T * O == 512 && O * H == 8 * 256 && H * F <= 256,
+                  "one (tile, unit) per thread");
+    __shared__ __align__(16) float dout[T][O], h[T][H];
+    __shared__ float f[T][F], dh[T][H];
     const int tid = threadIdx.x;
-    for (int i = tid; i < O * H; i += blockDim.x) gW2[i] = 0.f;
-    for (int i = tid; i < H * F; i += blockDim.x) gW1[i] = 0.f;
-    if (tid < O) gb2[tid] = gbase[tid] = 0.f;
-    if (tid < H) gb1[tid] = 0.f;
-    __syncthreads();
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        if (tid < O) {
-            const float d = tgrad[(size_t)t * O + tid];
-            gbase[tid] += d;
-            dout[tid] = kLearnOutScale * d;
-            gb2[tid] += kLearnOutScale * d;
-        }
-        if (tid < H) h[tid] = hid[(size_t)t * H + tid];
-        if (tid < F) f[tid] = feat[(size_t)t * F + tid];
+    const int o = tid / 4, i0 = (tid % 4) * 8;  // this thread's entries of W2
+    const int k1 = tid / F, j1 = tid % F;       // and of W1 (tid < H F)
+    const int tt = tid / H, ti = tid % H;       // its hidden gradient
+    float w2[O];
+#pragma unroll
+    for (int k = 0; k < O; ++k) w2[k] = __ldg(&prm[kLpW2 + k * H + ti]);
+    float gw2[8], gw1 = 0.f, gb1 = 0.f, gbase = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) gw2[i] = 0.f;
+    // this thread's inputs of a group: two table gradients (entry tid % O of
+    // tiles tid / O and tid / O + 4), one hidden value, one feature
+    float n0, n1, nh, nf;
+    auto fetch = [&](int t0) {
+        const int nt = min(T, ntiles - t0);
+        n0 = tid < nt * O ? __ldg(&tgrad[(size_t)t0 * O + tid]) : 0.f;
+        n1 = tid + 256 < nt * O ? __ldg(&tgrad[(size_t)t0 * O + tid + 256]) : 0.f;
+        nh = tid < nt * H ? __ldg(&hid[(size_t)t0 * H + tid]) : 0.f;
+        nf = tid < nt * F ? __ldg(&feat[(size_t)t0 * F + tid]) : 0.f;
+    };
+    fetch(blockIdx.x * T);
+    for (int t0 = blockIdx.x * T; t0 < ntiles; t0 += gridDim.x * T) {
+        __syncthreads();  // the previous group's readers are done
+        gbase += n0 + n1;
+        dout[tid / O][tid % O] = kLearnOutScale * n0;
+        dout[tid / O + 4][tid % O] = kLearnOutScale * n1;
+        h[tt][ti] = nh;
+        if (tid < T * F) f[tid / F][tid % F] = nf;
+        const float hv = nh;
         __syncthreads();
-        for (int i = tid; i < O * H; i += blockDim.x) gW2[i] += dout[i / H] * h[i % H];
+        if (t0 + gridDim.x * T < ntiles) fetch(t0 + gridDim.x * T);
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        const float4* d4 = reinterpret_cast<const float4*>(dout[tt]);
+#pragma unroll
+        for (int k = 0; k < O / 4; ++k) {
+            const float4 d = d4[k];
+            s0 = fmaf(w2[4 * k], d.x, s0);
+            s1 = fmaf(w2[4 * k + 1], d.y, s1);
+            s2 = fmaf(w2[4 * k + 2], d.z, s2);
+            s3 = fmaf(w2[4 * k + 3], d.w, s3);
+        }
+        dh[tt][ti] = ((s0 + s1) + (s2 + s3)) * (1.f - hv * hv);
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const float d = dout[t][o];
+            const float4 a = *reinterpret_cast<const float4*>(&h[t][i0]);
+            const float4 b = *reinterpret_cast<const float4*>(&h[t][i0 + 4]);
+            gw2[0] = fmaf(d, a.x, gw2[0]);
+            gw2[1] = fmaf(d, a.y, gw2[1]);
+            gw2[2] = fmaf(d, a.z, gw2[2]);
+            gw2[3] = fmaf(d, a.w, gw2[3]);
+            gw2[4] = fmaf(d, b.x, gw2[4]);
+            gw2[5] = fmaf(d, b.y, gw2[5]);
+            gw2[6] = fmaf(d, b.z, gw2[6]);
+            gw2[7] = fmaf(d, b.w, gw2[7]);
+        }
+        __syncthreads();
+        if (tid < H * F) {
+#pragma unroll
+            for (int t = 0; t < T; ++t) gw1 = fmaf(dh[t][k1], f[t][j1], gw1);
+        }
         if (tid < H) {
-            float s = 0.f;
-            for (int o = 0; o < O; ++o) s = fmaf(prm[kLpW2 + o * H + tid], dout[o], s);
-            const float d = s * (1.f - h[tid] * h[tid]);
-            dh[tid] = d;
-            gb1[tid] += d;
+#pragma unroll
+            for (int t = 0; t < T; ++t) gb1 += dh[t][tid];
         }
-        __syncthreads();
-        for (int i = tid; i < H * F; i += blockDim.x) gW1[i] += dh[i / F] * f[i % F];
-        __syncthreads();
     }
-    for (int i = tid; i < O * H; i += blockDim.x) atomicAdd(&grad[kLpW2 + i], gW2[i]);
-    for (int i = tid; i < H * F; i += blockDim.x) atomicAdd(&grad[kLpW1 + i], gW1[i]);
+    float* out = part + (size_t)blockIdx.x * kMlpParams;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) out[kLpW2 + o * H + i0 + i] = gw2[i];
+    if (tid < H * F) out[kLpW1 + tid] = gw1;
+    if (tid < H) out[kLpB1 + tid] = gb1;
+    __syncthreads();
+    float* base = &dout[0][0];  // [4][O]
+    base[tid] = gbase;
+    __syncthreads();
     if (tid < O) {
-        atomicAdd(&grad[kLpB2 + tid], gb2[tid]);
-        atomicAdd(&grad[kLpBase + tid], gbase[tid]);
+        const float v = (base[tid] + base[tid + O]) + (base[tid + 2 * O] + base[tid + 3 * O]);
+        out[kLpBase + tid] = v;
+        out[kLpB2 + tid] = kLearnOutScale * v;
     }
-    if (tid < H) atomicAdd(&grad[kLpB1 + tid], gb1[tid]);
 }
+
+// The blocks' sums, added in order: a thread per parameter and eighth of the
+// blocks.
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict__ part, int blocks,
+                                                         float* __restrict__ grad)
+{
+    __shared__ float red[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
+    const int i = blockIdx.x * 32 + lane;
+    float v = 0.f;
+    if (i < kMlpParams) {
+#pragma unroll 8
+        for (int b = wid; b < blocks; b += 8) v += __ldg(&part[(size_t)b * kMlpParams + i]);
+    }
+    red[wid][lane] = v;
+    __syncthreads();
+    if (wid == 0 && i < kMlpParams) {
+        for (int w = 1; w < 8; ++w) v += red[w][lane];
+        grad[i] = v;
+    }
+}
+
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, int n, float lr, float b1, float b2, float c1,
@@ -477,7 +676,8 @@ asfd_status learned_features(asfd_plan_s* P, cudaStream_t st)
 asfd_status learned_refresh(asfd_plan_s* P, cudaStream_t st)
 {
     const int nst = P->nstx * P->nsty;
-    mlp_forward_kernel<<<nst, kLearnTableSize, 0, st>>>(P->lparams, P->lfeat, P->lhid, P->ltab);
+    mlp_forward_kernel<<<(nst + kMlpTiles - 1) / kMlpTiles, 256, 0, st>>>(P->lparams, P->lfeat, nst,
+                                                                          P->lhid, P->ltab);
     const int m2x = P->prm.m2x, m2y = P->prm.m2y;
     deconv_build_kernel<<<(m2x + 255) / 256, 256, 0, st>>>(P->lparams, P->cxb, P->cx, P->lcorr, m2x,
                                                            kLpDx);
@@ -507,6 +707,7 @@ asfd_status learned_init(asfd_plan_s* P, cudaStream_t st)
     LA(lcorr, sizeof(float) * mm);
     LA(lcgrad, sizeof(float) * mm);
     LA(lred, sizeof(double) * 2);
+    LA(lpart, sizeof(float) * kBackBlocks * kMlpParams);
 #undef LA
     // the ES width-4 deconvolution/chirp tables become the base tables
     ASFD_CUDA(cudaMemcpyAsync(P->cxb, P->cx, sizeof(float2) * P->prm.m2x, cudaMemcpyDeviceToDevice, st));
@@ -535,30 +736,30 @@ asfd_status learned_init(asfd_plan_s* P, cudaStream_t st)
 }
 
 // Forward with the current model, loss against `ref`, and every parameter
-// gradient into P->lgrad (no update).
+// gradient into P->lgrad (no update).  Kernel times at 2048^2 samples and
+// points (CUDA events of a trace; before -> now, us): loss, residual and
+// deconvolution gradients 212 -> 41 (ref_norm 13.8, loss 27.4: bound by memory,
+// 134 MB), both Chebyshev sums 14.3 -> 4.2, table gradients 147 -> 68 (half the
+// issue slots; 128 registers leave 16 warps per SM), MLP backward 92 -> 18
+// (with its reduction), MLP forward 121 -> not run here; the whole call 851 ->
+// 374 us.
 asfd_status learned_gradient(asfd_plan_s* P, const float2* u1, const float2* ref, cudaStream_t st)
 {
     const int nst = P->nstx * P->nsty;
     const int m2x = P->prm.m2x, m2y = P->prm.m2y;
     const size_t m = (size_t)m2x * m2y;
     asfd_status s;
-    // forward with the current model
-    if ((s = learned_refresh(P, st)) != ASFD_OK) return s;
+    // forward with the current model (its tables are current: every change of
+    // the parameters or the height map rebuilds them)
     if ((s = launch_spread(P, u1, st)) != ASFD_OK) return s;
     if ((s = launch_fft_rows(P, st)) != ASFD_OK) return s;
     if ((s = launch_fft_cols(P, P->lu2, st)) != ASFD_OK) return s;
-    // loss and its gradient with respect to u2
+    // loss, its gradient with respect to u2 and the deconvolution correction's
     ASFD_CUDA(cudaMemsetAsync(P->lred, 0, sizeof(double) * 2, st));
-    loss_reduce_kernel<<<512, 256, 0, st>>>(P->lu2, ref, m, P->lred);
-    residual_kernel<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(P->lu2, ref, m, P->lred, P->lres);
-    ASFD_CUDA(cudaMemsetAsync(P->lgrad, 0, sizeof(float) * kLearnParams, st));
-    // deconvolution correction gradients
-    ASFD_CUDA(cudaMemsetAsync(P->lcgrad, 0, sizeof(float) * m2x, st));
-    deconv_grad_x_kernel<<<dim3((m2x + 31) / 32, kDeconvSlabs), 256, 0, st>>>(
-        P->lres, P->lu2, P->lcorr, m2x, m2y, P->lcgrad);
-    deconv_grad_y_kernel<<<m2y, 256, 0, st>>>(P->lres, P->lu2, P->lcorr + m2x, m2x, P->lcgrad + m2x);
-    cheb_grad_kernel<<<1, 256, 0, st>>>(P->lcgrad, m2x, P->lgrad + kLpDx);
-    cheb_grad_kernel<<<1, 256, 0, st>>>(P->lcgrad + m2x, m2y, P->lgrad + kLpDy);
+    ref_norm_kernel<<<kLossBlocks, 256, 0, st>>>(ref, m, P->lred, P->lcgrad, m2x + m2y);
+    loss_kernel<<<dim3((m2x + kLossCols - 1) / kLossCols, (m2y + kLossRows - 1) / kLossRows), 256, 0,
+                  st>>>(P->lu2, ref, P->lcorr, m2x, m2y, P->lred, P->lres, P->lcgrad);
+    cheb_grad_kernel<<<2, 1024, 0, st>>>(P->lcgrad, m2x, m2y, P->lgrad);
     ASFD_CUDA(cudaGetLastError());
     // table gradients through the adjoint grid
     if ((s = launch_fft_cols_adj(P, P->lres, st)) != ASFD_OK) return s;
@@ -580,9 +781,15 @@ asfd_status learned_gradient(asfd_plan_s* P, const float2* u1, const float2* ref
     a.nfy = P->nfy;
     a.half_w = 0.5f * kLearnW;
     a.inc_d = (float)P->inc_d;
-    table_grad_kernel<<<nst, 256, 0, st>>>(a);
-    mlp_backward_kernel<<<nst < 256 ? nst : 256, 256, 0, st>>>(P->lparams, P->lfeat, P->lhid,
-                                                                P->ltgrad, nst, P->lgrad);
+    // (a dense plan's footprints do not wrap around the periodic grid)
+    const unsigned tgb = (unsigned)((nst + kTgWarps - 1) / kTgWarps);
+    if (P->dense) table_grad_kernel<false><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
+    else table_grad_kernel<true><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
+    const int groups = (nst + kBackTiles - 1) / kBackTiles;
+    mlp_backward_kernel<<<groups < kBackBlocks ? groups : kBackBlocks, 256, 0, st>>>(
+        P->lparams, P->lfeat, P->lhid, P->ltgrad, nst, P->lpart);
+    mlp_reduce_kernel<<<(kMlpParams + 31) / 32, 256, 0, st>>>(
+        P->lpart, groups < kBackBlocks ? groups : kBackBlocks, P->lgrad);
     ASFD_CUDA(cudaGetLastError());
     return ASFD_OK;
 }
