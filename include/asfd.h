@@ -77,9 +77,10 @@ typedef struct {
     int deterministic;   /* 0 (fastest): for monotone maps and ES widths up to 7 the    */
                          /*   spread accumulates register windows into the fine grid   */
                          /*   with float atomic adds, so the last bits of a result may  */
-                         /*   differ from run to run; 1: conflict-free shared-memory    */
-                         /*   tiles without atomics where the map allows them (results */
-                         /*   bit-identical run to run), shared-memory atomics else     */
+                         /*   differ from run to run; 1: shared-memory tiles without    */
+                         /*   atomics where the map allows them (results bit-identical */
+                         /*   run to run), as widths above 7 always; float atomic adds  */
+                         /*   else (folding or wrapping maps)                           */
     double incidence_sx, incidence_sy; /* direction cosines of the incident plane wave */
                          /*   u_I = exp(ik(sx x1 + sy y1 + sz d1)), sz = sqrt(1 - sx^2  */
                          /*   - sy^2), sx^2 + sy^2 < 1; 0, 0: normal incidence, the     */
@@ -99,21 +100,22 @@ typedef struct {
     int band_y0, band_y1;    /* touched fine-grid rows    [y0, y1)                      */
     int spread_tiles;        /* output tiles the spreading kernel processes             */
     long long tile_pairs;    /* (output tile, source tile) pairs in the binning of the  */
-                             /*    shared-memory-atomic spread (spread_kind 1; else 0)  */
+                             /*    persistent batch's shared-memory-atomic spread       */
+                             /*    (spread_kind 1; else 0)                              */
     double es_beta;          /* ES beta in use                                          */
     double max_abs_eps;      /* max |d1| / z0 over the surface                          */
     size_t device_bytes;     /* device memory owned by the plan                         */
-    int spread_kind;         /* 0: conflict-free warp tiles (no atomics) -- used when   */
-                             /*    the map n -> g is monotone with positive spacing and */
-                             /*    no footprint wraps; 1: shared-memory atomics;        */
+    int spread_kind;         /* 0: shared-memory tiles without atomics at widths above  */
+                             /*    7 -- used when the map n -> g is monotone with       */
+                             /*    positive spacing and no footprint wraps; 1: register */
+                             /*    windows flushed with atomic adds to wrapped cells;   */
                              /*    2: conflict-free warp tiles with a sliding register  */
                              /*    window per lane (ES widths up to 7); 3: dense maps   */
                              /*    (many samples per cell): register windows flushed    */
                              /*    to the fine grid with atomic adds (widths up to 7);  */
-                             /*    4: deterministic plans whose samples are at least a  */
-                             /*    fine cell apart in x (widths up to 7): register      */
-                             /*    windows flushed into per-item shared-memory tiles in */
-                             /*    a fixed order, then an ordered gather (no atomics)   */
+                             /*    4: deterministic plans (widths up to 7): register    */
+                             /*    windows flushed into shared-memory tiles in a fixed  */
+                             /*    order, then an ordered gather or merge (no atomics)  */
     int stride_x, stride_y;  /* sample strides between lanes of one warp step (0, 2)    */
     int run_rows;            /* source rows per lane run of the register-window spread  */
                              /*    (spread_kind 3; 0 otherwise)                         */

@@ -116,6 +116,8 @@ struct asfd_plan_s {
     bool colored = false;
     bool windowed = false;          // register-window kernel applies (w <= kMaxWindowWidth)
     bool dense = false;             // dense map: register windows flushed with global atomics
+    bool fold = false;              // folding or wrapping map: register windows flushed with
+                                    // global atomics to wrapped cells
     int dense_rows = 0, dense_items = 0;
     // atomic-free spread through per-item shared-memory tiles and an ordered
     // gather (deterministic plans whose samples are >= 1 cell apart in x)
@@ -125,6 +127,12 @@ struct asfd_plan_s {
     int* it_ybox = nullptr;         // [runs][2] first tap row range
     int* it_xmap = nullptr;         // [band columns] first covering block | count << 24
     int* it_ymap = nullptr;         // [band rows] first covering run | count << 24
+    // atomic-free spread by block items merged in four colours (spread_block.cu)
+    bool blk = false, blk_dup = false;
+    int blk_warps = 0, blk_chunks = 0, blk_rows = 0, blk_ncols = 0, blk_nbx = 0, blk_nby = 0;
+    int blk_tw = 0, blk_th = 0;
+    int* blk_xbox = nullptr;        // [warp columns][2] first tap ranges, then
+    int* blk_ybox = nullptr;        // [block rows][2] (same allocation)
     int sx_min = 0, h_min = 0, sxw_min = 0;
     double min_step_x = 0.0, min_step_y = 0.0, row_spread_y = 0.0, col_spread_x = 0.0;
     long long tile_pairs = 0;
@@ -193,6 +201,11 @@ asfd_status launch_spread(asfd_plan_s* P, const float2* u1, cudaStream_t st);
 // deterministic item-tile spread (spread_item.cu): plan set-up and launch
 asfd_status plan_build_itemtile(asfd_plan_s* P, cudaStream_t st);
 asfd_status launch_spread_itemtile(asfd_plan_s* P, const float2* u1, cudaStream_t st);
+// atomic-free spread by block items (spread_block.cu): plan set-up from the
+// columns' x and rows' y coordinate ranges, and launch (into a zero band)
+asfd_status plan_build_block(asfd_plan_s* P, const std::vector<double>& cr,
+                             const std::vector<double>& rr, cudaStream_t st);
+asfd_status launch_spread_block(asfd_plan_s* P, const float2* u1, cudaStream_t st);
 // dense plans: add the spread of u1 into `grid` (not cleared; another plan's grid)
 asfd_status launch_spread_into(asfd_plan_s* P, const float2* u1, float2* grid, cudaStream_t st);
 // row / column passes over the band rows [ty0, ty1) (and columns [tx0, tx1)) in tiles
@@ -220,6 +233,12 @@ asfd_status launch_interp_grad(asfd_plan_s* P, const float2* u1, float2* gu1, fl
 // (two waves when the runs stay at least 32 rows long, else one).
 asfd_status dense_spread_warp_slots(int w, bool table, long long* slots);
 asfd_status interp_window_warp_slots(int w, long long* slots);
+// folding or wrapping maps: the same for spread_es_dense_kernel<.., true> and,
+// above kMaxWindowWidth, spread_fold_kernel (spread_split(w) lanes per column)
+asfd_status fold_spread_warp_slots(int w, bool table, long long* slots);
+asfd_status wide_fold_warp_slots(int w, long long* slots);
+// lanes that share a source column's register window
+__host__ __device__ constexpr int spread_split(int w) { return w <= kMaxWindowWidth ? 1 : w <= 12 ? 2 : 4; }
 int window_run_rows(long long n1y, long long ncb, long long slots);
 
 // plan helpers

@@ -19,7 +19,7 @@
 // error of g is that of the small term s q (about 1e-7 cells at the standard
 // workloads) rather than that of g itself.
 //
-// Both kernels own fine-grid tiles (storage coordinates, centred: cell index
+// The tile kernels own fine-grid tiles (storage coordinates, centred: cell index
 // = g + nf/2 mod nf): each CTA accumulates in shared memory every tap of
 // every sample whose footprint reaches its tile, and writes the tile to
 // global memory once.  No global atomics.
@@ -36,20 +36,22 @@
 //    each lane walks its samples down a source column and keeps their taps
 //    in a sliding W x W register window, so that shared memory sees about
 //    one row of W updates per sample instead of W rows.
-//  * spread_es_atomic_kernel (fallback for folding or wrapping maps):
-//    256 threads, one sample per thread, shared-memory atomics.
+//  * spread_es_dense_kernel<..., WRAP> and spread_fold_kernel (folding or
+//    wrapping maps, and what fits no atomic-free path): register windows
+//    flushed to wrapped cells of the fine grid with atomic adds.
 #include "spread.cuh"
 
 namespace asfd {
 
 namespace {
 
-template <int W, bool TAB>
-__global__ void __launch_bounds__(256) spread_es_atomic_kernel(SpreadArgs a)
+cudaError_t clear_band(const SpreadArgs& a, int tiles, cudaStream_t st)
 {
-    __shared__ float tre[kTileY * kTileX];
-    __shared__ float tim[kTileY * kTileX];
-    atomic_tile<W, TAB>(a, blockIdx.x, tre, tim, threadIdx.x, blockDim.x);
+    const size_t pitch = sizeof(float2) * (size_t)a.nfx;
+    const int c0 = a.band_tx0 * kTileX, r0 = a.band_ty0 * kTileY;
+    const size_t width = sizeof(float2) * (size_t)a.band_ntx * kTileX;
+    const size_t height = (size_t)(tiles / a.band_ntx) * kTileY;
+    return cudaMemset2DAsync(a.grid + (size_t)r0 * a.nfx + c0, pitch, 0, width, height, st);
 }
 
 // The dense kernels accumulate with atomic adds into a zero band: clear it
@@ -58,16 +60,12 @@ template <int W, bool TAB>
 cudaError_t launch_dense(const SpreadArgs& a, int tiles, bool clear, cudaStream_t st)
 {
     if (clear) {
-        const size_t pitch = sizeof(float2) * (size_t)a.nfx;
-        const int c0 = a.band_tx0 * kTileX, r0 = a.band_ty0 * kTileY;
-        const size_t width = sizeof(float2) * (size_t)a.band_ntx * kTileX;
-        const size_t height = (size_t)(tiles / a.band_ntx) * kTileY;
-        const cudaError_t e =
-            cudaMemset2DAsync(a.grid + (size_t)r0 * a.nfx + c0, pitch, 0, width, height, st);
+        const cudaError_t e = clear_band(a, tiles, st);
         if (e != cudaSuccess) return e;
     }
-    spread_es_dense_kernel<W, TAB><<<(a.dense_items + kDenseWarps - 1) / kDenseWarps,
-                                     32 * kDenseWarps, 0, st>>>(a, a.dense_items);
+    const unsigned blocks = (a.dense_items + kDenseWarps - 1) / kDenseWarps;
+    if (a.wrap) spread_es_dense_kernel<W, TAB, true><<<blocks, 32 * kDenseWarps, 0, st>>>(a, a.dense_items);
+    else spread_es_dense_kernel<W, TAB><<<blocks, 32 * kDenseWarps, 0, st>>>(a, a.dense_items);
     return cudaGetLastError();
 }
 
@@ -91,18 +89,18 @@ cudaError_t launch_w(const SpreadArgs& a, int tiles, bool colored, bool windowed
             return cudaGetLastError();
         }
     }
-    spread_es_atomic_kernel<W, false><<<tiles, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    if (clear) {
+        const cudaError_t e = clear_band(a, tiles, st);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_wide_fold(a, W, st);
 }
 
-cudaError_t launch_table(const SpreadArgs& a, int tiles, bool colored, bool clear, cudaStream_t st)
+cudaError_t launch_table(const SpreadArgs& a, int tiles, bool clear, cudaStream_t st)
 {
     if (a.dense_rows > 0) return launch_dense<kLearnW, true>(a, tiles, clear, st);
-    if (colored)
-        spread_es_colored_kernel<kLearnW, kTileX, kColTileY, true>
-            <<<tiles * (kTileY / kColTileY), 32, 0, st>>>(a);
-    else
-        spread_es_atomic_kernel<kLearnW, true><<<tiles, 256, 0, st>>>(a);
+    spread_es_colored_kernel<kLearnW, kTileX, kColTileY, true>
+        <<<tiles * (kTileY / kColTileY), 32, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -121,6 +119,17 @@ asfd_status resident_warps(const void* kernel, long long* slots)
 }
 
 }  // namespace
+
+asfd_status fold_spread_warp_slots(int w, bool table, long long* slots)
+{
+    if (table) return resident_warps((const void*)spread_es_dense_kernel<kLearnW, true, true>, slots);
+    switch (w) {
+#define ASFD_SW(W) case W: return resident_warps((const void*)spread_es_dense_kernel<W, false, true>, slots);
+        ASFD_SW(2) ASFD_SW(3) ASFD_SW(4) ASFD_SW(5) ASFD_SW(6) ASFD_SW(7)
+#undef ASFD_SW
+        default: return wide_fold_warp_slots(w, slots);
+    }
+}
 
 asfd_status dense_spread_warp_slots(int w, bool table, long long* slots)
 {
@@ -171,8 +180,9 @@ SpreadArgs make_spread_args(const asfd_plan_s* P, const float2* u1)
     a.sx_min = P->sx_min;
     a.h_min = P->h_min;
     a.sxw_min = P->sxw_min;
-    a.dense_rows = P->dense ? P->dense_rows : 0;
-    a.dense_items = P->dense ? P->dense_items : 0;
+    a.dense_rows = P->dense || P->fold ? P->dense_rows : 0;
+    a.dense_items = P->dense || P->fold ? P->dense_items : 0;
+    a.wrap = P->fold;
     a.inc_d = (float)P->inc_d;
     a.half_w = 0.5f * (float)P->w;
     a.beta_log2e = (float)(P->beta * 1.4426950408889634074);
@@ -216,9 +226,13 @@ asfd_status launch_spread(asfd_plan_s* P, const float2* u1, cudaStream_t st)
     const bool clear = !P->band_clean;
     P->band_clean = false;
     if (P->itemtile) return launch_spread_itemtile(P, u1, st);
+    if (P->blk) {
+        if (clear) ASFD_CUDA(clear_band(a, tiles, st));
+        return launch_spread_block(P, u1, st);
+    }
     cudaError_t e;
     if (P->learned) {
-        e = launch_table(a, tiles, colored, clear, st);
+        e = launch_table(a, tiles, clear, st);
         if (e != cudaSuccess) return cuda_fail(e, "learned spread kernel launch");
         return ASFD_OK;
     }

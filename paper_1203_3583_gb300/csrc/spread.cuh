@@ -27,6 +27,7 @@ struct SpreadArgs {
     int sxw_min;       // column stride of the register-window kernel
     int dense_rows;    // rows per run of the dense (global-atomic) window kernel (0: not used)
     int dense_items;   // its warp items (32 columns x dense_rows rows each)
+    bool wrap;         // the map folds or wraps (dense_rows of the wrapping kernels)
     float inc_d;       // incident depth phase, half-turns per unit d1/z0
     float half_w;      // w/2
     float beta_log2e;  // beta * log2(e)
@@ -559,7 +560,8 @@ constexpr int kDenseSpare = 0;
 constexpr int kDenseRing = 4;   // ring slots (> kDenseAhead, power of two)
 constexpr int kDenseRingBytes = kDenseRing * (32 * (8 + 4) + 32);  // per warp
 
-template <int W, bool TAB = false>
+// WRAP: the cells' columns wrap around the periodic grid.
+template <int W, bool TAB = false, bool WRAP = false>
 __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, int lane,
                                                    char* ring, float4* tsm = nullptr)
 {
@@ -608,11 +610,18 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
         // periodic grid, so the window's columns lie in [0, nfx) and the
         // addresses are one base plus constant offsets; the clamp keeps every
         // address inside the row all the same
-        const int xc = min(max(X0, 0), a.nfx - W - maxoff);
-        float2* row = a.grid + (size_t)((R0 + b) & my) * a.nfx + xc;
+        if constexpr (WRAP) {
+            float2* row = a.grid + (size_t)((R0 + b) & my) * a.nfx;
 #pragma unroll
-        for (int i = 0; i < WX; ++i)
-            if (lane_on && i < W + maxoff) atomicAdd(row + i, acc[b][i]);
+            for (int i = 0; i < WX; ++i)
+                if (lane_on && i < W + maxoff) atomicAdd(row + ((X0 + i) & (a.nfx - 1)), acc[b][i]);
+        } else {
+            const int xc = min(max(X0, 0), a.nfx - W - maxoff);
+            float2* row = a.grid + (size_t)((R0 + b) & my) * a.nfx + xc;
+#pragma unroll
+            for (int i = 0; i < WX; ++i)
+                if (lane_on && i < W + maxoff) atomicAdd(row + i, acc[b][i]);
+        }
     };
     // u1 and q of the run's rows are copied asynchronously (cp.async) into a
     // per-lane ring of kDenseRing slots in shared memory, kDenseAhead rows
@@ -721,15 +730,15 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
 // registers capped for more resident warps spilled and ran slower)
 constexpr int kDenseWarps = 4;
 
-template <int W, bool TAB = false>
+template <int W, bool TAB = false, bool WRAP = false>
 __global__ void __launch_bounds__(32 * kDenseWarps) spread_es_dense_kernel(SpreadArgs a, int items)
 {
     __shared__ float4 tsm[kDenseWarps][TAB ? 8 * W : 1];
     __shared__ __align__(16) char ring[kDenseWarps][kDenseRingBytes];
     const int it = blockIdx.x * kDenseWarps + threadIdx.x / 32;
     if (it < items)
-        window_atomic_item<W, TAB>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
-                                   tsm[threadIdx.x / 32]);
+        window_atomic_item<W, TAB, WRAP>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
+                                         tsm[threadIdx.x / 32]);
 }
 
 // Fallback spread of band tile `tile` (kTileX x kTileY) by a whole block:
@@ -813,6 +822,9 @@ __device__ __forceinline__ void atomic_tile(const SpreadArgs& a, int tile, float
         g4[o] = make_float4(tre[l], tim[l], tre[l + 1], tim[l + 1]);
     }
 }
+
+// widths above kMaxWindowWidth of a folding or wrapping map (spread_block.cu)
+cudaError_t launch_wide_fold(const SpreadArgs& a, int w, cudaStream_t st);
 
 // Spread arguments of a plan for the field u1.
 SpreadArgs make_spread_args(const asfd_plan_s* P, const float2* u1);
