@@ -116,6 +116,7 @@ struct asfd_plan_s {
     bool colored = false;
     bool windowed = false;          // register-window kernel applies (w <= kMaxWindowWidth)
     bool dense = false;             // dense map: register windows flushed with global atomics
+    bool wraps = false;             // some footprint wraps around the periodic grid
     bool fold = false;              // folding or wrapping map: register windows flushed with
                                     // global atomics to wrapped cells
     int dense_rows = 0, dense_items = 0;
@@ -226,13 +227,12 @@ asfd_status launch_fft_rows_adj(asfd_plan_s* P, cudaStream_t st);
 asfd_status launch_interp_grad(asfd_plan_s* P, const float2* u1, float2* gu1, float* gd1,
                                cudaStream_t st);
 
-// Warp-item scheduling of the column-walking window kernels (dense spread,
-// windowed interpolation): warps of the kernel that the current device keeps
+// Warp-item scheduling of the column-walking window kernels (dense spread):
+// warps of the kernel that the current device keeps
 // resident at once (SMs x resident blocks x 4 warps), and the rows per run
 // that make the items of 32 columns x rows fill whole waves of those slots
 // (two waves when the runs stay at least 32 rows long, else one).
 asfd_status dense_spread_warp_slots(int w, bool table, long long* slots);
-asfd_status interp_window_warp_slots(int w, long long* slots);
 // folding or wrapping maps: the same for spread_es_dense_kernel<.., true> and,
 // above kMaxWindowWidth, spread_fold_kernel (spread_split(w) lanes per column)
 asfd_status fold_spread_warp_slots(int w, bool table, long long* slots);

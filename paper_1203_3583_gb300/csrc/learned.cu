@@ -781,9 +781,8 @@ asfd_status learned_gradient(asfd_plan_s* P, const float2* u1, const float2* ref
     a.nfy = P->nfy;
     a.half_w = 0.5f * kLearnW;
     a.inc_d = (float)P->inc_d;
-    // (a dense plan's footprints do not wrap around the periodic grid)
     const unsigned tgb = (unsigned)((nst + kTgWarps - 1) / kTgWarps);
-    if (P->dense) table_grad_kernel<false><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
+    if (!P->wraps) table_grad_kernel<false><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
     else table_grad_kernel<true><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
     const int groups = (nst + kBackTiles - 1) / kBackTiles;
     mlp_backward_kernel<<<groups < kBackBlocks ? groups : kBackBlocks, 256, 0, st>>>(

@@ -693,6 +693,7 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
     P->band_ty0 = by0;
     P->band_ty1 = by1 + 1;
     P->max_abs_eps = me;
+    P->wraps = wrapx || wrapy;
     asfd_status cs = plan_build_colored(P, wrapx || wrapy, st);
     if (cs != ASFD_OK) return cs;
     P->tile_pairs = 0;

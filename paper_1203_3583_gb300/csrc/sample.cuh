@@ -146,27 +146,6 @@ __device__ __forceinline__ float2 sample_value_fast(const Raw& r, float inc_d)
 
 namespace asfd {
 
-// psi(z) and d psi / dz of the ES kernel at z (fast MUFU forms).  The
-// derivative -psi beta (2/w) u / sqrt(1 - u^2) is infinite at the support
-// edge, where psi itself is e^-beta; 1 - u^2 is floored at 1e-12 so that the
-// edge tap (weight ~e^-beta) stays finite.
-__device__ __forceinline__ void es_weight_deriv_fast(float z, float two_over_w, float beta_log2e,
-                                                     float beta, float& psi, float& dpsi)
-{
-    const float u = z * two_over_w;
-    const float r = fmaxf(fmaf(-u, u, 1.0f), 1e-12f);
-    float rs, e;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs) : "f"(r));
-    const float arg = beta_log2e * fmaf(r, rs, -1.0f);
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(arg));
-    psi = e;
-    dpsi = -e * beta * two_over_w * u * rs;
-}
-
-}  // namespace asfd
-
-namespace asfd {
-
 // Learned kernel weights: tap a of axis x is sum_k c[0][a][k] t^k with
 // t = 2 dx - 1 (monomials on [-1, 1], Horner), likewise y with dy.
 template <int W>
