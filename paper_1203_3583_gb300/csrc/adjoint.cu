@@ -88,6 +88,8 @@ template <int W, bool WRAP>
 __global__ void __launch_bounds__(32 * kInterpWarps) interp_kernel(InterpArgs a, int iters)
 {
     constexpr int NX = (W + 2) & ~1;
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
     const int nx = blockIdx.x * 32 + lane;
     if (nx >= a.n1x) return;
@@ -234,18 +236,18 @@ asfd_status launch_interp_grad(asfd_plan_s* P, const float2* u1, float2* gu1, fl
            (long long)cols * ((P->prm.n1y + iters * kInterpWarps - 1) / (iters * kInterpWarps)) < 2432)
         iters /= 2;
     const dim3 grid(cols, (P->prm.n1y + iters * kInterpWarps - 1) / (iters * kInterpWarps));
+    cudaError_t e = cudaSuccess;
     switch (P->w) {
-#define ASFD_IW(W)                                                                          \
-    case W:                                                                                 \
-        if (P->wraps) interp_kernel<W, true><<<grid, 32 * kInterpWarps, 0, st>>>(a, iters); \
-        else interp_kernel<W, false><<<grid, 32 * kInterpWarps, 0, st>>>(a, iters);         \
+#define ASFD_IW(W)                                                                                    \
+    case W:                                                                                           \
+        e = P->wraps ? launch_chained(interp_kernel<W, true>, grid, 32 * kInterpWarps, 0, st, a, iters) \
+                     : launch_chained(interp_kernel<W, false>, grid, 32 * kInterpWarps, 0, st, a, iters); \
         break;
         ASFD_IW(2) ASFD_IW(3) ASFD_IW(4) ASFD_IW(5) ASFD_IW(6) ASFD_IW(7) ASFD_IW(8) ASFD_IW(9)
         ASFD_IW(10) ASFD_IW(11) ASFD_IW(12) ASFD_IW(13) ASFD_IW(14) ASFD_IW(15) ASFD_IW(16)
 #undef ASFD_IW
         default: return fail(ASFD_ERR_UNSUPPORTED, "kernel width outside 2..16");
     }
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "interp_kernel launch");
     return ASFD_OK;
 }

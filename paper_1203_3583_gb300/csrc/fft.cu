@@ -26,6 +26,8 @@ __global__ void __launch_bounds__(RowCfg<L>::THREADS, L == 4096 ? 4 : 1)
 fft_rows_kernel(RowArgs a)
 {
     extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
     rows_body<L>(a, blockIdx.x, sm, threadIdx.x);
 }
 
@@ -34,6 +36,8 @@ __global__ void __launch_bounds__(ColCfg<L>::THREADS, ColCfgSel<L>::MIN_BLOCKS)
 fft_cols_kernel(ColArgs a)
 {
     extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
     cols_body<L, ColCfg<L>::LPC>(a, blockIdx.x, sm, threadIdx.x);
 }
 
@@ -47,6 +51,8 @@ fft_cols_adj_kernel(const float2* __restrict__ g, int m2x, int m2y, const float2
 {
     using C = ColCfg<L>;
     extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
     const int c = threadIdx.x % C::LPC, t = threadIdx.x / C::LPC;
     const int col = blockIdx.x * C::LPC + c;
     const bool active = col < m2x;
@@ -78,6 +84,8 @@ fft_rows_adj_kernel(const float2* __restrict__ rows, int nrows, int m2x, float2*
 {
     using C = RowCfg<L>;
     extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
     const int line = threadIdx.x / C::TPL, t = threadIdx.x % C::TPL;
     const int r = blockIdx.x * C::LPC + line;
     const bool active = r < nrows;
@@ -102,6 +110,8 @@ fft_lines_kernel(const float2* in, float2* out, int lines, const float2* __restr
 {
     using C = RowCfg<L>;
     extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
     const int line = threadIdx.x / C::TPL, t = threadIdx.x % C::TPL;
     const int r = blockIdx.x * C::LPC + line;
     const bool active = r < lines;
@@ -130,8 +140,7 @@ cudaError_t rows_L(const RowArgs& a, cudaStream_t st)
     std::call_once(once, [] { attr = set_smem(fft_rows_kernel<L>, C::SMEM_BYTES); });
     if (attr != cudaSuccess) return attr;
     const int blocks = (a.nrows + C::LPC - 1) / C::LPC;
-    fft_rows_kernel<L><<<blocks, C::THREADS, C::SMEM_BYTES, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fft_rows_kernel<L>, blocks, C::THREADS, C::SMEM_BYTES, st, a);
 }
 
 template <int L>
@@ -144,8 +153,7 @@ cudaError_t cols_L(const ColArgs& a, cudaStream_t st)
     if (attr != cudaSuccess) return attr;
     const int blocks = (a.col1 - a.col0 + C::LPC - 1) / C::LPC;
     if (blocks <= 0) return cudaSuccess;
-    fft_cols_kernel<L><<<blocks, C::THREADS, C::SMEM_BYTES, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(fft_cols_kernel<L>, blocks, C::THREADS, C::SMEM_BYTES, st, a);
 }
 
 template <int L>
@@ -158,9 +166,8 @@ cudaError_t cols_adj_L(const float2* g, int m2x, int m2y, const float2* cx, cons
     std::call_once(once, [] { attr = set_smem(fft_cols_adj_kernel<L>, C::SMEM_BYTES); });
     if (attr != cudaSuccess) return attr;
     const int blocks = (m2x + C::LPC - 1) / C::LPC;
-    fft_cols_adj_kernel<L><<<blocks, C::THREADS, C::SMEM_BYTES, st>>>(g, m2x, m2y, cx, cy, rows,
-                                                                      row0, nrows, tw);
-    return cudaGetLastError();
+    return launch_chained(fft_cols_adj_kernel<L>, blocks, C::THREADS, C::SMEM_BYTES, st, g, m2x, m2y,
+                          cx, cy, rows, row0, nrows, tw);
 }
 
 template <int L>
@@ -173,9 +180,8 @@ cudaError_t rows_adj_L(const float2* rows, int nrows, int m2x, float2* grid, int
     std::call_once(once, [] { attr = set_smem(fft_rows_adj_kernel<L>, C::SMEM_BYTES); });
     if (attr != cudaSuccess) return attr;
     const int blocks = (nrows + C::LPC - 1) / C::LPC;
-    fft_rows_adj_kernel<L><<<blocks, C::THREADS, C::SMEM_BYTES, st>>>(rows, nrows, m2x, grid, row0,
-                                                                      col_lo, col_hi, tw);
-    return cudaGetLastError();
+    return launch_chained(fft_rows_adj_kernel<L>, blocks, C::THREADS, C::SMEM_BYTES, st, rows, nrows,
+                          m2x, grid, row0, col_lo, col_hi, tw);
 }
 
 template <int L, int S>
@@ -187,8 +193,8 @@ cudaError_t lines_L(const float2* in, float2* out, int lines, const float2* tw, 
     std::call_once(once, [] { attr = set_smem(fft_lines_kernel<L, S>, C::SMEM_BYTES); });
     if (attr != cudaSuccess) return attr;
     const int blocks = (lines + C::LPC - 1) / C::LPC;
-    fft_lines_kernel<L, S><<<blocks, C::THREADS, C::SMEM_BYTES, st>>>(in, out, lines, tw);
-    return cudaGetLastError();
+    return launch_chained(fft_lines_kernel<L, S>, blocks, C::THREADS, C::SMEM_BYTES, st, in, out, lines,
+                          tw);
 }
 
 #define ASFD_FFT_SWITCH(n, CALL)       \

@@ -64,9 +64,11 @@ cudaError_t launch_dense(const SpreadArgs& a, int tiles, bool clear, cudaStream_
         if (e != cudaSuccess) return e;
     }
     const unsigned blocks = (a.dense_items + kDenseWarps - 1) / kDenseWarps;
-    if (a.wrap) spread_es_dense_kernel<W, TAB, true><<<blocks, 32 * kDenseWarps, 0, st>>>(a, a.dense_items);
-    else spread_es_dense_kernel<W, TAB><<<blocks, 32 * kDenseWarps, 0, st>>>(a, a.dense_items);
-    return cudaGetLastError();
+    if (a.wrap)
+        return launch_chained(spread_es_dense_kernel<W, TAB, true>, blocks, 32 * kDenseWarps, 0, st, a,
+                              a.dense_items);
+    return launch_chained(spread_es_dense_kernel<W, TAB, false>, blocks, 32 * kDenseWarps, 0, st, a,
+                          a.dense_items);
 }
 
 template <int W>
@@ -198,18 +200,18 @@ asfd_status launch_spread_into(asfd_plan_s* P, const float2* u1, float2* grid, c
     a.grid = grid;
     if (a.dense_items <= 0) return ASFD_OK;
     cudaError_t e = cudaSuccess;
+    const unsigned blocks = (a.dense_items + kDenseWarps - 1) / kDenseWarps;
     if (P->learned) {
-        spread_es_dense_kernel<kLearnW, true><<<(a.dense_items + kDenseWarps - 1) / kDenseWarps,
-                                               32 * kDenseWarps, 0, st>>>(a, a.dense_items);
+        e = launch_chained(spread_es_dense_kernel<kLearnW, true, false>, blocks, 32 * kDenseWarps, 0, st, a,
+                           a.dense_items);
     } else {
         switch (P->w) {
-#define ASFD_SI(W) case W: spread_es_dense_kernel<W, false><<<(a.dense_items + kDenseWarps - 1) / kDenseWarps, 32 * kDenseWarps, 0, st>>>(a, a.dense_items); break;
+#define ASFD_SI(W) case W: e = launch_chained(spread_es_dense_kernel<W, false, false>, blocks, 32 * kDenseWarps, 0, st, a, a.dense_items); break;
             ASFD_SI(2) ASFD_SI(3) ASFD_SI(4) ASFD_SI(5) ASFD_SI(6) ASFD_SI(7)
 #undef ASFD_SI
             default: return fail(ASFD_ERR_UNSUPPORTED, "dense spread widths are 2..7");
         }
     }
-    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "spread kernel launch");
     return ASFD_OK;
 }

@@ -736,6 +736,8 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_es_dense_kernel(Sprea
     __shared__ float4 tsm[kDenseWarps][TAB ? 8 * W : 1];
     __shared__ __align__(16) char ring[kDenseWarps][kDenseRingBytes];
     const int it = blockIdx.x * kDenseWarps + threadIdx.x / 32;
+    chain_next();
+    chain_wait();
     if (it < items)
         window_atomic_item<W, TAB, WRAP>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
                                          tsm[threadIdx.x / 32]);

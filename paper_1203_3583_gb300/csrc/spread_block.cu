@@ -90,6 +90,8 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
     constexpr int S = blk_split(W), WS = blk_cols(W), HC = 32 / S;
     constexpr unsigned full = 0xffffffffu;
     extern __shared__ float4 blk_smem[];
+    chain_next();
+    chain_wait();
     const SpreadArgs& a = ba.s;
     const int warps = blockDim.x / 32, wid = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int sub = lane / HC, slot = lane % HC;
@@ -341,6 +343,8 @@ template <int W>
 __global__ void __launch_bounds__(32 * kDenseWarps) spread_fold_kernel(SpreadArgs a)
 {
     constexpr int S = blk_split(W), WS = blk_cols(W), HC = 32 / S, PAIRS = (W + WS + 1) / 2;
+    chain_next();
+    chain_wait();
     const int it = blockIdx.x * kDenseWarps + threadIdx.x / 32, lane = threadIdx.x % 32;
     const int sub = lane / HC, slot = lane % HC;
     const int ncb = (a.n1x + HC - 1) / HC;
@@ -576,13 +580,12 @@ cudaError_t launch_wide_fold(const SpreadArgs& a, int w, cudaStream_t st)
 {
     const unsigned blocks = (unsigned)((a.dense_items + kDenseWarps - 1) / kDenseWarps);
     switch (w) {
-#define ASFD_FL(W) case W: spread_fold_kernel<W><<<blocks, 32 * kDenseWarps, 0, st>>>(a); break;
+#define ASFD_FL(W) case W: return launch_chained(spread_fold_kernel<W>, blocks, 32 * kDenseWarps, 0, st, a);
         ASFD_FL(8) ASFD_FL(9) ASFD_FL(10) ASFD_FL(11) ASFD_FL(12) ASFD_FL(13) ASFD_FL(14) ASFD_FL(15)
         ASFD_FL(16)
 #undef ASFD_FL
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 asfd_status launch_spread_block(asfd_plan_s* P, const float2* u1, cudaStream_t st)
@@ -606,10 +609,9 @@ asfd_status launch_spread_block(asfd_plan_s* P, const float2* u1, cudaStream_t s
         a.cy = c / 2;
         const dim3 grid((a.nbx + 1 - a.cx) / 2, (a.nby + 1 - a.cy) / 2);
         if (grid.x == 0 || grid.y == 0) continue;
-        kern<<<grid, 32 * P->blk_warps, smem, st>>>(a);
+        const cudaError_t e = launch_chained(kern, grid, 32 * P->blk_warps, smem, st, a);
+        if (e != cudaSuccess) return cuda_fail(e, "spread_block_kernel launch");
     }
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "spread_block_kernel launch");
     return ASFD_OK;
 }
 

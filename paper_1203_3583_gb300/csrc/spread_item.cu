@@ -207,6 +207,8 @@ template <int W>
 __global__ void __launch_bounds__(32 * kItemWarps) spread_item_kernel(ItemArgs ia, int items)
 {
     extern __shared__ float4 item_smem[];
+    chain_next();
+    chain_wait();
     const int wid = threadIdx.x / 32;
     char* ring = reinterpret_cast<char*>(item_smem) + wid * kDenseRingBytes;
     float2* tile = reinterpret_cast<float2*>(reinterpret_cast<char*>(item_smem) +
@@ -229,6 +231,8 @@ item_gather_kernel(const float2* __restrict__ scratch, const int* __restrict__ x
                    const int* __restrict__ ymap, int x0, int y0, int bw, int bh, int ncb, int tw,
                    int th, float2* __restrict__ grid, int nfx)
 {
+    chain_next();
+    chain_wait();
     const int bx = blockIdx.x * blockDim.x + threadIdx.x;
     if (bx >= bw) return;
     const int x = x0 + bx;
@@ -403,23 +407,20 @@ asfd_status launch_spread_itemtile(asfd_plan_s* P, const float2* u1, cudaStream_
     ia.th = P->it_th;
     const size_t smem = kItemWarps * ((size_t)kDenseRingBytes + sizeof(float2) * ia.tw * ia.th);
     const unsigned blocks = (unsigned)((P->it_items + kItemWarps - 1) / kItemWarps);
+    cudaError_t e = cudaSuccess;
     switch (P->w) {
-#define ASFD_IL(W)                                                                        \
-    case W:                                                                               \
-        spread_item_kernel<W><<<blocks, 32 * kItemWarps, smem, st>>>(ia, P->it_items);   \
-        break;
+#define ASFD_IL(W) case W: e = launch_chained(spread_item_kernel<W>, blocks, 32 * kItemWarps, smem, st, ia, P->it_items); break;
         ASFD_IL(2) ASFD_IL(3) ASFD_IL(4) ASFD_IL(5) ASFD_IL(6) ASFD_IL(7)
 #undef ASFD_IL
         default: return fail(ASFD_ERR_UNSUPPORTED, "item-tile spread widths are 2..7");
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "spread_item_kernel launch");
     const int bx0 = P->band_tx0 * kTileX, by0 = P->band_ty0 * kTileY;
     const int bw = (P->band_tx1 - P->band_tx0) * kTileX, bh = (P->band_ty1 - P->band_ty0) * kTileY;
-    item_gather_kernel<<<dim3((bw + 127) / 128, (bh + kGatherRows - 1) / kGatherRows), 128, 0, st>>>(
-        P->rows, P->it_xbox, P->it_ybox, P->it_xmap, P->it_ymap, bx0, by0, bw, bh, P->it_ncb,
-        P->it_tw, P->it_th, P->grid, P->nfx);
-    e = cudaGetLastError();
+    e = launch_chained(item_gather_kernel, dim3((bw + 127) / 128, (bh + kGatherRows - 1) / kGatherRows),
+                       128, 0, st, (const float2*)P->rows, (const int*)P->it_xbox,
+                       (const int*)P->it_ybox, (const int*)P->it_xmap, (const int*)P->it_ymap, bx0, by0,
+                       bw, bh, P->it_ncb, P->it_tw, P->it_th, P->grid, P->nfx);
     if (e != cudaSuccess) return cuda_fail(e, "item_gather_kernel launch");
     return ASFD_OK;
 }
