@@ -38,7 +38,8 @@ __device__ __forceinline__ void sample_pos(const AxisEntry& ex, const AxisEntry&
 __device__ __forceinline__ float sample_phase(const AxisEntry& ex, const AxisEntry& ey, float q,
                                               float inc_d)
 {
-    return fmaf(inc_d, __fdividef(q, 1.0f + q), (ex.a + ey.a) * q);
+    const float ph = (ex.a + ey.a) * q;
+    return inc_d != 0.f ? fmaf(inc_d, __fdividef(q, 1.0f + q), ph) : ph;  // (uniform)
 }
 
 // c = u1 E_x E_y exp(i pi (a_x + a_y) q + i pi inc_d q/(1 + q))

@@ -218,14 +218,18 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b)
 }
 
 // ES weights of two taps at once (packed FP32x2 arithmetic; the square root
-// and exponential on the MUFU unit as in es_weight_fast).
+// and exponential on the MUFU unit as in es_weight_fast).  CLAMP: a tap can
+// lie at the support's edge or beyond, where 1 - (2z/w)^2 is not positive.
+template <bool CLAMP = true>
 __device__ __forceinline__ float2 es_weight2_fast(float2 z, float neg_c2, float beta_log2e)
 {
     // r = 1 - (2z/w)^2 = fma(z * neg_c2, z, 1)
     const float2 t = mul2(z, neg_c2);
     float2 r = fma2v(t, z, make_float2(1.f, 1.f));
-    r.x = fmaxf(r.x, 1e-30f);
-    r.y = fmaxf(r.y, 1e-30f);
+    if constexpr (CLAMP) {
+        r.x = fmaxf(r.x, 1e-30f);
+        r.y = fmaxf(r.y, 1e-30f);
+    }
     float2 rs, e;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs.x) : "f"(r.x));
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(rs.y) : "f"(r.y));
@@ -253,8 +257,11 @@ __device__ __forceinline__ void window_add(float2 (&acc)[W][WX], bool fresh, int
 #pragma unroll
     for (int b = 0; b < W; ++b) {
         // tap b's offsets from the sample in y and x, one packed add
-        const float2 e = es_weight2_fast(add2(bxy, make_float2((float)b, (float)b)), neg_c2,
-                                         a.beta_log2e);
+        // (taps 1 .. W - 2 lie inside the support, unless offn moves them)
+        const float2 z = add2(bxy, make_float2((float)b, (float)b));
+        const float2 e = (WX == W && b > 0 && b + 1 < W)
+                             ? es_weight2_fast<false>(z, neg_c2, a.beta_log2e)
+                             : es_weight2_fast<true>(z, neg_c2, a.beta_log2e);
         wy[b] = e.x;
         wxe[b] = e.y;
     }

@@ -84,6 +84,46 @@ __device__ __forceinline__ void blk_weight_pair(const SpreadArgs& a, float neg_c
     e[k1] = v.y;
 }
 
+// Adds a sample to a window: fresh (every slot is overwritten), or with its
+// first tap row d = 0, 1 or 2 rows below the window's (whose d top rows have
+// left it: the rest moves up inside the multiply-adds).
+template <int W, int WS>
+__device__ __forceinline__ void blk_accumulate(float2 (&acc)[W][WS], bool fresh, int d, float2 c,
+                                               const float (&wy)[W], const float (&wx)[WS])
+{
+    if (fresh) {
+#pragma unroll
+        for (int b = 0; b < W; ++b) {
+            const float2 cb = mul2(c, wy[b]);
+#pragma unroll
+            for (int i = 0; i < WS; ++i) acc[b][i] = mul2(cb, wx[i]);
+        }
+    } else if (d == 0) {
+#pragma unroll
+        for (int b = 0; b < W; ++b) {
+            const float2 cb = mul2(c, wy[b]);
+#pragma unroll
+            for (int i = 0; i < WS; ++i) acc[b][i] = fma2(cb, wx[i], acc[b][i]);
+        }
+    } else if (d == 1) {
+#pragma unroll
+        for (int b = 0; b < W; ++b) {
+            const float2 cb = mul2(c, wy[b]);
+#pragma unroll
+            for (int i = 0; i < WS; ++i)
+                acc[b][i] = (b + 1 < W) ? fma2(cb, wx[i], acc[b + 1][i]) : mul2(cb, wx[i]);
+        }
+    } else {
+#pragma unroll
+        for (int b = 0; b < W; ++b) {
+            const float2 cb = mul2(c, wy[b]);
+#pragma unroll
+            for (int i = 0; i < WS; ++i)
+                acc[b][i] = (b + 2 < W) ? fma2(cb, wx[i], acc[b + 2][i]) : mul2(cb, wx[i]);
+        }
+    }
+}
+
 template <int W, bool DUP>
 __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs ba)
 {
@@ -252,37 +292,7 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
             }
             R0 = l0y;
             const float2 c = sample_value_fast(u, ex, ey, q, a.inc_d);
-            if (fresh) {
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float2 cb = mul2(c, wy[b]);
-#pragma unroll
-                    for (int i = 0; i < WS; ++i) acc[b][i] = mul2(cb, wx[i]);
-                }
-            } else if (d == 0) {
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float2 cb = mul2(c, wy[b]);
-#pragma unroll
-                    for (int i = 0; i < WS; ++i) acc[b][i] = fma2(cb, wx[i], acc[b][i]);
-                }
-            } else if (d == 1) {
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float2 cb = mul2(c, wy[b]);
-#pragma unroll
-                    for (int i = 0; i < WS; ++i)
-                        acc[b][i] = (b + 1 < W) ? fma2(cb, wx[i], acc[b + 1][i]) : mul2(cb, wx[i]);
-                }
-            } else {
-#pragma unroll
-                for (int b = 0; b < W; ++b) {
-                    const float2 cb = mul2(c, wy[b]);
-#pragma unroll
-                    for (int i = 0; i < WS; ++i)
-                        acc[b][i] = (b + 2 < W) ? fma2(cb, wx[i], acc[b + 2][i]) : mul2(cb, wx[i]);
-                }
-            }
+            blk_accumulate<W, WS>(acc, fresh, d, c, wy, wx);
         }
         flush(live ? W : 0, W);
         asm volatile("cp.async.wait_group 0;");
@@ -396,21 +406,12 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_fold_kernel(SpreadArg
         const float zy = dy - a.half_w, zx = dx - a.half_w + (float)(sub * WS);
 #pragma unroll
         for (int k = 0; k < PAIRS; ++k) blk_weight_pair<W, WS>(a, neg_c2, zy, zx, k, e);
-        // one row of the window after another; a sample `up` rows lower takes
-        // the sums of row b + up
-        const int up = fresh ? W : d;
+        float wx[WS], wy[W];
 #pragma unroll
-        for (int b = 0; b < W; ++b) {
-            const float2 cb = mul2(c, e[b]);
+        for (int b = 0; b < W; ++b) wy[b] = e[b];
 #pragma unroll
-            for (int i = 0; i < WS; ++i) {
-                float2 v = make_float2(0.f, 0.f);
-                if (up == 0) v = acc[b][i];
-                else if (up == 1 && b + 1 < W) v = acc[b + 1][i];
-                else if (up == 2 && b + 2 < W) v = acc[b + 2][i];
-                acc[b][i] = fma2(cb, e[W + i], v);
-            }
-        }
+        for (int i = 0; i < WS; ++i) wx[i] = e[W + i];
+        blk_accumulate<W, WS>(acc, fresh, d, c, wy, wx);
     }
     flush(W);
 }
