@@ -384,6 +384,31 @@ asfd_status launch_fft_lines_tw(int n, int lines, int sign, const float2* in, fl
     return ASFD_OK;
 }
 
+// One twiddle table per (device, length), built on first use.
+asfd_status fft_line_twiddles(int n, const float2** out, cudaStream_t st)
+{
+    static std::mutex mu;
+    static float2* tables[64][15] = {};
+    int dev = 0;
+    ASFD_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return fail(ASFD_ERR_UNSUPPORTED, "device ordinal above 63");
+    const int lg = ilog2_c(n);
+    std::lock_guard<std::mutex> g(mu);
+    if (!tables[dev][lg]) {
+        float2* p = nullptr;
+        ASFD_CUDA(cudaMalloc(&p, sizeof(float2) * n));
+        asfd_status s = build_twiddles(p, n, st);
+        if (s != ASFD_OK) {
+            cudaFree(p);
+            return s;
+        }
+        ASFD_CUDA(cudaStreamSynchronize(st));
+        tables[dev][lg] = p;
+    }
+    *out = tables[dev][lg];
+    return ASFD_OK;
+}
+
 asfd_status launch_fft_lines(int n, int lines, int sign, const float2* in, float2* out,
                              cudaStream_t st)
 {
@@ -392,29 +417,9 @@ asfd_status launch_fft_lines(int n, int lines, int sign, const float2* in, float
         return fail(ASFD_ERR_ARG, "asfd_fft_lines: n must be a power of two in [16, 16384], "
                                   "sign +-1, non-NULL buffers");
     if (lines == 0) return ASFD_OK;
-    // one twiddle table per (device, length), built on first use
-    static std::mutex mu;
-    static float2* tables[64][15] = {};
-    int dev = 0;
-    ASFD_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(ASFD_ERR_UNSUPPORTED, "device ordinal above 63");
-    const int lg = ilog2_c(n);
-    float2* tw = nullptr;
-    {
-        std::lock_guard<std::mutex> g(mu);
-        if (!tables[dev][lg]) {
-            float2* p = nullptr;
-            ASFD_CUDA(cudaMalloc(&p, sizeof(float2) * n));
-            asfd_status s = build_twiddles(p, n, st);
-            if (s != ASFD_OK) {
-                cudaFree(p);
-                return s;
-            }
-            ASFD_CUDA(cudaStreamSynchronize(st));
-            tables[dev][lg] = p;
-        }
-        tw = tables[dev][lg];
-    }
+    const float2* tw = nullptr;
+    const asfd_status ts = fft_line_twiddles(n, &tw, st);
+    if (ts != ASFD_OK) return ts;
     cudaError_t e = cudaSuccess;
     if (sign < 0) {
 #define ASFD_LN(L) e = lines_L<L, -1>(in, out, lines, tw, st)

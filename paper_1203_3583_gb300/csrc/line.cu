@@ -16,13 +16,19 @@
 // integer/fraction split of g + nf/2; an execution multiplies u1 by E,
 // spreads with the ES kernel (float2 atomic adds into the nf-point line),
 // transforms the line with the library's Stockham FFT and applies
-// (-1)^m' exp(ik x2^2/(2 z0)) / psi_hat(2 pi m'/nf) and the global factor.
+// (-1)^m' exp(ik x2^2/(2 z0)) / psi_hat(2 pi m'/nf) and the global factor:
+// one kernel of one block up to kLineOneBlock samples, with a spread kernel
+// before it above.  Such a line is all latency: as a memset and three kernels
+// 1024 samples took 6.7 us of GPU time in 21.
+#include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
 
 #include "asfd_impl.cuh"
+#include "fft.cuh"
 #include "sample.cuh"
 
 struct asfd_line_plan_s {
@@ -33,7 +39,9 @@ struct asfd_line_plan_s {
     float2* e = nullptr;      // [n] per-sample prefactor (with the weight)
     int* bi = nullptr;        // [n] integer part of g + nf/2 (mod nf)
     float* bf = nullptr;      // [n] fraction
-    float2* grid = nullptr;   // [nf]
+    float2* grid = nullptr;   // [nf], zero between calls
+    bool clean = false;       // the grid is zero
+    const float2* tw = nullptr;  // twiddles of nf points (a process-wide table)
     float2* c = nullptr;      // [m2] destination table
     double* quad = nullptr;
     unsigned* status = nullptr;
@@ -94,37 +102,100 @@ __global__ void line_dest_kernel(float2* __restrict__ C, int m2, double p2, doub
     C[k] = make_float2((float)(a * cs), (float)(a * sn));
 }
 
-template <int W>
-__global__ void __launch_bounds__(256) line_spread_kernel(const float2* __restrict__ u1,
-                                                          const float2* __restrict__ e,
-                                                          const int* __restrict__ bi,
-                                                          const float* __restrict__ bf, int n,
-                                                          int nf, float half_w, float two_over_w,
-                                                          float beta_log2e, float2* __restrict__ grid)
+struct LineArgs {
+    const float2* u1;
+    const float2* e;
+    const int* bi;
+    const float* bf;
+    int n, nf, w;
+    float half_w, two_over_w, beta_log2e;
+    float2* grid;
+    const float2* C;
+    int m2;
+    float2* u2;
+    const float2* tw;
+};
+
+constexpr int kLineOneBlock = 8192;  // samples that the transform's own block spreads
+
+// Adds sample j's taps to the line (periodic).
+__device__ __forceinline__ void line_spread_sample(const LineArgs& a, int j)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const float2 u = __ldg(&u1[j]), ej = __ldg(&e[j]);
+    const float2 u = __ldg(&a.u1[j]), ej = __ldg(&a.e[j]);
     const float2 c = make_float2(u.x * ej.x - u.y * ej.y, u.x * ej.y + u.y * ej.x);
-    const float f = __ldg(&bf[j]) - half_w;
+    const float f = __ldg(&a.bf[j]) - a.half_w;
     const float cf = ceilf(f);
-    const int l0 = __ldg(&bi[j]) + (int)cf;
+    const int l0 = __ldg(&a.bi[j]) + (int)cf;
     const float dx = cf - f;
-    const int mask = nf - 1;
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-        const float wv = es_weight_fast(dx + (float)i - half_w, two_over_w, beta_log2e);
-        atomicAdd(&grid[(l0 + i) & mask], make_float2(c.x * wv, c.y * wv));
+    const int mask = a.nf - 1;
+#pragma unroll 4
+    for (int i = 0; i < a.w; ++i) {
+        const float wv = es_weight_fast(dx + (float)i - a.half_w, a.two_over_w, a.beta_log2e);
+        atomicAdd(&a.grid[(l0 + i) & mask], make_float2(c.x * wv, c.y * wv));
     }
 }
 
-__global__ void line_finish_kernel(const float2* __restrict__ grid, const float2* __restrict__ C,
-                                   int m2, int nf, float2* __restrict__ u2)
+__global__ void __launch_bounds__(256) line_spread_kernel(LineArgs a)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= m2) return;
-    const float2 b = grid[(k - m2 / 2) & (nf - 1)], c = C[k];
-    u2[k] = make_float2(b.x * c.x - b.y * c.y, b.x * c.y + b.y * c.x);
+    chain_next();
+    chain_wait();
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < a.n) line_spread_sample(a, j);
+}
+
+// The block spreads the samples (SPREAD), and its first L/16 threads transform
+// the line, leave it zero for the next call and write the destination.
+template <int L, bool SPREAD>
+__global__ void __launch_bounds__(1024) line_transform_kernel(LineArgs a)
+{
+    extern __shared__ float2 sm[];
+    chain_next();
+    chain_wait();
+    const int t = threadIdx.x;
+    if constexpr (SPREAD) {
+        for (int j = t; j < a.n; j += blockDim.x) line_spread_sample(a, j);
+        __threadfence();  // the sums are in L2, where the loads below read
+        __syncthreads();
+    }
+    if (t >= L / 16) return;
+    auto ld = [&](int i) -> float2 {
+        const float2 v = __ldcg(&a.grid[i]);
+        a.grid[i] = make_float2(0.f, 0.f);
+        return v;
+    };
+    const int half = a.m2 / 2;
+    auto st = [&](int i, float2 v) {
+        int k;
+        if (i < half) k = i + half;
+        else if (i >= L - half) k = i - (L - half);
+        else return;
+        a.u2[k] = cmul(v, __ldg(&a.C[k]));
+    };
+    fft_line<L, -1>(t, sm, a.tw, ld, st);
+}
+
+template <int L>
+cudaError_t line_launch(const LineArgs& a, bool spread, cudaStream_t st)
+{
+    constexpr size_t smem = sizeof(float2) * FftShape<L>::SMEM;
+    if constexpr (smem > 48 * 1024) {
+        static std::once_flag once;
+        static cudaError_t attr = cudaSuccess;
+        std::call_once(once, [] {
+            attr = cudaFuncSetAttribute(line_transform_kernel<L, true>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (attr == cudaSuccess)
+                attr = cudaFuncSetAttribute(line_transform_kernel<L, false>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        });
+        if (attr != cudaSuccess) return attr;
+    }
+    if (!spread)
+        return launch_chained(line_transform_kernel<L, false>, dim3(1), L / 16 < 32 ? 32 : L / 16, smem, st,
+                              a);
+    int threads = std::min(1024, (a.n + 31) / 32 * 32);
+    threads = std::max(threads, std::max(32, L / 16));
+    return launch_chained(line_transform_kernel<L, true>, dim3(1), (unsigned)threads, smem, st, a);
 }
 
 void line_free(asfd_line_plan_s* P)
@@ -192,6 +263,9 @@ asfd_status asfd_line_plan_create(asfd_line_plan* out, const asfd_line_params* p
         ASFD_CUDA(cudaMemcpyAsync(P->quad, h.data(), sizeof(double) * h.size(),
                                   cudaMemcpyHostToDevice, st));
         ASFD_CUDA(cudaMemsetAsync(P->status, 0, sizeof(unsigned), st));
+        ASFD_CUDA(cudaMemsetAsync(P->grid, 0, sizeof(float2) * nf, st));
+        const asfd_status ts = fft_line_twiddles(nf, &P->tw, st);
+        if (ts != ASFD_OK) return ts;
         const double sz = std::sqrt(1.0 - p->incidence_s * p->incidence_s);
         line_prep_kernel<<<(n + 255) / 256, 256, 0, st>>>(x1_dev, d1_dev, w_dev, n, p->lambda,
                                                            p->z0, p->p2, nf, p->incidence_s, sz,
@@ -204,6 +278,7 @@ asfd_status asfd_line_plan_create(asfd_line_plan* out, const asfd_line_params* p
         ASFD_CUDA(cudaStreamSynchronize(st));
         if (bad)
             return fail(ASFD_ERR_ARG, "x1, d1 and w must be finite and every d1 below z0");
+        P->clean = true;
         return ASFD_OK;
     }();
     if (s != ASFD_OK) {
@@ -227,30 +302,37 @@ asfd_status asfd_line_execute(asfd_line_plan P, const float* u1_dev, float* u2_d
         if (e != cudaSuccess) return cuda_fail(e, "cudaSetDevice");
     }
     asfd_status s = [&]() -> asfd_status {
-        ASFD_CUDA(cudaMemsetAsync(P->grid, 0, sizeof(float2) * P->nf, st));
-        const float half_w = 0.5f * (float)P->w;
-        const float two_over_w = (float)(2.0 / P->w);
-        const float bl2e = (float)(P->beta * 1.4426950408889634074);
-        const unsigned blocks = (unsigned)((P->n + 255) / 256);
-        const float2* u1 = reinterpret_cast<const float2*>(u1_dev);
-        switch (P->w) {
-#define ASFD_LW(W)                                                                         \
-    case W:                                                                                \
-        line_spread_kernel<W><<<blocks, 256, 0, st>>>(u1, P->e, P->bi, P->bf, P->n, P->nf, \
-                                                      half_w, two_over_w, bl2e, P->grid);  \
-        break;
-            ASFD_LW(2) ASFD_LW(3) ASFD_LW(4) ASFD_LW(5) ASFD_LW(6) ASFD_LW(7) ASFD_LW(8)
-            ASFD_LW(9) ASFD_LW(10) ASFD_LW(11) ASFD_LW(12) ASFD_LW(13) ASFD_LW(14) ASFD_LW(15)
-            ASFD_LW(16)
-#undef ASFD_LW
-            default: return fail(ASFD_ERR_UNSUPPORTED, "kernel width outside 2..16");
+        LineArgs a;
+        a.u1 = reinterpret_cast<const float2*>(u1_dev);
+        a.e = P->e;
+        a.bi = P->bi;
+        a.bf = P->bf;
+        a.n = P->n;
+        a.nf = P->nf;
+        a.w = P->w;
+        a.half_w = 0.5f * (float)P->w;
+        a.two_over_w = (float)(2.0 / P->w);
+        a.beta_log2e = (float)(P->beta * 1.4426950408889634074);
+        a.grid = P->grid;
+        a.C = P->c;
+        a.m2 = P->prm.m2;
+        a.u2 = reinterpret_cast<float2*>(u2_dev);
+        a.tw = P->tw;
+        // (the transform leaves the line zero; not so after a failed launch)
+        if (!P->clean) ASFD_CUDA(cudaMemsetAsync(P->grid, 0, sizeof(float2) * P->nf, st));
+        P->clean = false;
+        const bool one = P->n <= kLineOneBlock;
+        if (!one) ASFD_CUDA(launch_chained(line_spread_kernel, dim3((P->n + 255) / 256), 256, 0, st, a));
+        cudaError_t e = cudaErrorInvalidValue;
+        switch (P->nf) {
+#define ASFD_LT(L) case L: e = line_launch<L>(a, one, st); break;
+            ASFD_LT(64) ASFD_LT(128) ASFD_LT(256) ASFD_LT(512) ASFD_LT(1024) ASFD_LT(2048) ASFD_LT(4096)
+            ASFD_LT(8192) ASFD_LT(16384)
+#undef ASFD_LT
+            default: break;
         }
-        ASFD_CUDA(cudaGetLastError());
-        asfd_status f = launch_fft_lines(P->nf, 1, -1, P->grid, P->grid, st);
-        if (f != ASFD_OK) return f;
-        line_finish_kernel<<<(P->prm.m2 + 255) / 256, 256, 0, st>>>(
-            P->grid, P->c, P->prm.m2, P->nf, reinterpret_cast<float2*>(u2_dev));
-        ASFD_CUDA(cudaGetLastError());
+        if (e != cudaSuccess) return cuda_fail(e, "line_transform_kernel launch");
+        P->clean = true;
         return ASFD_OK;
     }();
     if (dev != P->device && dev >= 0) cudaSetDevice(dev);
