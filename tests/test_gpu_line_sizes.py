@@ -1,5 +1,5 @@
-"""The 1D transform where its launch changes: one block up to 8192 samples, a
-spread kernel of its own above; lines of 64 to 16384 fine cells (4 to 1024
+"""The 1D transform where its launch changes: one block up to 1024 samples and
+two per fine cell, a spread kernel of its own above; lines of 64 to 16384 fine cells (4 to 1024
 transform threads); and a line that holds nothing over from call to call.
 Tolerance as in test_gpu_line: the width's truncation or 5e-6.
 """
@@ -17,8 +17,8 @@ from paper_1203_3583_gb300.fresnel import LinePlan  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,m2,width", [(1, 32, 7), (33, 64, 16), (1025, 256, 2), (8192, 512, 7),
-                                        (8193, 512, 7), (20000, 4096, 9), (700, 8192, 6)])
+@pytest.mark.parametrize("n,m2,width", [(1, 32, 7), (33, 64, 16), (128, 32, 7), (129, 32, 5),
+                                        (1024, 512, 7), (1025, 512, 2), (20000, 4096, 9), (700, 8192, 6)])
 def test_line_sizes(n, m2, width):
     rng = np.random.default_rng(n + m2)
     x1 = rng.uniform(-1.5e-3, 1.5e-3, n)
