@@ -92,6 +92,7 @@ struct asfd_plan_s {
     double* bux = nullptr;          // unreduced alpha x~ + nf/2 per axis (plan only)
     double* buy = nullptr;
     float* q = nullptr;             // [n1y][n1x]  d1 / (z0 - d1)
+    float* q_next = nullptr;        // [n1y][n1x]  the same of a height map being checked
     float2* cx = nullptr;           // [m2x] destination chirp * (-1)^m' / psi_hat
     float2* cy = nullptr;           // [m2y] same, times the global factor
     float2* twx = nullptr;          // [nfx] e^{-2 pi i k/nfx}
@@ -112,7 +113,6 @@ struct asfd_plan_s {
     int4* tile_rect = nullptr;      // per kTileX x kColTileY tile of the band
     double2* col_range = nullptr;   // per source column: [min, max] of the x storage coordinate
     double2* row_range = nullptr;   // per source row:    [min, max] of the y storage coordinate
-    float2* step_min = nullptr;     // per block of min_step_kernel: min spacing along x and y
     bool colored = false;
     bool windowed = false;          // register-window kernel applies (w <= kMaxWindowWidth)
     bool dense = false;             // dense map: register windows flushed with global atomics
@@ -149,6 +149,7 @@ struct asfd_plan_s {
                                     // (left so by the forward row pass, which
                                     // clears each cell it reads)
     unsigned* status = nullptr;     // device status word
+    float* stat = nullptr;          // a height map's statistics, per block
     // learned kernel (kind == ASFD_KERNEL_LEARNED)
     bool learned = false;
     float* ltab = nullptr;          // [source tiles][kLearnTableSize] current tables

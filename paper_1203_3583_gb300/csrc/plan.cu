@@ -90,42 +90,113 @@ __global__ void dest_table_kernel(float2* C, int m, double p2, double lam_z0, in
     C[k] = make_float2((float)re, (float)im);
 }
 
-// Checks d1 (finite, below z0) and reduces max |d1|/z0 (in FP32: a bound
-// checked against 0.1).
-// (grid-stride; the block's maximum goes out with one atomic: per-warp
-// atomics on the one word serialise)
-__global__ void __launch_bounds__(256) d1_check_kernel(const double* d1, size_t n, double z0,
-                                                       float inv_z0, unsigned* status,
-                                                       unsigned* maxeps_bits)
-{
-    float e = 0.f;
-    bool bad = false;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const double h = d1[i];
-        if (!isfinite(h) || !(h < z0)) bad = true;
-        else e = fmaxf(e, (float)fabs(h) * inv_z0);
-    }
-    if (bad) atomicOr(status, kStatusBadD1);
-    for (int o = 16; o > 0; o >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, o));
-    __shared__ float red[8];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x / 32] = e;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < 8; ++w) e = fmaxf(e, red[w]);
-        atomicMax(maxeps_bits, __float_as_uint(e));
-    }
-}
+// What a height map decides about its plan, as maxima: whether a sample is bad
+// (1: not finite or not below z0), |d1|/z0, the extremes of the unreduced
+// storage coordinates (x, -x, y, -y) and the negated least spacing of
+// neighbouring samples along x and y.  One set per block of d1_stats_kernel;
+// the host takes the maxima (608 x 32 bytes: atomics on one set serialise).
+enum { kStatBad = 0, kStatEps, kStatXMax, kStatXMin, kStatYMax, kStatYMin, kStatStepX, kStatStepY, kStatWords };
 
-// q = d1 / (z0 - d1), stored FP32: z0 - d1 formed in FP64 (no cancellation
-// error), both operands rounded to FP32 and divided there (within 1.5 FP32
-// ulp of the FP64 quotient; an FP64 division per sample is slow on this GPU).
-__global__ void d1_q_kernel(const double* d1, float* q, size_t n, double z0)
+constexpr int kStatBlocks = 608;    // blocks of d1_stats_kernel, at most
+constexpr int kStatCols = 8 * 31;   // columns of a block
+constexpr int kStatRows = 64;       // rows whose coordinates it stages at a time
+
+// One pass over a height map: q = d1 / (z0 - d1) (z0 - d1 formed in FP64, both
+// operands rounded to FP32 and divided there, within 1.5 FP32 ulp of the FP64
+// quotient; an FP64 division per sample is slow on this GPU) and everything
+// above.  A thread takes a column over a chunk of rows: its x extremes are
+// those of q, mapped, as the coordinate is monotone in q; the spacing takes the
+// FP64 difference of neighbouring base coordinates and FP32 q terms (~1 cell,
+// good to ~1e-6 cells; the binning adds a one-cell margin).  q goes to a buffer
+// of its own, so that a rejected map changes nothing.  (Four kernels with three
+// waits for their results, and loops over 4096 source tiles on the host, left
+// the GPU idle for 0.2 of a 0.41 ms optimisation step at 1024^2.)
+__global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* q,
+                                                       const AxisEntry* ax, const AxisEntry* ay,
+                                                       const double* bux, const double* buy,
+                                                       int n1x, int n1y, double z0, float inv_z0,
+                                                       unsigned* status, float* stat)
 {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double h = d1[i];
-    q[i] = __fdiv_rn((float)h, (float)(z0 - h));
+    // (a warp's last lane only forms the q that its neighbour compares with)
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int nx = (blockIdx.x * (kStatCols / 31) + warp) * 31 + lane;
+    const int chunk = (n1y + gridDim.y - 1) / gridDim.y;
+    const int r0 = blockIdx.y * chunk, r1 = min(n1y, r0 + chunk);
+    const bool in = nx < n1x, on = in && lane < 31, hasx = on && nx + 1 < n1x;
+    bool bad = false;
+    float eps = 0.f;
+    auto load = [&](int col, int row) -> float {
+        const double h = d1[(size_t)row * n1x + col];
+        const double d = z0 - h;
+        // (finite and below z0 by the bits: FP64 comparisons and conversions are
+        // slow here)
+        if ((__double2hiint(h) & 0x7ff00000) == 0x7ff00000 || __double_as_longlong(d) <= 0) {
+            bad = true;
+            return 0.f;
+        }
+        const float hf = (float)h;
+        eps = fmaxf(eps, fabsf(hf) * inv_z0);
+        return __fdiv_rn(hf, (float)d);
+    };
+    const float sx0 = on ? ax[nx].s : 0.f, sx1 = hasx ? ax[nx + 1].s : 0.f;
+    const float dbx = hasx ? (float)(bux[nx + 1] - bux[nx]) : 0.f;
+    float qlo = 3e38f, qhi = -3e38f, ylo = 3e38f, yhi = -3e38f, mx = 3e38f, my = 3e38f;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = 0;
+    float qn = in && r0 < r1 ? load(nx, r0) : 0.f;
+    // the rows' base coordinates, their FP64 differences and slopes in FP32, a
+    // batch of rows at a time
+    __shared__ float4 rows[kStatRows];
+    for (int b0 = r0; b0 < r1; b0 += kStatRows) {
+        const int b1 = min(r1, b0 + kStatRows);
+        __syncthreads();
+        if (b0 + (int)threadIdx.x < b1) {
+            const int ny = b0 + threadIdx.x;
+            const bool hasy = ny + 1 < n1y;
+            rows[threadIdx.x] = make_float4((float)buy[ny], hasy ? (float)(buy[ny + 1] - buy[ny]) : 0.f,
+                                            ay[ny].s, hasy ? ay[ny + 1].s : 0.f);
+        }
+        __syncthreads();
+        for (int ny = b0; ny < b1; ++ny) {
+            const float qq = qn;
+            const float qx = __shfl_down_sync(0xffffffffu, qq, 1);
+            if (in && ny + 1 < n1y) qn = load(nx, ny + 1);
+            if (on) {
+                q[(size_t)ny * n1x + nx] = qq;
+                qlo = fminf(qlo, qq);
+                qhi = fmaxf(qhi, qq);
+                const float4 r = rows[ny - b0];
+                const float uy = r.x + r.z * qq;
+                ylo = fminf(ylo, uy);
+                yhi = fmaxf(yhi, uy);
+                if (hasx) mx = fminf(mx, dbx + (sx1 * qx - sx0 * qq));
+                if (ny + 1 < n1y) my = fminf(my, r.y + (r.w * qn - r.z * qq));
+            }
+        }
+    }
+    float v[kStatWords];
+    v[kStatBad] = bad ? 1.f : 0.f;
+    v[kStatEps] = eps;
+    const float bx = on ? (float)bux[nx] : 0.f;
+    const bool any = on && r0 < r1;
+    v[kStatXMax] = any ? fmaxf(bx + sx0 * qlo, bx + sx0 * qhi) : -3e38f;
+    v[kStatXMin] = any ? -fminf(bx + sx0 * qlo, bx + sx0 * qhi) : -3e38f;
+    v[kStatYMax] = yhi;
+    v[kStatYMin] = -ylo;
+    v[kStatStepX] = -mx;
+    v[kStatStepY] = -my;
+    __shared__ float red[kStatWords][8];
+#pragma unroll
+    for (int k = 0; k < kStatWords; ++k) {
+        for (int o = 16; o > 0; o >>= 1) v[k] = fmaxf(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+        if (lane == 0) red[k][warp] = v[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < kStatWords) {
+        const int k = threadIdx.x;
+        float m = red[k][0];
+        for (int w = 1; w < 8; ++w) m = fmaxf(m, red[k][w]);
+        stat[(size_t)(blockIdx.y * gridDim.x + blockIdx.x) * kStatWords + k] = m;
+    }
 }
 
 // Per source tile: bounds of the unreduced storage coordinate alpha x~ (1+q) + nf/2,
@@ -240,53 +311,6 @@ __global__ void row_range_kernel(const float* q, const AxisEntry* ay, const doub
     }
 }
 
-// Minimum spacing on the fine grid of neighbouring samples: along x within a
-// row and along y within a column (one pair of minima per block).  A thread
-// takes one column over a chunk of rows: the FP64 difference of the
-// neighbouring columns' base coordinates is formed once, the q terms in
-// FP32 (the spacing is ~1 cell, so this is good to ~1e-6 cells).
-__global__ void min_step_kernel(const float* q, const AxisEntry* ax, const AxisEntry* ay,
-                                const double* bux, const double* buy, int n1x, int n1y,
-                                float2* out)
-{
-    const int nx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int chunk = (n1y + gridDim.y - 1) / gridDim.y;
-    const int r0 = blockIdx.y * chunk, r1 = min(n1y, r0 + chunk);
-    float mx = 3.0e38f, my = 3.0e38f;
-    if (nx < n1x) {
-        const bool hasx = nx + 1 < n1x;
-        const float sx0 = ax[nx].s, sx1 = hasx ? ax[nx + 1].s : 0.f;
-        const float dbx = hasx ? (float)(bux[nx + 1] - bux[nx]) : 0.f;
-        for (int ny = r0; ny < r1; ++ny) {
-            const size_t i = (size_t)ny * n1x + nx;
-            const float qq = q[i];
-            if (hasx) mx = fminf(mx, dbx + (sx1 * q[i + 1] - sx0 * qq));
-            if (ny + 1 < n1y) {
-                const float dby = (float)(buy[ny + 1] - buy[ny]);
-                my = fminf(my, dby + (ay[ny + 1].s * q[i + n1x] - ay[ny].s * qq));
-            }
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        mx = fminf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        my = fminf(my, __shfl_xor_sync(0xffffffffu, my, o));
-    }
-    __shared__ float red[2][32];
-    if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x / 32] = mx;
-        red[1][threadIdx.x / 32] = my;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x / 32); ++w) {
-            mx = fminf(mx, red[0][w]);
-            my = fminf(my, red[1][w]);
-        }
-        out[blockIdx.y * gridDim.x + blockIdx.x] = make_float2(mx, my);
-    }
-}
-
-constexpr int kStepBlocks = 1024;
 
 // Gauss-Legendre nodes and weights on [-1, 1] (Newton iteration on P_n).
 void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& wt)
@@ -379,7 +403,7 @@ bool pow2_in(int n, int lo, int hi) { return n >= lo && n <= hi && (n & (n - 1))
 
 }  // namespace
 
-asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, cudaStream_t st);
+asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double msy, cudaStream_t st);
 
 asfd_status plan_alloc_buffer(asfd_plan_s* P, void** p, size_t bytes) { return alloc(P, p, bytes); }
 
@@ -465,6 +489,7 @@ asfd_status plan_alloc(asfd_plan_s* P)
     A(bux, p.n1x);
     A(buy, p.n1y);
     A(q, nsrc);
+    A(q_next, nsrc);
     A(cx, p.m2x);
     A(cy, p.m2y);
     A(twx, P->nfx);
@@ -474,8 +499,8 @@ asfd_status plan_alloc(asfd_plan_s* P)
     A(tile_rect, (size_t)P->ntx * P->nty * (kTileY / kColTileY));
     A(col_range, p.n1x);
     A(row_range, p.n1y);
-    A(step_min, kStepBlocks);
-    A(status, 2);
+    A(status, 1);
+    A(stat, kStatBlocks * kStatWords);
 #undef A
     return ASFD_OK;
 }
@@ -633,59 +658,55 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
     const size_t nsrc = (size_t)p.n1x * p.n1y;
     // the band may move: its new cells were never cleared
     P->band_clean = false;
-    // 1. validate d1 without touching the plan's tables
-    ASFD_CUDA(cudaMemsetAsync(P->status, 0, 2 * sizeof(unsigned), st));
-    d1_check_kernel<<<(unsigned)std::min<size_t>((nsrc + 255) / 256, 1216), 256, 0, st>>>(
-        d1, nsrc, p.z0, (float)(1.0 / p.z0), P->status, P->status + 1);
+    // 1. one pass over d1: checks, q (beside the plan's), extremes and spacings
+    static_assert((65536 + kStatCols - 1) / kStatCols <= kStatBlocks, "n1x <= 65536 fits one row of blocks");
+    const int sgx = (p.n1x + kStatCols - 1) / kStatCols;
+    const int sgy = std::max(1, std::min(kStatBlocks / sgx, p.n1y));
+    d1_stats_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(d1, P->q_next, P->ax, P->ay, P->bux, P->buy, p.n1x,
+                                                    p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
     ASFD_CUDA(cudaGetLastError());
-    unsigned hs[2] = {0, 0};
-    ASFD_CUDA(cudaMemcpyAsync(hs, P->status, sizeof(hs), cudaMemcpyDeviceToHost, st));
+    std::vector<float> stats((size_t)sgx * sgy * kStatWords);
+    ASFD_CUDA(cudaMemcpyAsync(stats.data(), P->stat, sizeof(float) * stats.size(), cudaMemcpyDeviceToHost,
+                              st));
     ASFD_CUDA(cudaStreamSynchronize(st));
-    if (hs[0] & kStatusBadD1) return fail(ASFD_ERR_ARG, "d1 has a non-finite value or d1 >= z0");
-    float me;
-    std::memcpy(&me, &hs[1], sizeof(float));
+    const auto value = [&](int k) {
+        float m = stats[k];
+        for (size_t b = k + kStatWords; b < stats.size(); b += kStatWords) m = std::max(m, stats[b]);
+        return m;
+    };
+    if (value(kStatBad) != 0.f) {
+        cudaMemsetAsync(P->status, (int)kStatusBadD1, 1, st);  // (the word's low byte)
+        return fail(ASFD_ERR_ARG, "d1 has a non-finite value or d1 >= z0");
+    }
+    const float me = value(kStatEps);
     if (me > 0.1f)
         return fail(ASFD_ERR_UNSUPPORTED, "max |d1|/z0 = " + std::to_string(me) +
                                               " exceeds the supported 0.1");
+    // (copied, not swapped: captured launches hold the plan's pointer)
+    ASFD_CUDA(cudaMemcpyAsync(P->q, P->q_next, sizeof(float) * nsrc, cudaMemcpyDeviceToDevice, st));
 
-    // 2. per-sample correction and per-source-tile footprint bounds
-    d1_q_kernel<<<(unsigned)((nsrc + 255) / 256), 256, 0, st>>>(d1, P->q, nsrc, p.z0);
-    const int nst = P->nstx * P->nsty;
-    src_bbox_kernel<<<nst, kSrcTile * kSrcTile, 0, st>>>(P->q, P->ax, P->ay, P->bux, P->buy, p.n1x,
-                                                         p.n1y, P->nstx, P->src_bbox);
-    ASFD_CUDA(cudaGetLastError());
-    std::vector<float> bb(4 * (size_t)nst);
-    ASFD_CUDA(cudaMemcpyAsync(bb.data(), P->src_bbox, sizeof(float) * 4 * nst,
-                              cudaMemcpyDeviceToHost, st));
-    ASFD_CUDA(cudaStreamSynchronize(st));
-
-    // 3. the band (fine-grid tiles that footprints reach) and the wrap flags,
-    //    from each source tile's footprint bounds
+    // 2. the band (fine-grid tiles that footprints reach) and the wrap flags
     const double hw = 0.5 * P->w + 1.0;  // half width plus a one-cell safety margin
     struct Range { int x0, x1, y0, y1; };
-    std::vector<Range> rg(nst);
-    bool wrapx = false, wrapy = false;
-    int bx0 = P->ntx, bx1 = -1, by0 = P->nty, by1 = -1;
-    for (int t = 0; t < nst; ++t) {
-        const float* b = &bb[4 * (size_t)t];
+    const auto tiles_of = [&](float xlo, float xhi, float ylo, float yhi, bool* wx, bool* wy) {
         Range r;
-        r.x0 = (int)std::floor((b[0] - hw) / kTileX);
-        r.x1 = (int)std::floor((b[1] + hw) / kTileX);
-        r.y0 = (int)std::floor((b[2] - hw) / kTileY);
-        r.y1 = (int)std::floor((b[3] + hw) / kTileY);
+        r.x0 = (int)std::floor((xlo - hw) / kTileX);
+        r.x1 = (int)std::floor((xhi + hw) / kTileX);
+        r.y0 = (int)std::floor((ylo - hw) / kTileY);
+        r.y1 = (int)std::floor((yhi + hw) / kTileY);
         // a footprint reaching outside [0, nf) wraps around the periodic grid
-        if (b[0] - hw < 0.0 || b[1] + hw > (double)P->nfx) wrapx = true;
-        if (b[2] - hw < 0.0 || b[3] + hw > (double)P->nfy) wrapy = true;
+        if (xlo - hw < 0.0 || xhi + hw > (double)P->nfx) *wx = true;
+        if (ylo - hw < 0.0 || yhi + hw > (double)P->nfy) *wy = true;
         if (r.x1 - r.x0 + 1 >= P->ntx) { r.x0 = 0; r.x1 = P->ntx - 1; }
         if (r.y1 - r.y0 + 1 >= P->nty) { r.y0 = 0; r.y1 = P->nty - 1; }
-        if (r.x0 < 0 || r.x1 >= P->ntx) wrapx = true;
-        if (r.y0 < 0 || r.y1 >= P->nty) wrapy = true;
-        bx0 = std::min(bx0, r.x0);
-        bx1 = std::max(bx1, r.x1);
-        by0 = std::min(by0, r.y0);
-        by1 = std::max(by1, r.y1);
-        rg[t] = r;
-    }
+        if (r.x0 < 0 || r.x1 >= P->ntx) *wx = true;
+        if (r.y0 < 0 || r.y1 >= P->nty) *wy = true;
+        return r;
+    };
+    bool wrapx = false, wrapy = false;
+    const Range all = tiles_of(-value(kStatXMin), value(kStatXMax), -value(kStatYMin), value(kStatYMax),
+                               &wrapx, &wrapy);
+    int bx0 = all.x0, bx1 = all.x1, by0 = all.y0, by1 = all.y1;
     if (wrapx) { bx0 = 0; bx1 = P->ntx - 1; }
     if (wrapy) { by0 = 0; by1 = P->nty - 1; }
     P->band_tx0 = bx0;
@@ -694,12 +715,26 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
     P->band_ty1 = by1 + 1;
     P->max_abs_eps = me;
     P->wraps = wrapx || wrapy;
-    asfd_status cs = plan_build_colored(P, wrapx || wrapy, st);
+    asfd_status cs = plan_build_colored(P, wrapx || wrapy, -value(kStatStepX), -value(kStatStepY), st);
     if (cs != ASFD_OK) return cs;
     P->tile_pairs = 0;
     if (!P->colored && !P->dense) {
         // the shared-memory-atomic spread walks, per band tile, the source
         // tiles whose footprints reach it: a CSR list built here
+        const int nst = P->nstx * P->nsty;
+        src_bbox_kernel<<<nst, kSrcTile * kSrcTile, 0, st>>>(P->q, P->ax, P->ay, P->bux, P->buy, p.n1x,
+                                                             p.n1y, P->nstx, P->src_bbox);
+        ASFD_CUDA(cudaGetLastError());
+        std::vector<float> bb(4 * (size_t)nst);
+        ASFD_CUDA(cudaMemcpyAsync(bb.data(), P->src_bbox, sizeof(float) * 4 * nst,
+                                  cudaMemcpyDeviceToHost, st));
+        ASFD_CUDA(cudaStreamSynchronize(st));
+        std::vector<Range> rg(nst);
+        bool wx = false, wy = false;
+        for (int t = 0; t < nst; ++t) {
+            const float* b = &bb[4 * (size_t)t];
+            rg[t] = tiles_of(b[0], b[1], b[2], b[3], &wx, &wy);
+        }
         const int bntx = bx1 - bx0 + 1, bnty = by1 - by0 + 1;
         const int ntiles = bntx * bnty;
         std::vector<int> off(ntiles + 1, 0);
@@ -754,7 +789,7 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
 // columns) at least h * min_step_y - row_spread_y, where row_spread_y bounds
 // the variation of the y coordinate along a row.  Both distances must reach
 // the kernel width (plus a margin for FP32 rounding of the coordinates).
-asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, cudaStream_t st)
+asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double msy, cudaStream_t st)
 {
     const asfd_params& p = P->prm;
     P->colored = false;
@@ -763,24 +798,6 @@ asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, cudaStream_t st)
     P->itemtile = false;
     P->blk = false;
     P->fold = false;
-    // a column per thread (blocks of 256 columns), rows in chunks, at most
-    // kStepBlocks blocks
-    static_assert((65536 + 255) / 256 <= kStepBlocks, "n1x <= 65536 fits one row of blocks");
-    const int sgx = (p.n1x + 255) / 256;
-    const int sgy = std::max(1, std::min(kStepBlocks / sgx, p.n1y));
-    min_step_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(P->q, P->ax, P->ay, P->bux, P->buy, p.n1x,
-                                                    p.n1y, P->step_min);
-    ASFD_CUDA(cudaGetLastError());
-    const int nsb = sgx * sgy;
-    std::vector<float> sm(2 * (size_t)nsb);
-    ASFD_CUDA(cudaMemcpyAsync(sm.data(), P->step_min, sizeof(float) * sm.size(),
-                              cudaMemcpyDeviceToHost, st));
-    ASFD_CUDA(cudaStreamSynchronize(st));
-    double msx = 3e38, msy = 3e38;
-    for (int b = 0; b < nsb; ++b) {
-        msx = std::min(msx, (double)sm[2 * b]);
-        msy = std::min(msy, (double)sm[2 * b + 1]);
-    }
     if (p.n1x < 2) msx = 1e30;
     if (p.n1y < 2) msy = 1e30;
     P->min_step_x = msx;
