@@ -20,9 +20,10 @@ namespace asfd {
 
 namespace {
 
-// (4096-point rows: at most 64 registers, four 256-thread blocks per SM)
+// (4096-point rows: at most 64 registers, four 256-thread blocks per SM; 8192:
+// 128 registers, two)
 template <int L>
-__global__ void __launch_bounds__(RowCfg<L>::THREADS, L == 4096 ? 4 : 1)
+__global__ void __launch_bounds__(RowCfg<L>::THREADS, L == 4096 ? 4 : L == 8192 ? 2 : 1)
 fft_rows_kernel(RowArgs a)
 {
     extern __shared__ float2 sm[];
@@ -59,26 +60,26 @@ fft_cols_adj_kernel(const float2* __restrict__ g, int m2x, int m2y, const float2
     const int colc = active ? col : 0;
     const float2 fx = __ldg(&cx[colc]);
     const int half = m2y / 2;
+    auto bin = [&](int i) { return i < half ? i + half : i - (L - half); };
+    auto kept = [&](int i) { return active && (i < half || i >= L - half); };
     auto ld = [&](int i) -> float2 {
-        int k;
-        if (i < half) k = i + half;
-        else if (i >= L - half) k = i - (L - half);
-        else return make_float2(0.f, 0.f);
-        if (!active) return make_float2(0.f, 0.f);
-        // conj(fx * cy[k]) * g
-        return cmulc(cmulc(__ldg(&g[(size_t)k * m2x + colc]), fx), __ldg(&cy[k]));
+        return kept(i) ? __ldg(&g[(size_t)bin(i) * m2x + colc]) : make_float2(0.f, 0.f);
+    };
+    auto scale = [&](int i, float2 v) -> float2 {  // conj(fx * cy[k]) * g
+        const float2 f = kept(i) ? __ldg(&cy[bin(i)]) : make_float2(0.f, 0.f);
+        return cmulc(cmulc(v, fx), f);
     };
     auto st = [&](int i, float2 v) {
         const int rr = i - row0;
         if (active && rr >= 0 && rr < nrows) rows[(size_t)rr * m2x + colc] = v;
     };
-    fft_line<L, 1>(t, sm + c * C::LS, tw, ld, st);
+    fft_line<L, 1>(t, sm + c * C::LS, tw, ld, st, scale);
 }
 
 // Adjoint row pass: band row r of rows[][] placed at the kept bins, FFT with
 // e^{+i} along x, band columns [col_lo, col_hi) stored to the fine grid.
 template <int L>
-__global__ void __launch_bounds__(RowCfg<L>::THREADS)
+__global__ void __launch_bounds__(RowCfg<L>::THREADS, L == 4096 ? 4 : 1)
 fft_rows_adj_kernel(const float2* __restrict__ rows, int nrows, int m2x, float2* __restrict__ grid,
                     int row0, int col_lo, int col_hi, const float2* __restrict__ tw)
 {
@@ -93,10 +94,8 @@ fft_rows_adj_kernel(const float2* __restrict__ rows, int nrows, int m2x, float2*
     float2* dst = grid + (size_t)(row0 + (active ? r : 0)) * L;
     const int half = m2x / 2;
     auto ld = [&](int i) -> float2 {
-        if (!active) return make_float2(0.f, 0.f);
-        if (i < half) return __ldg(&src[i + half]);
-        if (i >= L - half) return __ldg(&src[i - (L - half)]);
-        return make_float2(0.f, 0.f);
+        const bool kept = active && (i < half || i >= L - half);
+        return kept ? __ldg(&src[i < half ? i + half : i - (L - half)]) : make_float2(0.f, 0.f);
     };
     auto st = [&](int i, float2 v) {
         if (active && i >= col_lo && i < col_hi) dst[i] = v;

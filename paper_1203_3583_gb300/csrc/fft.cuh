@@ -2,7 +2,7 @@
 //
 // NUFFTs combine an interpolation with a uniform FFT (Sec. 2, after Eq. 9);
 // this is the uniform FFT.  Each line of length L is processed by L/16
-// threads holding 16 complex values in registers.  Passes are radix 16
+// threads holding 16 complex values in registers (8192 points: L/32 and 32).  Passes are radix 16
 // (one leading radix-2/4/8 pass when log2 L is not a multiple of 4), in the
 // self-sorting Stockham order: pass p with accumulated stride NS reads
 // x[j + r L/R], multiplies by W_{NS R}^{r (j mod NS)}, takes an R-point DFT in
@@ -95,6 +95,25 @@ __device__ __forceinline__ float2 rot16(float2 d, int j)
     return fma_f2(make_float2(d.x, d.x), make_float2(c, s), make_float2(-p.x, p.y));
 }
 
+// d * exp(S * 2 pi i j / 32), j known at compile time: odd j from the closed
+// forms cos(pi/16) = sqrt(2 + sqrt(2 + sqrt2))/2 and so on.
+__device__ __forceinline__ constexpr float cos32(int j)
+{
+    constexpr float A = 0.980785280403230449f, B = 0.831469612302545237f,
+                    C = 0.555570233019602225f, D = 0.195090322016128268f;
+    constexpr float t[16] = {A, B, C, D, -D, -C, -B, -A, -A, -B, -C, -D, D, C, B, A};
+    return t[(j >> 1) & 15];  // j odd: cos(2 pi j / 32)
+}
+
+template <int S>
+__device__ __forceinline__ float2 rot32(float2 d, int j)
+{
+    if (j % 2 == 0) return rot16<S>(d, j / 2);
+    const float c = cos32(j), s = S < 0 ? -cos32(j - 8) : cos32(j - 8);
+    const float2 p = mul_f2(make_float2(d.y, d.y), make_float2(s, c));
+    return fma_f2(make_float2(d.x, d.x), make_float2(c, s), make_float2(-p.x, p.y));
+}
+
 template <int R>
 __device__ __forceinline__ constexpr int bitrev_c(int i)
 {
@@ -103,7 +122,7 @@ __device__ __forceinline__ constexpr int bitrev_c(int i)
     return r;
 }
 
-// In-register R-point DFT (R = 2, 4, 8, 16), sign S: X_k = sum_r v_r e^{S 2 pi i r k/R}.
+// In-register R-point DFT (R = 2, 4, 8, 16, 32), sign S: X_k = sum_r v_r e^{S 2 pi i r k/R}.
 // Radix-2 decimation in frequency followed by a compile-time bit reversal.
 template <int R, int S>
 __device__ __forceinline__ void dft_reg(float2* v)
@@ -117,7 +136,7 @@ __device__ __forceinline__ void dft_reg(float2* v)
             for (int k = 0; k < half; ++k) {
                 const float2 a = v[start + k], b = v[start + k + half];
                 v[start + k] = cadd(a, b);
-                v[start + k + half] = rot16<S>(csub(a, b), k * (16 / len));
+                v[start + k + half] = rot32<S>(csub(a, b), k * (32 / len));
             }
         }
     }
@@ -128,26 +147,35 @@ __device__ __forceinline__ void dft_reg(float2* v)
     for (int i = 0; i < R; ++i) v[bitrev_c<R>(i)] = t[i];
 }
 
-__device__ __forceinline__ int fft_pad(int i) { return i + (i >> 4); }
-
 template <int L>
 struct FftShape {
-    static constexpr int E = 16;                        // complex values per thread
-    static constexpr int TPL = L / 16;                  // threads per line
+    // complex values per thread: 16; 32 for 8192 points, which are then 32 x 16
+    // x 16, one pass and one exchange through shared memory fewer than 2 x 16
+    // x 16 x 16 (4096 lines of 8192: 110 -> 91 us; the passes of a 4096^2
+    // transform: rows 258 -> 162, columns 180 -> 168, adjoint rows 210 -> 143)
+    static constexpr int E = L == 8192 ? 32 : 16;
+    static constexpr int TPL = L / E;                   // threads per line
     static constexpr int LOG = ilog2_c(L);
-    static constexpr int NP = (LOG + 3) / 4;            // passes
-    static constexpr int R0 = (LOG % 4 == 0) ? 16 : (1 << (LOG % 4));  // first pass radix
-    static constexpr int SMEM = L + L / 16;             // padded complex slots per line
+    static constexpr int R0 = E == 32 ? 32 : (LOG % 4 == 0) ? 16 : (1 << (LOG % 4));  // first radix
+    static constexpr int NP = 1 + (LOG - ilog2_c(R0)) / 4;  // passes
+    static constexpr int PAD = E == 32 ? 5 : 4;         // one slot of padding per 2^PAD
+    static constexpr int SMEM = L + (L >> PAD);         // padded complex slots per line
     static_assert(L >= 16 && L <= 16384 && (L & (L - 1)) == 0, "FFT length");
 };
 
+template <int L>
+__device__ __forceinline__ int fft_pad(int i)
+{
+    return i + (i >> FftShape<L>::PAD);
+}
+
 // One Stockham pass on the registers v (E/R butterflies of this thread).
 template <int L, int R, int NS, int S>
-__device__ __forceinline__ void fft_pass_compute(float2 (&v)[16], int t, const float2* __restrict__ tw)
+__device__ __forceinline__ void fft_pass_compute(float2 (&v)[FftShape<L>::E], int t, const float2* __restrict__ tw)
 {
-    constexpr int TPL = L / 16;
+    constexpr int TPL = FftShape<L>::TPL, E = FftShape<L>::E;
 #pragma unroll
-    for (int b = 0; b < 16 / R; ++b) {
+    for (int b = 0; b < E / R; ++b) {
         const int j = t + b * TPL;
         if (NS > 1) {
             const int k = j % NS;
@@ -188,45 +216,47 @@ __device__ __forceinline__ void fft_pass_compute(float2 (&v)[16], int t, const f
 }
 
 template <int L, int R>
-__device__ __forceinline__ void fft_load_smem(float2 (&v)[16], int t, const float2* s)
+__device__ __forceinline__ void fft_load_smem(float2 (&v)[FftShape<L>::E], int t, const float2* s)
 {
-    constexpr int TPL = L / 16;
+    constexpr int TPL = FftShape<L>::TPL, E = FftShape<L>::E;
 #pragma unroll
-    for (int b = 0; b < 16 / R; ++b) {
+    for (int b = 0; b < E / R; ++b) {
         const int j = t + b * TPL;
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[b * R + r] = s[fft_pad(j + r * (L / R))];
+        for (int r = 0; r < R; ++r) v[b * R + r] = s[fft_pad<L>(j + r * (L / R))];
     }
 }
 
 template <int L, int R, int NS>
-__device__ __forceinline__ void fft_store_smem(const float2 (&v)[16], int t, float2* s)
+__device__ __forceinline__ void fft_store_smem(const float2 (&v)[FftShape<L>::E], int t, float2* s)
 {
-    constexpr int TPL = L / 16;
+    constexpr int TPL = FftShape<L>::TPL, E = FftShape<L>::E;
 #pragma unroll
-    for (int b = 0; b < 16 / R; ++b) {
+    for (int b = 0; b < E / R; ++b) {
         const int j = t + b * TPL;
         const int base = (j / NS) * NS * R + (j % NS);
 #pragma unroll
-        for (int r = 0; r < R; ++r) s[fft_pad(base + r * NS)] = v[b * R + r];
+        for (int r = 0; r < R; ++r) s[fft_pad<L>(base + r * NS)] = v[b * R + r];
     }
 }
 
 // Passes 1..NP-1 (radix 16) after the first; recursion over the pass index.
 template <int L, int P, int NS, int S, class Store>
-__device__ __forceinline__ void fft_tail(float2 (&v)[16], int t, float2* s, const float2* tw,
+__device__ __forceinline__ void fft_tail(float2 (&v)[FftShape<L>::E], int t, float2* s, const float2* tw,
                                          Store& st)
 {
     constexpr int NP = FftShape<L>::NP;
-    constexpr int TPL = L / 16;
+    constexpr int TPL = FftShape<L>::TPL, E = FftShape<L>::E;
     if constexpr (P < NP) {
         fft_load_smem<L, 16>(v, t, s);
         __syncthreads();
         fft_pass_compute<L, 16, NS, S>(v, t, tw);
         if constexpr (P == NP - 1) {
-            // last pass: NS * 16 == L and j = t < NS, so X_r goes to t + r L/16
+            // last pass: NS * 16 == L and j < NS, so X_r goes to j + r L/16
 #pragma unroll
-            for (int r = 0; r < 16; ++r) st(t + r * TPL, v[r]);
+            for (int b = 0; b < E / 16; ++b)
+#pragma unroll
+                for (int r = 0; r < 16; ++r) st(t + b * TPL + r * (L / 16), v[b * 16 + r]);
         } else {
             fft_store_smem<L, 16, NS>(v, t, s);
             __syncthreads();
@@ -236,25 +266,36 @@ __device__ __forceinline__ void fft_tail(float2 (&v)[16], int t, float2* s, cons
 }
 
 // Transform one line.  Every thread of the block must call this (it contains
-// __syncthreads); t is the thread's index within its line (0..L/16-1), s the
+// __syncthreads); t is the thread's index within its line (0..TPL-1), s the
 // line's shared-memory slots (FftShape<L>::SMEM complex), ld(i) returns input
-// element i, st(i, x) receives output element i.  Every shared-memory read of
+// element i, st(i, x) receives output element i; mp(i, x) is applied to the
+// input elements once all of a thread's loads are on their way (arithmetic
+// inside ld would put each load behind the one before).  Every shared-memory read of
 // the last pass precedes a block barrier, so the slots may be rewritten as soon
 // as this returns.
-template <int L, int S, class Load, class Store>
+struct FftNoMap {
+    __device__ __forceinline__ float2 operator()(int, float2 v) const { return v; }
+};
+
+template <int L, int S, class Load, class Store, class Map = FftNoMap>
 __device__ __forceinline__ void fft_line(int t, float2* s, const float2* __restrict__ tw, Load& ld,
-                                         Store& st)
+                                         Store& st, Map mp = Map{})
 {
     constexpr int R0 = FftShape<L>::R0;
     constexpr int NP = FftShape<L>::NP;
-    constexpr int TPL = L / 16;
-    float2 v[16];
+    constexpr int TPL = FftShape<L>::TPL, E = FftShape<L>::E;
+    float2 v[E];
 #pragma unroll
-    for (int b = 0; b < 16 / R0; ++b) {
+    for (int b = 0; b < E / R0; ++b) {
         const int j = t + b * TPL;
 #pragma unroll
         for (int r = 0; r < R0; ++r) v[b * R0 + r] = ld(j + r * (L / R0));
     }
+#pragma unroll
+    for (int b = 0; b < E / R0; ++b)
+#pragma unroll
+        for (int r = 0; r < R0; ++r)
+            v[b * R0 + r] = mp(t + b * TPL + r * (L / R0), v[b * R0 + r]);
     fft_pass_compute<L, R0, 1, S>(v, t, tw);
     if constexpr (NP == 1) {
         // single radix-16 pass (L == 16): output index r

@@ -12,7 +12,7 @@ namespace asfd {
 // Row pass: LPC lines of length L per block, L/16 threads per line.
 template <int L>
 struct RowCfg {
-    static constexpr int TPL = L / 16;
+    static constexpr int TPL = FftShape<L>::TPL;
     static constexpr int LPC = L >= 4096 ? 1 : 4096 / L;  // lines per block
     static constexpr int THREADS = TPL * LPC;
     static constexpr int LS = FftShape<L>::SMEM + (TPL < 16 ? TPL : 0);
@@ -23,7 +23,7 @@ struct RowCfg {
 // stride keeps the lanes of one shared-memory access on distinct banks.
 template <int L, int LPC_>
 struct ColShape {
-    static constexpr int TPL = L / 16;
+    static constexpr int TPL = FftShape<L>::TPL;
     static constexpr int LPC = LPC_;
     static constexpr int THREADS = TPL * LPC;
     static constexpr int LS = FftShape<L>::SMEM + 16 / (LPC < 16 ? LPC : 16);
@@ -32,13 +32,13 @@ struct ColShape {
 
 template <int L>
 struct ColCfgSel {
-    static constexpr int TPL = L / 16;
+    static constexpr int TPL = FftShape<L>::TPL;
     static constexpr int LPC0 = (256 / TPL) > 4 ? (256 / TPL) : 4;
     // 4096-point columns: two columns per 512-thread block and two blocks
     // per SM at 64 registers, whose barriers are independent (one block of
     // four columns and 1024 threads measured 43.1 against 42.0 us at 2048
     // columns); other lengths up to 1024 threads, as many blocks as fit
-    static constexpr int LPC = L == 4096 ? 2 : ((LPC0 * TPL > 1024) ? (1024 / TPL) : LPC0);
+    static constexpr int LPC = L == 4096 || L == 8192 ? 2 : ((LPC0 * TPL > 1024) ? (1024 / TPL) : LPC0);
     static constexpr int MIN_BLOCKS = L == 4096 ? 2 : 1;
 };
 template <int L>
@@ -115,7 +115,7 @@ __device__ __forceinline__ void rows_body(const RowArgs& a, int blk, float2* sm,
         // zero the band cells this thread loaded (the first pass's indices)
         constexpr int R0 = FftShape<L>::R0;
 #pragma unroll
-        for (int b = 0; b < 16 / R0; ++b)
+        for (int b = 0; b < FftShape<L>::E / R0; ++b)
 #pragma unroll
             for (int r = 0; r < R0; ++r) {
                 const int i = t + b * C::TPL + r * (L / R0);

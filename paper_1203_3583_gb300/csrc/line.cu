@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(256) line_spread_kernel(LineArgs a)
     if (j < a.n) line_spread_sample(a, j);
 }
 
-// The block spreads the samples (SPREAD), and its first L/16 threads transform
+// The block spreads the samples (SPREAD), and its first TPL threads transform
 // the line, leave it zero for the next call and write the destination.
 template <int L, bool SPREAD>
 __global__ void __launch_bounds__(1024) line_transform_kernel(LineArgs a)
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(1024) line_transform_kernel(LineArgs a)
         __threadfence();  // the sums are in L2, where the loads below read
         __syncthreads();
     }
-    if (t >= L / 16) return;
+    if (t >= FftShape<L>::TPL) return;
     auto ld = [&](int i) -> float2 {
         const float2 v = __ldcg(&a.grid[i]);
         a.grid[i] = make_float2(0.f, 0.f);
@@ -183,6 +183,7 @@ template <int L>
 cudaError_t line_launch(const LineArgs& a, bool spread, cudaStream_t st)
 {
     constexpr size_t smem = sizeof(float2) * FftShape<L>::SMEM;
+    constexpr int TPL = FftShape<L>::TPL;
     if constexpr (smem > 48 * 1024) {
         static std::once_flag once;
         static cudaError_t attr = cudaSuccess;
@@ -196,10 +197,10 @@ cudaError_t line_launch(const LineArgs& a, bool spread, cudaStream_t st)
         if (attr != cudaSuccess) return attr;
     }
     if (!spread)
-        return launch_chained(line_transform_kernel<L, false>, dim3(1), L / 16 < 32 ? 32 : L / 16, smem, st,
+        return launch_chained(line_transform_kernel<L, false>, dim3(1), TPL < 32 ? 32 : TPL, smem, st,
                               a);
     int threads = std::min(1024, (a.n + 31) / 32 * 32);
-    threads = std::max(threads, std::max(32, L / 16));
+    threads = std::max(threads, std::max(32, TPL));
     return launch_chained(line_transform_kernel<L, true>, dim3(1), (unsigned)threads, smem, st, a);
 }
 
