@@ -116,6 +116,8 @@ struct asfd_plan_s {
     bool colored = false;
     bool windowed = false;          // register-window kernel applies (w <= kMaxWindowWidth)
     bool dense = false;             // dense map: register windows flushed with global atomics
+    bool dup = false;               // dense: samples well below a cell apart in x, rows added up
+                                    // over neighbouring lanes before their reductions
     bool wraps = false;             // some footprint wraps around the periodic grid
     bool fold = false;              // folding or wrapping map: register windows flushed with
                                     // global atomics to wrapped cells
@@ -264,7 +266,7 @@ asfd_status launch_interp_grad(asfd_plan_s* P, const float2* u1, float2* gu1, fl
 // resident at once (SMs x resident blocks x 4 warps), and the rows per run
 // that make the items of 32 columns x rows fill whole waves of those slots
 // (two waves when the runs stay at least 32 rows long, else one).
-asfd_status dense_spread_warp_slots(int w, bool table, long long* slots);
+asfd_status dense_spread_warp_slots(int w, bool table, bool dup, long long* slots);
 // folding or wrapping maps: the same for spread_es_dense_kernel<.., true> and,
 // above kMaxWindowWidth, spread_fold_kernel (spread_split(w) lanes per column)
 asfd_status fold_spread_warp_slots(int w, bool table, long long* slots);

@@ -403,6 +403,12 @@ bool pow2_in(int n, int lo, int hi) { return n >= lo && n <= hi && (n & (n - 1))
 
 }  // namespace
 
+// Sample spacing in x (fine cells) below which rows are added up over lanes
+// before they go to the grid.  The spread of 1024^2 samples, without and with
+// (us): 0.5 cells apart 23.1, 21.1; 0.2: 27.2, 21.4; 0.05: 56.7, 23.0; but 2048^2
+// at 0.49, whose band is large: 62.3, 69.3.
+constexpr double kDupSpacing = 0.45;
+
 asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double msy, cudaStream_t st);
 
 asfd_status plan_alloc_buffer(asfd_plan_s* P, void** p, size_t bytes) { return alloc(P, p, bytes); }
@@ -813,7 +819,9 @@ asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double ms
         // dense_rows rows per lane, in whole waves of the resident warps
         const long long ncb = (p.n1x + 31) / 32;
         long long slots = 0;
-        const asfd_status s = dense_spread_warp_slots(P->w, p.kind == ASFD_KERNEL_LEARNED, &slots);
+        P->dup = msx < kDupSpacing;
+        const asfd_status s =
+            dense_spread_warp_slots(P->w, p.kind == ASFD_KERNEL_LEARNED, P->dup, &slots);
         if (s != ASFD_OK) return s;
         const long long rows = window_run_rows(p.n1y, ncb, slots);
         P->dense_rows = (int)rows;

@@ -65,9 +65,12 @@ cudaError_t launch_dense(const SpreadArgs& a, int tiles, bool clear, cudaStream_
     }
     const unsigned blocks = (a.dense_items + kDenseWarps - 1) / kDenseWarps;
     if (a.wrap)
-        return launch_chained(spread_es_dense_kernel<W, TAB, true>, blocks, 32 * kDenseWarps, 0, st, a,
+        return launch_chained(spread_es_dense_kernel<W, TAB, true, false>, blocks, 32 * kDenseWarps, 0, st, a,
                               a.dense_items);
-    return launch_chained(spread_es_dense_kernel<W, TAB, false>, blocks, 32 * kDenseWarps, 0, st, a,
+    if (a.dup)
+        return launch_chained(spread_es_dense_kernel<W, TAB, false, true>, blocks, 32 * kDenseWarps, 0, st,
+                              a, a.dense_items);
+    return launch_chained(spread_es_dense_kernel<W, TAB, false, false>, blocks, 32 * kDenseWarps, 0, st, a,
                           a.dense_items);
 }
 
@@ -133,11 +136,16 @@ asfd_status fold_spread_warp_slots(int w, bool table, long long* slots)
     }
 }
 
-asfd_status dense_spread_warp_slots(int w, bool table, long long* slots)
+asfd_status dense_spread_warp_slots(int w, bool table, bool dup, long long* slots)
 {
-    if (table) return resident_warps((const void*)spread_es_dense_kernel<kLearnW, true>, slots);
+    if (table)
+        return resident_warps(dup ? (const void*)spread_es_dense_kernel<kLearnW, true, false, true>
+                                  : (const void*)spread_es_dense_kernel<kLearnW, true>, slots);
     switch (w) {
-#define ASFD_SW(W) case W: return resident_warps((const void*)spread_es_dense_kernel<W, false>, slots);
+#define ASFD_SW(W)                                                                               \
+    case W:                                                                                      \
+        return resident_warps(dup ? (const void*)spread_es_dense_kernel<W, false, false, true>   \
+                                  : (const void*)spread_es_dense_kernel<W, false>, slots);
         ASFD_SW(2) ASFD_SW(3) ASFD_SW(4) ASFD_SW(5) ASFD_SW(6) ASFD_SW(7)
 #undef ASFD_SW
         default: return fail(ASFD_ERR_UNSUPPORTED, "dense spread widths are 2..7");
@@ -185,6 +193,7 @@ SpreadArgs make_spread_args(const asfd_plan_s* P, const float2* u1)
     a.dense_rows = P->dense || P->fold ? P->dense_rows : 0;
     a.dense_items = P->dense || P->fold ? P->dense_items : 0;
     a.wrap = P->fold;
+    a.dup = P->dense && P->dup;
     a.inc_d = (float)P->inc_d;
     a.half_w = 0.5f * (float)P->w;
     a.beta_log2e = (float)(P->beta * 1.4426950408889634074);
@@ -200,13 +209,11 @@ asfd_status launch_spread_into(asfd_plan_s* P, const float2* u1, float2* grid, c
     a.grid = grid;
     if (a.dense_items <= 0) return ASFD_OK;
     cudaError_t e = cudaSuccess;
-    const unsigned blocks = (a.dense_items + kDenseWarps - 1) / kDenseWarps;
     if (P->learned) {
-        e = launch_chained(spread_es_dense_kernel<kLearnW, true, false>, blocks, 32 * kDenseWarps, 0, st, a,
-                           a.dense_items);
+        e = launch_dense<kLearnW, true>(a, 0, false, st);
     } else {
         switch (P->w) {
-#define ASFD_SI(W) case W: e = launch_chained(spread_es_dense_kernel<W, false, false>, blocks, 32 * kDenseWarps, 0, st, a, a.dense_items); break;
+#define ASFD_SI(W) case W: e = launch_dense<W, false>(a, 0, false, st); break;
             ASFD_SI(2) ASFD_SI(3) ASFD_SI(4) ASFD_SI(5) ASFD_SI(6) ASFD_SI(7)
 #undef ASFD_SI
             default: return fail(ASFD_ERR_UNSUPPORTED, "dense spread widths are 2..7");

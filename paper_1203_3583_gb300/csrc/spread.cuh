@@ -28,6 +28,7 @@ struct SpreadArgs {
     int dense_rows;    // rows per run of the dense (global-atomic) window kernel (0: not used)
     int dense_items;   // its warp items (32 columns x dense_rows rows each)
     bool wrap;         // the map folds or wraps (dense_rows of the wrapping kernels)
+    bool dup;          // samples well below a cell apart: rows added up over lanes first
     float inc_d;       // incident depth phase, half-turns per unit d1/z0
     float half_w;      // w/2
     float beta_log2e;  // beta * log2(e)
@@ -568,7 +569,12 @@ constexpr int kDenseRing = 4;   // ring slots (> kDenseAhead, power of two)
 constexpr int kDenseRingBytes = kDenseRing * (32 * (8 + 4) + 32);  // per warp
 
 // WRAP: the cells' columns wrap around the periodic grid.
-template <int W, bool TAB = false, bool WRAP = false>
+// DUP (samples well below a cell apart): many lanes of a warp hold windows at
+// the same cells, and their reductions would meet in L2 one after the other.
+// Rows that leave the windows of neighbouring lanes with one first tap are
+// added up over those lanes first (a segmented shuffle reduction) and sent by
+// the first of them.
+template <int W, bool TAB = false, bool WRAP = false, bool DUP = false>
 __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, int lane,
                                                    char* ring, float4* tsm = nullptr)
 {
@@ -580,8 +586,8 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
     // lanes that stay in the item (without the learned kernel, lanes past
     // the last column return below)
     const int ncols = a.n1x - (it % ncb) * 32;
-    const unsigned wmask = (TAB || ncols >= 32) ? 0xffffffffu : ((1u << max(ncols, 0)) - 1u);
-    if constexpr (TAB) {
+    const unsigned wmask = (TAB || DUP || ncols >= 32) ? 0xffffffffu : ((1u << max(ncols, 0)) - 1u);
+    if constexpr (TAB || DUP) {
         // learned kernel: the warp's lanes span two source-tile columns and
         // step through the same rows, so the two tiles' polynomial tables
         // are staged in shared memory (tsm: 2 x 4W float4) per tile row
@@ -589,9 +595,9 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
     } else {
         if (nx >= a.n1x || ny0 > nyl) return;
     }
-    // (learned kernel: lanes past the last column follow along without flushing)
-    const bool lane_on = !TAB || nx < a.n1x;
-    const int nxc = (!TAB || lane_on) ? nx : a.n1x - 1;
+    // (lanes past the last column follow along without flushing)
+    const bool lane_on = !(TAB || DUP) || nx < a.n1x;
+    const int nxc = lane_on ? nx : a.n1x - 1;
     const int my = a.nfy - 1;
     const float neg_c2 = -a.two_over_w * a.two_over_w;
     const AxisEntry ex = a.ax[nxc];
@@ -628,6 +634,40 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
 #pragma unroll
             for (int i = 0; i < WX; ++i)
                 if (lane_on && i < W + maxoff) atomicAdd(row + i, acc[b][i]);
+        }
+    };
+    // DUP: runs of lanes with one first tap (the lane's run ends at seg_end,
+    // starts at a head), the longest of them, and a row of them added up
+    int seg_end = 0, seg_most = 1;
+    bool head = true;
+    auto segments = [&](bool on) {
+        const unsigned key = on ? (unsigned)R0 << 16 | ((unsigned)X0 & 0xffffu) : ~(unsigned)lane;
+        const unsigned prev = __shfl_up_sync(0xffffffffu, key, 1);
+        head = lane == 0 || key != prev;
+        const unsigned heads = __ballot_sync(0xffffffffu, head);
+        const unsigned above = lane == 31 ? 0u : heads & ~((2u << lane) - 1u);
+        seg_end = above ? __ffs(above) - 2 : 31;
+        seg_most = __reduce_max_sync(0xffffffffu, head ? seg_end - lane + 1 : 1);
+    };
+    auto flush_segment_row = [&](int b, bool on) {
+        float2 v[WX];
+#pragma unroll
+        for (int i = 0; i < WX; ++i) v[i] = on ? acc[b][i] : make_float2(0.f, 0.f);
+        const unsigned any = __ballot_sync(0xffffffffu, on);
+        for (int o = 1; o < seg_most; o <<= 1) {  // warp-uniform
+            const bool take = lane + o <= seg_end;
+#pragma unroll
+            for (int i = 0; i < WX; ++i) {
+                const float x = __shfl_down_sync(0xffffffffu, v[i].x, o);
+                const float y = __shfl_down_sync(0xffffffffu, v[i].y, o);
+                if (take) v[i] = add2(v[i], make_float2(x, y));
+            }
+        }
+        const unsigned mine = (0xffffffffu >> (31 - seg_end)) & (0xffffffffu << lane);
+        if (head && (any & mine)) {
+            float2* row = a.grid + (size_t)((R0 + b) & my) * a.nfx + min(max(X0, 0), a.nfx - W - maxoff);
+#pragma unroll
+            for (int i = 0; i < WX; ++i) atomicAdd(row + i, v[i]);
         }
     };
     // u1 and q of the run's rows are copied asynchronously (cp.async) into a
@@ -685,7 +725,18 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
         float dx, dy;
         sample_pos(ex, ey, px, py, q, a.half_w, l0x, l0y, dx, dy);
         const int off = l0x - X0, d = l0y - R0;
-        if (live && (off < 0 || off > maxoff || d < 0 || d > 2)) {
+        const bool restart = live && (off < 0 || off > maxoff || d < 0 || d > 2);
+        if constexpr (DUP) {
+            // rows that leave the windows of the lanes that go on
+            const int n = lane_on && live && !restart ? d : 0;
+            const int most = __reduce_max_sync(0xffffffffu, n);
+            if (most > 0) {
+                segments(n > 0);
+                flush_segment_row(0, n > 0);
+                if (most > 1) flush_segment_row(1, n > 1);
+            }
+        }
+        if (restart) {
 #pragma unroll
             for (int b = 0; b < W; ++b) flush_row(b);
             live = false;
@@ -699,6 +750,9 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
             R0 = l0y;
             live = true;
         }
+        auto leave = [&](int b) {  // (DUP: the rows have left above)
+            if constexpr (!DUP) flush_row(b);
+        };
         const float2 c = sample_value_fast(u, ex, ey, q, a.inc_d);
         if constexpr (TAB) {
             if (ny / kSrcTile != tab_ty) {  // warp-uniform: every lane is on row ny
@@ -721,13 +775,17 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
             }
             float wx[W], wy[W];
             table_weights_smem<W>(tsm + (nxc / kSrcTile - tcol0) * (4 * W), dx, dy, wx, wy);
-            window_add_w<W, WX>(acc, fresh, l0y - R0, l0x - X0, wx, wy, c, flush_row);
+            window_add_w<W, WX>(acc, fresh, l0y - R0, l0x - X0, wx, wy, c, leave);
         } else {
-            window_add<W, WX>(acc, fresh, l0y - R0, l0x - X0, dx, dy, c, a, neg_c2, flush_row);
+            window_add<W, WX>(acc, fresh, l0y - R0, l0x - X0, dx, dy, c, a, neg_c2, leave);
         }
         R0 = l0y;
     }
-    if (live) {
+    if constexpr (DUP) {
+        segments(lane_on);
+#pragma unroll
+        for (int b = 0; b < W; ++b) flush_segment_row(b, lane_on);
+    } else if (live) {
 #pragma unroll
         for (int b = 0; b < W; ++b) flush_row(b);
     }
@@ -737,7 +795,7 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
 // registers capped for more resident warps spilled and ran slower)
 constexpr int kDenseWarps = 4;
 
-template <int W, bool TAB = false, bool WRAP = false>
+template <int W, bool TAB = false, bool WRAP = false, bool DUP = false>
 __global__ void __launch_bounds__(32 * kDenseWarps) spread_es_dense_kernel(SpreadArgs a, int items)
 {
     __shared__ float4 tsm[kDenseWarps][TAB ? 8 * W : 1];
@@ -746,8 +804,8 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_es_dense_kernel(Sprea
     chain_next();
     chain_wait();
     if (it < items)
-        window_atomic_item<W, TAB, WRAP>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
-                                         tsm[threadIdx.x / 32]);
+        window_atomic_item<W, TAB, WRAP, DUP>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
+                                              tsm[threadIdx.x / 32]);
 }
 
 // Fallback spread of band tile `tile` (kTileX x kTileY) by a whole block:
