@@ -37,9 +37,11 @@ struct ColCfgSel {
     // 4096-point columns: two columns per 512-thread block and two blocks
     // per SM at 64 registers, whose barriers are independent (one block of
     // four columns and 1024 threads measured 43.1 against 42.0 us at 2048
-    // columns); other lengths up to 1024 threads, as many blocks as fit
+    // columns); 2048-point columns: four per 512-thread block, two blocks per SM
+    // likewise (1024 columns then run in one wave, not two: a 1024^2 transform 52.0
+    // -> 46.6 us); other lengths up to 1024 threads, as many blocks as fit
     static constexpr int LPC = L == 4096 || L == 8192 ? 2 : ((LPC0 * TPL > 1024) ? (1024 / TPL) : LPC0);
-    static constexpr int MIN_BLOCKS = L == 4096 ? 2 : 1;
+    static constexpr int MIN_BLOCKS = L == 4096 || L == 2048 ? 2 : 1;
 };
 template <int L>
 using ColCfg = ColShape<L, ColCfgSel<L>::LPC>;
