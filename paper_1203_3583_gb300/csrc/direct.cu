@@ -90,6 +90,8 @@ direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
                    DirectTerms* __restrict__ out, unsigned* __restrict__ bad)
 {
     __shared__ double ys[kPrepRows];
+    chain_next();
+    chain_wait();
     const int nx = blockIdx.x * 256 + threadIdx.x, ny0 = blockIdx.y * kPrepRows;
     if (threadIdx.x < kPrepRows)
         ys[threadIdx.x] = (ny0 + (int)threadIdx.x - g.n1y / 2) * g.p1y + g.oy;
@@ -202,6 +204,8 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
 {
     constexpr int P = kDirectPoints;
     static_assert(P % 2 == 0 && P <= 32, "points in pairs, a lane each for the sums");
+    chain_next();
+    chain_wait();
     __shared__ double red[2][P][kDirectThreads / 32];
     const int p0 = blockIdx.x * P;
     unsigned ix[P], iy[P];
@@ -355,6 +359,8 @@ __global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int
                                      const double2* __restrict__ part,
                                      const unsigned* __restrict__ bad, float2* __restrict__ out)
 {
+    chain_next();
+    chain_wait();
     const int i = (int)(((size_t)blockIdx.x * blockDim.x + threadIdx.x) / 32);
     const int lane = threadIdx.x % 32;
     if (i >= npts) return;  // warp-uniform
@@ -442,20 +448,29 @@ asfd_status direct_sum(const asfd_params* p, const double* d1, const float2* u1,
     double2* part = reinterpret_cast<double2*>(s + n);
     unsigned* bad = reinterpret_cast<unsigned*>(part + chunks * npts);
     e = cudaMemsetAsync(bad, 0, sizeof(unsigned), st);
-    direct_prep_kernel<<<dim3((unsigned)((p->n1x + 255) / 256),
-                              (unsigned)((p->n1y + kPrepRows - 1) / kPrepRows)),
-                         256, 0, st>>>(g, d1, eq, s, bad);
+    if (e == cudaSuccess)
+        e = launch_chained(direct_prep_kernel,
+                           dim3((unsigned)((p->n1x + 255) / 256),
+                                (unsigned)((p->n1y + kPrepRows - 1) / kPrepRows)),
+                           256, 0, st, g, d1, eq, s, bad);
     const dim3 grid((unsigned)groups, (unsigned)chunks);
     const size_t chunk = rows * kDirectThreads;
-    switch (eq) {
-#define ASFD_DS(F) case F: direct_sum_kernel<F><<<grid, kDirectThreads, 0, st>>>(g, s, u1, npts, mx, my, chunk, part); break;
-        ASFD_DS(kEq2) ASFD_DS(kEq5) ASFD_DS(kEq5Uneven) ASFD_DS(kEq7)
+    using T = const DirectTerms*;
+    if (e == cudaSuccess) {
+        switch (eq) {
+#define ASFD_DS(F)                                                                                      \
+    case F:                                                                                             \
+        e = launch_chained(direct_sum_kernel<F>, grid, kDirectThreads, 0, st, g, T(s), u1, npts, mx, my, \
+                           chunk, part);                                                                \
+        break;
+            ASFD_DS(kEq2) ASFD_DS(kEq5) ASFD_DS(kEq5Uneven) ASFD_DS(kEq7)
 #undef ASFD_DS
-        default: break;
+            default: break;
+        }
     }
-    direct_finish_kernel<<<(unsigned)(((size_t)npts + 7) / 8), 256, 0, st>>>(
-        g, eq, npts, mx, my, (int)chunks, part, bad, out);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = launch_chained(direct_finish_kernel, dim3((unsigned)(((size_t)npts + 7) / 8)), 256, 0, st, g, eq,
+                           npts, mx, my, (int)chunks, (const double2*)part, (const unsigned*)bad, out);
     const cudaError_t ef = cudaFreeAsync(s, st);
     if (e != cudaSuccess) return cuda_fail(e, "direct_sum_kernel launch");
     if (ef != cudaSuccess) return cuda_fail(ef, "cudaFreeAsync");

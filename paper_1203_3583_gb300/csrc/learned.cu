@@ -25,6 +25,7 @@
 //   (likewise y); MLP backward over tiles; Adam update; tables refreshed.
 // All of it runs in the kernels of this file and the FFT passes; the host only
 // sequences launches and reads back the loss.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -108,6 +109,8 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restric
     static_assert(O == 64 && H % 4 == 0, "four tiles at a time in 256 threads");
     __shared__ float w1[H][F + 1], f[T][F];
     __shared__ __align__(16) float h[T][H];
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x, t0 = blockIdx.x * T, nt = min(T, ntiles - t0);
     for (int i = tid; i < H * F; i += 256) w1[i / F][i % F] = prm[kLpW1 + i];
     for (int i = tid; i < nt * F; i += 256) f[i / F][i % F] = feat[(size_t)t0 * F + i];
@@ -159,6 +162,8 @@ __device__ __forceinline__ void cheb_even(float u, float (&T)[kLearnCheb])
 __global__ void deconv_build_kernel(const float* __restrict__ prm, const float2* __restrict__ cb,
                                     float2* __restrict__ c, float* __restrict__ corr, int m, int off)
 {
+    chain_next();
+    chain_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= m) return;
     const float u = 2.f * (float)(k - m / 2) / (float)m;
@@ -223,6 +228,8 @@ __global__ void __launch_bounds__(256) ref_norm_kernel(const float2* __restrict_
                                                        double* red, float* __restrict__ gcorr,
                                                        int ncorr)
 {
+    chain_next();
+    chain_wait();
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t step = (size_t)gridDim.x * blockDim.x;
     for (size_t i = i0; i < (size_t)ncorr; i += step) gcorr[i] = 0.f;
@@ -255,6 +262,8 @@ loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
             const float* __restrict__ corr, int m2x, int m2y, double* red, float2* __restrict__ g,
             float* __restrict__ gcorr)
 {
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c0 = blockIdx.x * kLossCols + lane;
     const int y1 = min(m2y, (int)(blockIdx.y + 1) * kLossRows);
@@ -312,6 +321,8 @@ loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
 __global__ void __launch_bounds__(1024) cheb_grad_kernel(const float* __restrict__ gcorr, int m2x,
                                                          int m2y, float* __restrict__ grad)
 {
+    chain_next();
+    chain_wait();
     const int m = blockIdx.x == 0 ? m2x : m2y;
     if (blockIdx.x == 1) gcorr += m2x;
     grad += blockIdx.x == 0 ? kLpDx : kLpDy;
@@ -368,6 +379,8 @@ __global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int
     constexpr int W = kLearnW, K = kLearnCoef;
     static_assert(kSrcTile == 16 && 2 * W * K == 64, "half a column per lane, 64 sums over 32 lanes");
     __shared__ __align__(16) float tsm[kTgWarps][2 * W * K];
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
     const int t = blockIdx.x * kTgWarps + wid;
     if (t >= ntiles) return;  // warp-uniform
@@ -491,6 +504,8 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
                   "one (tile, unit) per thread");
     __shared__ __align__(16) float dout[T][O], h[T][H];
     __shared__ float f[T][F], dh[T][H];
+    chain_next();
+    chain_wait();
     const int tid = threadIdx.x;
     const int o = tid / 4, i0 = (tid % 4) * 8;  // this thread's entries of W2
     const int k1 = tid / F, j1 = tid % F;       // and of W1 (tid < H F)
@@ -579,6 +594,8 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict
                                                          float* __restrict__ grad)
 {
     __shared__ float red[8][32];
+    chain_next();
+    chain_wait();
     const int lane = threadIdx.x & 31, wid = threadIdx.x / 32;
     const int i = blockIdx.x * 32 + lane;
     float v = 0.f;
@@ -599,6 +616,8 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
                             float* __restrict__ v, int n, float lr, float b1, float b2, float c1,
                             float c2, float eps)
 {
+    chain_next();
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -676,14 +695,14 @@ asfd_status learned_features(asfd_plan_s* P, cudaStream_t st)
 asfd_status learned_refresh(asfd_plan_s* P, cudaStream_t st)
 {
     const int nst = P->nstx * P->nsty;
-    mlp_forward_kernel<<<(nst + kMlpTiles - 1) / kMlpTiles, 256, 0, st>>>(P->lparams, P->lfeat, nst,
-                                                                          P->lhid, P->ltab);
+    using F = const float*;
+    ASFD_CUDA(launch_chained(mlp_forward_kernel, dim3((nst + kMlpTiles - 1) / kMlpTiles), 256, 0, st,
+                             F(P->lparams), F(P->lfeat), nst, P->lhid, P->ltab));
     const int m2x = P->prm.m2x, m2y = P->prm.m2y;
-    deconv_build_kernel<<<(m2x + 255) / 256, 256, 0, st>>>(P->lparams, P->cxb, P->cx, P->lcorr, m2x,
-                                                           kLpDx);
-    deconv_build_kernel<<<(m2y + 255) / 256, 256, 0, st>>>(P->lparams, P->cyb, P->cy,
-                                                           P->lcorr + m2x, m2y, kLpDy);
-    ASFD_CUDA(cudaGetLastError());
+    ASFD_CUDA(launch_chained(deconv_build_kernel, dim3((m2x + 255) / 256), 256, 0, st, F(P->lparams),
+                             (const float2*)P->cxb, P->cx, P->lcorr, m2x, kLpDx));
+    ASFD_CUDA(launch_chained(deconv_build_kernel, dim3((m2y + 255) / 256), 256, 0, st, F(P->lparams),
+                             (const float2*)P->cyb, P->cy, P->lcorr + m2x, m2y, kLpDy));
     return ASFD_OK;
 }
 
@@ -751,16 +770,21 @@ asfd_status learned_gradient(asfd_plan_s* P, const float2* u1, const float2* ref
     asfd_status s;
     // forward with the current model (its tables are current: every change of
     // the parameters or the height map rebuilds them)
+    // (the memset first: it would break the chain of the kernels' launches)
+    ASFD_CUDA(cudaMemsetAsync(P->lred, 0, sizeof(double) * 2, st));
     if ((s = launch_spread(P, u1, st)) != ASFD_OK) return s;
     if ((s = launch_fft_rows(P, st)) != ASFD_OK) return s;
     if ((s = launch_fft_cols(P, P->lu2, st)) != ASFD_OK) return s;
     // loss, its gradient with respect to u2 and the deconvolution correction's
-    ASFD_CUDA(cudaMemsetAsync(P->lred, 0, sizeof(double) * 2, st));
-    ref_norm_kernel<<<kLossBlocks, 256, 0, st>>>(ref, m, P->lred, P->lcgrad, m2x + m2y);
-    loss_kernel<<<dim3((m2x + kLossCols - 1) / kLossCols, (m2y + kLossRows - 1) / kLossRows), 256, 0,
-                  st>>>(P->lu2, ref, P->lcorr, m2x, m2y, P->lred, P->lres, P->lcgrad);
-    cheb_grad_kernel<<<2, 1024, 0, st>>>(P->lcgrad, m2x, m2y, P->lgrad);
-    ASFD_CUDA(cudaGetLastError());
+    using F = const float*;
+    using F2 = const float2*;
+    ASFD_CUDA(launch_chained(ref_norm_kernel, dim3(kLossBlocks), 256, 0, st, ref, m, P->lred, P->lcgrad,
+                             m2x + m2y));
+    ASFD_CUDA(launch_chained(loss_kernel,
+                             dim3((m2x + kLossCols - 1) / kLossCols, (m2y + kLossRows - 1) / kLossRows),
+                             256, 0, st, F2(P->lu2), ref, F(P->lcorr), m2x, m2y, P->lred, P->lres,
+                             P->lcgrad));
+    ASFD_CUDA(launch_chained(cheb_grad_kernel, dim3(2), 1024, 0, st, F(P->lcgrad), m2x, m2y, P->lgrad));
     // table gradients through the adjoint grid
     if ((s = launch_fft_cols_adj(P, P->lres, st)) != ASFD_OK) return s;
     if ((s = launch_fft_rows_adj(P, st)) != ASFD_OK) return s;
@@ -782,14 +806,13 @@ asfd_status learned_gradient(asfd_plan_s* P, const float2* u1, const float2* ref
     a.half_w = 0.5f * kLearnW;
     a.inc_d = (float)P->inc_d;
     const unsigned tgb = (unsigned)((nst + kTgWarps - 1) / kTgWarps);
-    if (!P->wraps) table_grad_kernel<false><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
-    else table_grad_kernel<true><<<tgb, 32 * kTgWarps, 0, st>>>(a, nst);
-    const int groups = (nst + kBackTiles - 1) / kBackTiles;
-    mlp_backward_kernel<<<groups < kBackBlocks ? groups : kBackBlocks, 256, 0, st>>>(
-        P->lparams, P->lfeat, P->lhid, P->ltgrad, nst, P->lpart);
-    mlp_reduce_kernel<<<(kMlpParams + 31) / 32, 256, 0, st>>>(
-        P->lpart, groups < kBackBlocks ? groups : kBackBlocks, P->lgrad);
-    ASFD_CUDA(cudaGetLastError());
+    ASFD_CUDA(launch_chained(P->wraps ? table_grad_kernel<true> : table_grad_kernel<false>, dim3(tgb),
+                             32 * kTgWarps, 0, st, a, nst));
+    const int groups = std::min((nst + kBackTiles - 1) / kBackTiles, kBackBlocks);
+    ASFD_CUDA(launch_chained(mlp_backward_kernel, dim3(groups), 256, 0, st, F(P->lparams), F(P->lfeat),
+                             F(P->lhid), F(P->ltgrad), nst, P->lpart));
+    ASFD_CUDA(launch_chained(mlp_reduce_kernel, dim3((kMlpParams + 31) / 32), 256, 0, st, F(P->lpart),
+                             groups, P->lgrad));
     return ASFD_OK;
 }
 
@@ -811,9 +834,8 @@ asfd_status learned_train_step(asfd_plan_s* P, const float2* u1, const float2* r
     ++P->lstep;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)P->lstep), c2 = 1.f - std::pow(b2, (float)P->lstep);
-    adam_kernel<<<(kLearnParams + 255) / 256, 256, 0, st>>>(P->lparams, P->lgrad, P->lm, P->lv,
-                                                           kLearnParams, lr, b1, b2, c1, c2, 1e-12f);
-    ASFD_CUDA(cudaGetLastError());
+    ASFD_CUDA(launch_chained(adam_kernel, dim3((kLearnParams + 255) / 256), 256, 0, st, P->lparams,
+                             (const float*)P->lgrad, P->lm, P->lv, kLearnParams, lr, b1, b2, c1, c2, 1e-12f));
     if ((s = learned_refresh(P, st)) != ASFD_OK) return s;
     if (loss_out) return learned_read_loss(P, loss_out, st);
     return ASFD_OK;
