@@ -600,8 +600,11 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
     const int nxc = lane_on ? nx : a.n1x - 1;
     const int my = a.nfy - 1;
     const float neg_c2 = -a.two_over_w * a.two_over_w;
+    // (the axis tables are the plan's for its lifetime; everything else is read
+    // after the kernel before this one has ended)
     const AxisEntry ex = a.ax[nxc];
     const AxisPos px = a.px[nxc];
+    chain_wait();
 
     // window columns: first tap columns of the run's first and last samples
     int X0, maxoff;
@@ -802,7 +805,6 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_es_dense_kernel(Sprea
     __shared__ __align__(16) char ring[kDenseWarps][kDenseRingBytes];
     const int it = blockIdx.x * kDenseWarps + threadIdx.x / 32;
     chain_next();
-    chain_wait();
     if (it < items)
         window_atomic_item<W, TAB, WRAP, DUP>(a, it, threadIdx.x % 32, ring[threadIdx.x / 32],
                                               tsm[threadIdx.x / 32]);
