@@ -197,7 +197,7 @@ def stage_bytes(info, g):
 
 
 STAGE_KERNELS = ["spread", "fft_rows_kernel", "fft_cols_kernel"]
-SPREAD_KERNEL = {0: "spread_es_colored_kernel", 1: "spread_es_atomic_kernel",
+SPREAD_KERNEL = {0: "spread_block_kernel", 1: "spread_fold_kernel",
                  2: "spread_es_window_kernel", 3: "spread_es_dense_kernel",
                  4: "spread_item_kernel"}
 # bytes per source sample of the whole forward step in the unpruned model:
@@ -211,10 +211,10 @@ STEP_BYTES_PER_SAMPLE = 116
 # changed since its capture, or without one, reports null)
 SPREAD_SOURCES = ("paper_1203_3583_gb300/csrc/spread.cuh", "paper_1203_3583_gb300/csrc/sample.cuh")
 NCU_TRAFFIC = {("spread_es_dense_kernel<7>", "smooth_random2048"): {
-    "bytes": 86.784000e6 + 1.624832e6,
+    "bytes": 86.785024e6 + 1.359616e6,
     "grid": 912,
     "capture": "profiles/spread_es_dense_w7_smooth_random2048.md",
-    "sources_sha1": "025f3964b6ff962a8ece156c70b2c7dcb768ebdb"}}
+    "sources_sha1": "22d068fa9d6d96011d17ea12b89e652eedd6efd0"}}
 
 
 def sources_sha1(paths) -> str:

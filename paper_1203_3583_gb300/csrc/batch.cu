@@ -28,7 +28,7 @@
 // device memory and are refreshed from a pinned host copy by a memcpy node of
 // the same graph, so one graph launch runs a whole batch for new field
 // pointers.  (At 24 surfaces of 256^2..2048^2 the stage barriers leave SMs
-// idle while the last items of a stage finish: 1.86 ms against 0.92 ms for
+// idle while the last items of a stage finish: 1.86 ms against 0.88 ms for
 // the stream schedule.)
 #include <cooperative_groups.h>
 

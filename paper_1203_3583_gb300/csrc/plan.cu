@@ -725,8 +725,8 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
     if (cs != ASFD_OK) return cs;
     P->tile_pairs = 0;
     if (!P->colored && !P->dense) {
-        // the shared-memory-atomic spread walks, per band tile, the source
-        // tiles whose footprints reach it: a CSR list built here
+        // the persistent batch's shared-memory-atomic tiles walk, per band tile,
+        // the source tiles whose footprints reach it: a CSR list built here
         const int nst = P->nstx * P->nsty;
         src_bbox_kernel<<<nst, kSrcTile * kSrcTile, 0, st>>>(P->q, P->ax, P->ay, P->bux, P->buy, p.n1x,
                                                              p.n1y, P->nstx, P->src_bbox);
@@ -875,7 +875,7 @@ asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double ms
     // the register-window tiles also need columns w apart across rows
     const double sxw = std::ceil((P->w + spread_x + margin) / msx);
     // beyond 64 samples between lanes (samples packed far below one cell
-    // apart) few lanes find work in a tile and the atomic kernel is faster
+    // apart) few lanes find work in a tile and the atomic windows are faster
     if (!(sxd <= 64.0) || !(hd <= 64.0)) return placed ? ASFD_OK : fold();
 
     // per band tile: source columns whose x range meets the tile's x range

@@ -19,12 +19,16 @@
 // error of g is that of the small term s q (about 1e-7 cells at the standard
 // workloads) rather than that of g itself.
 //
-// The tile kernels own fine-grid tiles (storage coordinates, centred: cell index
-// = g + nf/2 mod nf): each CTA accumulates in shared memory every tap of
-// every sample whose footprint reaches its tile, and writes the tile to
-// global memory once.  No global atomics.
+// Most plans take the register windows of spread_es_dense_kernel (default),
+// the item tiles of spread_item.cu or the block items of spread_block.cu (no
+// atomics between samples that share cells).  The tile kernels below serve the
+// plans whose item tiles fit no scratch and no shared memory, and the learned
+// kernel's deterministic plans.  They own fine-grid tiles (storage coordinates,
+// centred: cell index = g + nf/2 mod nf): each CTA accumulates in shared memory
+// every tap of every sample whose footprint reaches its tile, and writes the
+// tile to global memory once.  No global atomics.
 //
-//  * spread_es_colored_kernel (the fast path): one warp per tile, plain
+//  * spread_es_colored_kernel: one warp per tile, plain
 //    shared-memory read-modify-write without atomics.  The plan proves that
 //    the footprints of the 32 samples a warp handles in one step are
 //    pairwise disjoint: lanes form 4 row groups x 8 column groups; lanes of

@@ -31,7 +31,7 @@
 // Measured, whole transforms, against the conflict-free tiles and, for maps
 // denser than 64 samples per kernel width, the shared-memory float atomics that
 // these maps took before (us):
-//   2048^2, 1.04 cells per sample   w8 501 -> 229, w12 1465 -> 371, w16 3470 -> 707
+//   2048^2, 1.04 cells per sample   w8 501 -> 217, w12 1465 -> 359, w16 3470 -> 707
 //   600^2 onto 256^2 (0.4 cells)    w7 346 -> 124, w8 817 -> 89, w12 2617 -> 130
 //   1300 x 1258 onto 64^2 (0.03)    w7 199000 -> 818, w12 584000 -> 4980
 //   4096^2, 1.44 cells, w7          1871 -> 1184
