@@ -150,6 +150,9 @@ struct asfd_plan_s {
     bool band_clean = false;        // the band of the fine grid is known to be zero
                                     // (left so by the forward row pass, which
                                     // clears each cell it reads)
+    bool captured = false;          // a call of the plan's was captured: its replays write
+                                    // the grid without the plan's knowing
+    bool in_batch = false;          // the plan is a batch's own (its replays are the batch's)
     unsigned* status = nullptr;     // device status word
     float* stat = nullptr;          // a height map's statistics, per block
     // learned kernel (kind == ASFD_KERNEL_LEARNED)
@@ -228,6 +231,15 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, si
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Notes a call on P that is being captured into a graph (of the caller's).
+inline void note_capture(asfd_plan_s* P, cudaStream_t st)
+{
+    if (P->captured || P->in_batch) return;
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
+    else P->captured = s != cudaStreamCaptureStatusNone;
 }
 
 // stage launchers (each returns ASFD_OK or an error with a message)

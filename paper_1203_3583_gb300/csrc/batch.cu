@@ -455,6 +455,7 @@ asfd_status asfd_batch_create(asfd_batch* out, const asfd_params* params,
             asfd_plan p = nullptr;
             asfd_status r = asfd_plan_create(&p, &params[i], d1_devs[i], stream);
             if (r != ASFD_OK) return r;
+            p->in_batch = true;
             B->plans.push_back(p);
             if (p->nfx > kBatchMaxNf || p->nfy > kBatchMaxNf) B->persistent_ok = false;
             // both schedules read the plans' work buffers

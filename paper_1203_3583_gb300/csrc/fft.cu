@@ -354,6 +354,7 @@ asfd_status launch_fft_rows_adj(asfd_plan_s* P, cudaStream_t st)
     ASFD_FFT_SWITCH(P->nfx, ASFD_RA)
 #undef ASFD_RA
     P->band_clean = false;  // the band now holds the adjoint grid
+    note_capture(P, st);
     if (e != cudaSuccess) return cuda_fail(e, "fft_rows_adj_kernel launch");
     return ASFD_OK;
 }

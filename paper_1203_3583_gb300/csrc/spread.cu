@@ -239,8 +239,15 @@ asfd_status launch_spread(asfd_plan_s* P, const float2* u1, cudaStream_t st)
     const bool windowed = P->colored && P->windowed;
     // the accumulating (dense) kernels need a zero band; the tile kernels
     // overwrite every band cell
-    const bool clear = !P->band_clean;
+    bool clear = !P->band_clean;
     P->band_clean = false;
+    if (P->blk || P->fold) {
+        // these also clear a band that another writer may have used since the
+        // plan's own calls: a workspace's other plans, or replays of a graph
+        // (7.5 us at 2048^2, where a w = 12 transform takes 358)
+        note_capture(P, st);
+        clear = clear || P->ws || P->captured;
+    }
     if (P->itemtile) return launch_spread_itemtile(P, u1, st);
     if (P->blk) {
         if (clear) ASFD_CUDA(clear_band(a, tiles, st));
