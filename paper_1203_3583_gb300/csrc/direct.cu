@@ -81,9 +81,16 @@ constexpr unsigned kIndexBias = 0x80000000u;
 // A block takes 256 columns x kPrepRows rows: a thread's column terms serve its
 // rows, the rows' terms are formed once per block (FP64 is 2 lanes per clock
 // and SM: 45 FP64 operations per sample in a thread each took 90 us at 1024^2).
-// *bad is set when a term is not finite (d1 is not checked: a NaN, or d1 =
-// z0, makes every sum a NaN, which fixed point cannot carry).
+// *bad is set when a height or a term of the phase is not finite (d1 is not
+// checked: a NaN or an infinity, d1 = z0, or a term that overflows makes every
+// sum a NaN, which fixed point cannot carry).
 constexpr int kPrepRows = 8;
+
+// by the bits: FP64 comparisons are slow here
+__device__ __forceinline__ bool not_finite(double v)
+{
+    return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000;
+}
 
 __global__ void __launch_bounds__(256)
 direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
@@ -114,13 +121,18 @@ direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
             t.d = (unsigned long long)__double_as_longlong(w - 2.0 * rint(0.5 * w));
         } else {
             const double inv = 1.0 / (g.lambda * (g.z0 - h));
-            const unsigned long long b = turn_fraction(xp * inv);
-            const unsigned long long c = turn_fraction(y * g.p2y * inv);
-            t.a = turn_fraction(0.5 * (xx + y * y) * inv) +
-                  b * ((unsigned long long)kIndexBias + (unsigned)(g.m2x / 2)) +
+            const double ta = 0.5 * (xx + y * y) * inv, tb = xp * inv, tc = y * g.p2y * inv;
+            const unsigned long long b = turn_fraction(tb);
+            const unsigned long long c = turn_fraction(tc);
+            t.a = turn_fraction(ta) + b * ((unsigned long long)kIndexBias + (unsigned)(g.m2x / 2)) +
                   c * ((unsigned long long)kIndexBias + (unsigned)(g.m2y / 2));
-            if (tilted)
-                t.a += turn_fraction((g.sx * x + g.sy * y + (g.sz - 1.0) * h) * g.inv_lambda);
+            // (1 / (lambda (z0 - h)) of an infinite height is a finite zero)
+            bool nonfinite = not_finite(h) || not_finite(ta) || not_finite(tb) || not_finite(tc);
+            if (tilted) {
+                const double ti = (g.sx * x + g.sy * y + (g.sz - 1.0) * h) * g.inv_lambda;
+                t.a += turn_fraction(ti);
+                nonfinite = nonfinite || not_finite(ti);
+            }
             t.b = 0ull - b;
             t.c = 0ull - c;
             const double d = half_pp * inv;
@@ -129,7 +141,7 @@ direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
                 t.d = (unsigned long long)__double_as_longlong(d);
             else if (form == kEq5)
                 t.d = (unsigned long long)__double2ll_rn((d - rint(d)) * 18446744073709551616.0);
-            if (!isfinite(inv)) atomicOr(bad, 1u);
+            if (nonfinite || not_finite(d)) atomicOr(bad, 1u);
         }
         out[n] = t;
     }
