@@ -233,7 +233,8 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, si
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Notes a call on P that is being captured into a graph (of the caller's).
+// Notes a call on P that is being captured into a graph (of the caller's): what the
+// call does to the band happens at the replays, not now.
 inline void note_capture(asfd_plan_s* P, cudaStream_t st)
 {
     if (P->captured || P->in_batch) return;

@@ -174,6 +174,7 @@ asfd_status asfd_execute_stage(asfd_plan P, int stage, const float* u1_dev, floa
         const asfd_status s = plan_ensure_work(P, kWorkTransform);
         if (s != ASFD_OK) return s;
         if (stage == 0) return launch_spread(P, reinterpret_cast<const float2*>(u1_dev), st);
+        note_capture(P, st);  // (a row pass captured alone clears the band at its replays)
         if (stage == 1) return launch_fft_rows(P, st);
         return launch_fft_cols(P, reinterpret_cast<float2*>(u2_dev), st);
     });

@@ -314,6 +314,7 @@ asfd_status launch_fft_rows_band(asfd_plan_s* P, int ty0, int ty1, int tx0, int 
 #undef ASFD_ROWS
     if (e != cudaSuccess) return cuda_fail(e, "fft_rows_kernel launch");
     // the given band contains the plan's own band (a sum over several plans)
+    note_capture(P, st);
     P->band_clean = true;
     return ASFD_OK;
 }

@@ -237,17 +237,14 @@ asfd_status launch_spread(asfd_plan_s* P, const float2* u1, cudaStream_t st)
     if (tiles <= 0) return ASFD_OK;
     const bool colored = P->colored;
     const bool windowed = P->colored && P->windowed;
-    // the accumulating (dense) kernels need a zero band; the tile kernels
-    // overwrite every band cell
-    bool clear = !P->band_clean;
+    // the accumulating kernels (dense, fold, blk) need a zero band; the tile kernels
+    // overwrite every band cell.  The row pass leaves the band zero, but not for
+    // long where others write the grid without the plan's knowing -- a
+    // workspace's other plans, or replays of a captured call -- so there the band
+    // is cleared on every call (7.5 us at 2048^2, where a transform takes 123)
+    note_capture(P, st);
+    const bool clear = !P->band_clean || P->ws || P->captured;
     P->band_clean = false;
-    if (P->blk || P->fold) {
-        // these also clear a band that another writer may have used since the
-        // plan's own calls: a workspace's other plans, or replays of a graph
-        // (7.5 us at 2048^2, where a w = 12 transform takes 358)
-        note_capture(P, st);
-        clear = clear || P->ws || P->captured;
-    }
     if (P->itemtile) return launch_spread_itemtile(P, u1, st);
     if (P->blk) {
         if (clear) ASFD_CUDA(clear_band(a, tiles, st));
