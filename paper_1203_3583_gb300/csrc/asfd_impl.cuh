@@ -152,7 +152,7 @@ struct asfd_plan_s {
                                     // clears each cell it reads)
     bool captured = false;          // a call of the plan's was captured: its replays write
                                     // the grid without the plan's knowing
-    bool in_batch = false;          // the plan is a batch's own (its replays are the batch's)
+    bool own_capture = false;       // a batch is capturing the plan's calls for its own replays
     unsigned* status = nullptr;     // device status word
     float* stat = nullptr;          // a height map's statistics, per block
     // learned kernel (kind == ASFD_KERNEL_LEARNED)
@@ -237,7 +237,7 @@ cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, si
 // call does to the band happens at the replays, not now.
 inline void note_capture(asfd_plan_s* P, cudaStream_t st)
 {
-    if (P->captured || P->in_batch) return;
+    if (P->captured || P->own_capture) return;
     cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &s) != cudaSuccess) cudaGetLastError();
     else P->captured = s != cudaStreamCaptureStatusNone;

@@ -402,11 +402,14 @@ asfd_status streams_execute(asfd_batch_s* B, const float* const* u1, float* cons
     ASFD_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     asfd_status r = ASFD_OK;
     cudaGraph_t g = nullptr;
+    // (the batch's own replays leave the bands as its direct calls do)
+    for (asfd_plan_s* P : B->plans) P->own_capture = true;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         r = streams_enqueue(B, u1, u2, cap);
         e = cudaStreamEndCapture(cap, &g);
     }
+    for (asfd_plan_s* P : B->plans) P->own_capture = false;
     if (r == ASFD_OK && e == cudaSuccess && g) e = cudaGraphInstantiate(&B->sexec, g, 0);
     if (g) cudaGraphDestroy(g);
     cudaStreamDestroy(cap);
@@ -455,7 +458,6 @@ asfd_status asfd_batch_create(asfd_batch* out, const asfd_params* params,
             asfd_plan p = nullptr;
             asfd_status r = asfd_plan_create(&p, &params[i], d1_devs[i], stream);
             if (r != ASFD_OK) return r;
-            p->in_batch = true;
             B->plans.push_back(p);
             if (p->nfx > kBatchMaxNf || p->nfy > kBatchMaxNf) B->persistent_ok = false;
             // both schedules read the plans' work buffers
