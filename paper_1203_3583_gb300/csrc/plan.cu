@@ -672,9 +672,9 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
                                                     p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
     ASFD_CUDA(cudaGetLastError());
     std::vector<float> stats((size_t)sgx * sgy * kStatWords);
+    // (to pageable memory: the call returns when the copy has ended)
     ASFD_CUDA(cudaMemcpyAsync(stats.data(), P->stat, sizeof(float) * stats.size(), cudaMemcpyDeviceToHost,
                               st));
-    ASFD_CUDA(cudaStreamSynchronize(st));
     const auto value = [&](int k) {
         float m = stats[k];
         for (size_t b = k + kStatWords; b < stats.size(); b += kStatWords) m = std::max(m, stats[b]);
@@ -780,6 +780,9 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
         ASFD_CUDA(cudaStreamSynchronize(st));
         P->tile_pairs = (long long)lst.size();
     }
+    // the plan is ready on every stream when this returns (the copy of q has run
+    // while the host chose the launches)
+    ASFD_CUDA(cudaStreamSynchronize(st));
     if (P->learned && P->lfeat) {
         cs = learned_features(P, st);
         if (cs != ASFD_OK) return cs;
