@@ -139,8 +139,10 @@ asfd_status asfd_plan_create(asfd_plan* out, const asfd_params* p, const double*
                              void* stream);
 
 /* Replace the plan's height map (same sizes) and rebuild the d1-dependent
- * tables and binning.  Same errors as asfd_plan_create; the plan is unchanged
- * on failure. */
+ * tables and binning.  Synchronises `stream`: the new map is in place, for
+ * every stream, when the call returns.  Uses the plan's work buffers (not
+ * concurrent with other calls on the plan).  Same errors as asfd_plan_create;
+ * the plan is unchanged on failure. */
 asfd_status asfd_plan_update_d1(asfd_plan plan, const double* d1_dev, void* stream);
 
 /*
@@ -166,8 +168,8 @@ asfd_status asfd_plan_update_d1(asfd_plan plan, const double* d1_dev, void* stre
  * detaches the workspace; the plan then allocates its own work buffers again
  * on first use.  Without a workspace a plan allocates its work buffers at the
  * first call that needs them (asfd_execute, asfd_execute_stage,
- * asfd_execute_host, asfd_adjoint, the learned training calls, and
- * asfd_multi_execute for its first plan): make one such call, or set a
+ * asfd_execute_host, asfd_adjoint, the learned training calls,
+ * asfd_plan_update_d1, and asfd_multi_execute for its first plan): make one such call, or set a
  * workspace, before capturing calls into a CUDA graph.  Synchronises the
  * device (work queued on the old buffers must finish).  Several plans may
  * share one workspace only if their calls never overlap in time.

@@ -92,7 +92,7 @@ struct asfd_plan_s {
     double* bux = nullptr;          // unreduced alpha x~ + nf/2 per axis (plan only)
     double* buy = nullptr;
     float* q = nullptr;             // [n1y][n1x]  d1 / (z0 - d1)
-    float* q_next = nullptr;        // [n1y][n1x]  the same of a height map being checked
+    float* q_next = nullptr;        // [n1y][n1x]  the same of a height map being checked (on need)
     float2* cx = nullptr;           // [m2x] destination chirp * (-1)^m' / psi_hat
     float2* cy = nullptr;           // [m2y] same, times the global factor
     float2* twx = nullptr;          // [nfx] e^{-2 pi i k/nfx}
@@ -298,7 +298,8 @@ asfd_status direct_sum(const asfd_params* p, const double* d1, const float2* u1,
 asfd_status plan_alloc(asfd_plan_s* P);
 asfd_status build_twiddles(float2* tw, int L, cudaStream_t st);
 asfd_status plan_build_tables(asfd_plan_s* P, cudaStream_t st);
-asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st);
+// (fresh: the plan is being created)
+asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStream_t st);
 asfd_status plan_alloc_buffer(asfd_plan_s* P, void** p, size_t bytes);
 
 // Work buffers (sizes scale with the grids; everything else a plan holds is

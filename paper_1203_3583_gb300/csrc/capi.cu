@@ -119,7 +119,7 @@ asfd_status asfd_plan_create(asfd_plan* out, const asfd_params* p, const double*
         if (r != ASFD_OK) return r;
         r = plan_build_tables(P, st);
         if (r != ASFD_OK) return r;
-        r = plan_build_d1(P, d1_dev, st);
+        r = plan_build_d1(P, d1_dev, true, st);
         if (r != ASFD_OK) return r;
         if (p->kind == ASFD_KERNEL_LEARNED) {
             P->learned = true;
@@ -141,7 +141,7 @@ asfd_status asfd_plan_update_d1(asfd_plan P, const double* d1_dev, void* stream)
     clear_error();
     if (!P || !d1_dev) return fail(ASFD_ERR_ARG, "plan or d1 is NULL");
     return on_device(P->device, [&] {
-        return plan_build_d1(P, d1_dev, static_cast<cudaStream_t>(stream));
+        return plan_build_d1(P, d1_dev, false, static_cast<cudaStream_t>(stream));
     });
 }
 

@@ -107,10 +107,10 @@ constexpr int kStatRows = 64;       // rows whose coordinates it stages at a tim
 // above.  A thread takes a column over a chunk of rows: its x extremes are
 // those of q, mapped, as the coordinate is monotone in q; the spacing takes the
 // FP64 difference of neighbouring base coordinates and FP32 q terms (~1 cell,
-// good to ~1e-6 cells; the binning adds a one-cell margin).  q goes to a buffer
-// of its own, so that a rejected map changes nothing.  (Four kernels with three
-// waits for their results, and loops over 4096 source tiles on the host, left
-// the GPU idle for 0.2 of a 0.41 ms optimisation step at 1024^2.)
+// good to ~1e-6 cells; the binning adds a one-cell margin).  An update's q
+// goes beside the plan's, so that a rejected map changes nothing.  (Four kernels
+// with three waits for their results, and loops over 4096 source tiles on the
+// host, left the GPU idle for 0.2 of a 0.41 ms optimisation step at 1024^2.)
 __global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* q,
                                                        const AxisEntry* ax, const AxisEntry* ay,
                                                        const double* bux, const double* buy,
@@ -495,7 +495,6 @@ asfd_status plan_alloc(asfd_plan_s* P)
     A(bux, p.n1x);
     A(buy, p.n1y);
     A(q, nsrc);
-    A(q_next, nsrc);
     A(cx, p.m2x);
     A(cy, p.m2y);
     A(twx, P->nfx);
@@ -658,17 +657,37 @@ asfd_status plan_build_tables(asfd_plan_s* P, cudaStream_t st)
     return ASFD_OK;
 }
 
-asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
+asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStream_t st)
 {
     const asfd_params& p = P->prm;
     const size_t nsrc = (size_t)p.n1x * p.n1y;
+    // where q of the new map waits to be accepted: in place for a new plan (which
+    // is given up with its map), else in a work buffer, which lies idle between
+    // calls; where none is large enough in a buffer of the plan's own
+    float* q_next = P->q;
+    if (!fresh) {
+        const size_t bytes = sizeof(float) * nsrc;
+        const size_t rows = sizeof(float2) * (size_t)P->nfy * row_buffer_width(p.m2x);
+        const size_t grid = sizeof(float2) * (size_t)P->nfx * P->nfy;
+        asfd_status s = ASFD_OK;
+        if (P->ws) {
+            q_next = reinterpret_cast<float*>(P->stage_u1);  // 8 bytes per sample
+        } else if (bytes <= std::max(rows, grid)) {
+            s = plan_ensure_work(P, kWorkTransform);
+            q_next = reinterpret_cast<float*>(bytes <= rows ? P->rows : P->grid);
+        } else {
+            if (!P->q_next) s = alloc_n(P, &P->q_next, nsrc);
+            q_next = P->q_next;
+        }
+        if (s != ASFD_OK) return s;
+    }
     // the band may move: its new cells were never cleared
     P->band_clean = false;
     // 1. one pass over d1: checks, q (beside the plan's), extremes and spacings
     static_assert((65536 + kStatCols - 1) / kStatCols <= kStatBlocks, "n1x <= 65536 fits one row of blocks");
     const int sgx = (p.n1x + kStatCols - 1) / kStatCols;
     const int sgy = std::max(1, std::min(kStatBlocks / sgx, p.n1y));
-    d1_stats_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(d1, P->q_next, P->ax, P->ay, P->bux, P->buy, p.n1x,
+    d1_stats_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(d1, q_next, P->ax, P->ay, P->bux, P->buy, p.n1x,
                                                     p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
     ASFD_CUDA(cudaGetLastError());
     std::vector<float> stats((size_t)sgx * sgy * kStatWords);
@@ -689,7 +708,8 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, cudaStream_t st)
         return fail(ASFD_ERR_UNSUPPORTED, "max |d1|/z0 = " + std::to_string(me) +
                                               " exceeds the supported 0.1");
     // (copied, not swapped: captured launches hold the plan's pointer)
-    ASFD_CUDA(cudaMemcpyAsync(P->q, P->q_next, sizeof(float) * nsrc, cudaMemcpyDeviceToDevice, st));
+    if (q_next != P->q)
+        ASFD_CUDA(cudaMemcpyAsync(P->q, q_next, sizeof(float) * nsrc, cudaMemcpyDeviceToDevice, st));
 
     // 2. the band (fine-grid tiles that footprints reach) and the wrap flags
     const double hw = 0.5 * P->w + 1.0;  // half width plus a one-cell safety margin
