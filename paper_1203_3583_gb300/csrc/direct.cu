@@ -23,7 +23,8 @@
 // bits of 5.1e-8 instead of 6.2e-8.)
 //   Eq. 2: 2 (s.x1 + sz d1 + r)/lambda half-turns, amplitude 1/r^2,
 //          r = |(x2 - x1, z0 - d1)|, in FP64 from an FP32 reciprocal square
-//          root and one Newton step (relative error below 2^-44).
+//          root and its residual to third order (as good as an FP64 square
+//          root, which is slow here: r counts up to 1e8 half-turns and more).
 // The high 32 bits of the phase go to an FP32 sine and cosine on a quarter
 // turn (polynomials, |error| < 6e-8); products with u1 are FP32 and the sums
 // of a thread are carried as an FP32 value and its exact rounding errors
@@ -33,6 +34,7 @@
 #include <algorithm>
 #include <cmath>
 #include <string>
+#include <type_traits>
 
 #include "asfd_impl.cuh"
 #include "fft.cuh"
@@ -246,23 +248,36 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
         }
     }
     // phase (2^-32 turns) and amplitude of the sample's terms t at point j
-    auto phase = [&](const ulonglong2& t0, const ulonglong2& t1, int j, float& amp) -> unsigned {
+    // (exact: with FP64 square root and reciprocal, for a thread's second pass)
+    auto phase = [&](auto exact, const ulonglong2& t0, const ulonglong2& t1, int j, float& amp) -> unsigned {
         if constexpr (FORM == kEq2) {
             const double dx = x2x[j] - __longlong_as_double((long long)t0.x);
             const double dy = x2y[j] - __longlong_as_double((long long)t0.y);
             const double r2 = fma(dx, dx, fma(dy, dy, __longlong_as_double((long long)t1.x)));
-            const float r2f = (float)r2;
-            // (a sample on the point itself: r = 0, amplitude infinite)
-            const float y = rsqrtf(fmaxf(r2f, 1e-37f));
-            const double yd = (double)y;
-            const double ra = r2 * yd;  // r to 2^-22; one Newton step
-            const double r = fma(0.5 * yd, fma(-ra, ra, r2), ra);
+            double r;
+            if constexpr (exact.value) {
+                r = sqrt(r2);
+                amp = (float)(1.0 / r2);
+            } else {
+                const float r2f = (float)r2;
+                // with y = (1 + e)/r: ra = r2 y = r (1 + e), the residual r2 - ra^2 =
+                // -(2e + e^2) r2, and r = ra + c + (3/4) t c up to e^3, with c =
+                // residual y/2 and t = residual y^2 = -2e, for which FP32 is enough
+                const float y = rsqrtf(r2f);
+                const double yd = (double)y, ra = r2 * yd, res = fma(-ra, ra, r2);
+                const double c = 0.5 * yd * res;
+                const float t = y * ((float)res * y);
+                r = ra + fma(c, (double)(0.75f * t), c);
+                // 1/r^2 = y^2 (1 + t) up to t^2, y^2 with its rounding error
+                const float a0 = y * y;
+                amp = a0 + fmaf(a0, t, fmaf(y, y, -a0));
+                // (out of FP32's range: a NaN sends the thread to its second pass)
+                if (!(r2f > 1e-24f && r2f < 1e30f)) amp = __int_as_float(0x7fc00000);
+            }
             double h = fma(2.0 * g.inv_lambda, r, __longlong_as_double((long long)t1.y));
             h -= 2.0 * rint(0.5 * h);
-            // 1/r^2 from its FP32 estimate and that one's residual in FP64
-            const float a0 = y * y;
-            amp = r2f == 0.f ? __int_as_float(0x7f800000)
-                             : fmaf(a0, (float)fma(-r2, (double)a0, 1.0), a0);
+            if constexpr (exact.value)
+                if (!isfinite(h)) amp = __int_as_float(0x7fc00000);  // (no such phase)
             // units of 2^-31 half-turns from the low bits of h + 1.5 2^21
             return (unsigned)__double_as_longlong(h + 3145728.0);
         } else {
@@ -275,10 +290,10 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
         }
     };
     // products u exp(2 pi i phase) amp of points j and j + 1
-    auto products = [&](const ulonglong2& t0, const ulonglong2& t1, float2 u, int j, float2& re,
-                        float2& im) {
+    auto products = [&](auto exact, const ulonglong2& t0, const ulonglong2& t1, float2 u, int j,
+                        float2& re, float2& im) {
         float2 amp = pair2(1.f), sn, cs;
-        const unsigned pa = phase(t0, t1, j, amp.x), pb = phase(t0, t1, j + 1, amp.y);
+        const unsigned pa = phase(exact, t0, t1, j, amp.x), pb = phase(exact, t0, t1, j + 1, amp.y);
         turn_sincos2(pa, pb, sn, cs);
         float2 ux = pair2(u.x), uy = pair2(u.y);
         if constexpr (FORM == kEq2) {
@@ -306,7 +321,7 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
 #pragma unroll
             for (int k = 0; k < P / 2; ++k) {
                 float2 re, im;
-                products(t0, t1, u, 2 * k, re, im);
+                products(std::false_type{}, t0, t1, u, 2 * k, re, im);
                 kahan_add(sr[k], lr[k], re);
                 kahan_add(si[k], li[k], im);
             }
@@ -316,13 +331,14 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
         for (int k = 0; k < P / 2; ++k) {
             double v[4] = {(double)sr[k].x - lr[k].x, (double)si[k].x - li[k].x,
                            (double)sr[k].y - lr[k].y, (double)si[k].y - li[k].y};
-            // overflow of an FP32 sum (or infinite fields): the sums in FP64
+            // overflow of an FP32 sum, infinite fields, distances out of FP32's
+            // range: the sums in FP64
             if (!(isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]) && isfinite(v[3]))) {
                 v[0] = v[1] = v[2] = v[3] = 0.0;
                 for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
                     const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
                     float2 re, im;
-                    products(__ldg(tp), __ldg(tp + 1), __ldg(&u1[n]), 2 * k, re, im);
+                    products(std::true_type{}, __ldg(tp), __ldg(tp + 1), __ldg(&u1[n]), 2 * k, re, im);
                     v[0] += re.x;
                     v[1] += im.x;
                     v[2] += re.y;
