@@ -756,7 +756,9 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
         auto leave = [&](int b) {  // (DUP: the rows have left above)
             if constexpr (!DUP) flush_row(b);
         };
-        const float2 c = sample_value_fast(u, ex, ey, q, a.inc_d);
+        // (wrapping and folding maps have the accurate sine and cosine)
+        const float2 c = WRAP ? sample_value(u, ex, ey, q, a.inc_d)
+                              : sample_value_fast(u, ex, ey, q, a.inc_d);
         if constexpr (TAB) {
             if (ny / kSrcTile != tab_ty) {  // warp-uniform: every lane is on row ny
                 tab_ty = ny / kSrcTile;

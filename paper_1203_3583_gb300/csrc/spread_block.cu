@@ -129,6 +129,9 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
 {
     constexpr int S = blk_split(W), WS = blk_cols(W), HC = 32 / S;
     constexpr unsigned full = 0xffffffffu;
+    // prefactors with the accurate sine and cosine: the widths asked for where the
+    // last digits matter, and the maps of many samples per kernel width
+    constexpr bool ACCURATE = DUP || W > kMaxRingWidth;
     extern __shared__ float4 blk_smem[];
     chain_next();
     chain_wait();
@@ -291,7 +294,8 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
                 live = true;
             }
             R0 = l0y;
-            const float2 c = sample_value_fast(u, ex, ey, q, a.inc_d);
+            const float2 c = ACCURATE ? sample_value(u, ex, ey, q, a.inc_d)
+                                      : sample_value_fast(u, ex, ey, q, a.inc_d);
             blk_accumulate<W, WS>(acc, fresh, d, c, wy, wx);
         }
         flush(live ? W : 0, W);
@@ -401,7 +405,7 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_fold_kernel(SpreadArg
         X0 = l0x;
         R0 = l0y;
         live = true;
-        const float2 c = sample_value_fast(u, ex, ey, q, a.inc_d);
+        const float2 c = sample_value(u, ex, ey, q, a.inc_d);
         float e[W + WS + 1];
         const float zy = dy - a.half_w, zx = dx - a.half_w + (float)(sub * WS);
 #pragma unroll
@@ -484,7 +488,9 @@ asfd_status plan_build_block(asfd_plan_s* P, const std::vector<double>& cr,
     int dev = 0, sms = 0;
     ASFD_CUDA(cudaGetDevice(&dev));
     ASFD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const bool dup = P->min_step_x < 1.0 + 1e-3;
+    // (beyond 64 samples per kernel width: see ACCURATE)
+    const bool dup = P->min_step_x < 1.0 + 1e-3 || w + 0.01 > 64.0 * P->min_step_x ||
+                     w + P->row_spread_y + 0.01 > 64.0 * P->min_step_y;
     const BlkKernel kern = dup ? blk_kernel<true>(w) : blk_kernel<false>(w);
     if (!kern) return ASFD_OK;
     // (process-wide, the same value for every plan)
