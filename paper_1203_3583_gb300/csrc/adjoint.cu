@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(32 * kInterpWarps) interp_kernel(InterpArgs a,
         if (r >= ny1) return;
         const size_t i = (size_t)r * a.n1x + nx;
         qn = __ldg(&a.q[i]);
-        if (a.gd1) un = __ldg(&a.u1[i]);
+        if (a.gd1) un = a.u1[i];
         eyn = a.ay[r];
         pyn = a.py[r];
     };
@@ -173,8 +173,8 @@ __global__ void __launch_bounds__(32 * kInterpWarps) interp_kernel(InterpArgs a,
             float2 s0 = make_float2(0.f, 0.f), sd = s0;
 #pragma unroll
             for (int j = 0; j < NX; j += 2) {
-                const float4 v = WRAP ? __ldg(reinterpret_cast<const float4*>(g + ((c0 + j) & mx)))
-                                      : __ldg(reinterpret_cast<const float4*>(g + c0) + j / 2);
+                const float4 v = WRAP ? *reinterpret_cast<const float4*>(g + ((c0 + j) & mx))
+                                      : reinterpret_cast<const float4*>(g + c0)[j / 2];
                 const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
                 s0 = fma2(v0, wx[j], s0);
                 sd = fma2(v0, dwx[j], sd);

@@ -172,7 +172,7 @@ struct asfd_plan_s {
     float* lcgrad = nullptr;        // [m2x + m2y] dL/dcorrection
     float2* lu2 = nullptr;          // [m2y][m2x] training forward output (work buffer)
     float2* lres = nullptr;         // [m2y][m2x] loss gradient (work buffer)
-    double* lred = nullptr;         // [2] loss reductions
+    double* lred = nullptr;         // [2] loss reductions, and a word that learned_refresh clears
     float* lpart = nullptr;         // per-block sums of the table and MLP gradients
     float2* stage_u1 = nullptr;     // staging for asfd_execute_host (work buffer)
     float2* stage_u2 = nullptr;

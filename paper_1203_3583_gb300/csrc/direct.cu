@@ -95,8 +95,7 @@ __device__ __forceinline__ bool not_finite(double v)
 }
 
 __global__ void __launch_bounds__(256)
-direct_prep_kernel(DirectGeom g, const double* __restrict__ d1, int form,
-                   DirectTerms* __restrict__ out, unsigned* __restrict__ bad)
+direct_prep_kernel(DirectGeom g, const double* d1, int form, DirectTerms* out, unsigned* bad)
 {
     __shared__ double ys[kPrepRows];
     chain_next();
@@ -212,9 +211,8 @@ __host__ __device__ constexpr int direct_blocks_per_sm(int form)
 // so the samples are split as well.
 template <DirectForm FORM>
 __global__ void __launch_bounds__(kDirectThreads, direct_blocks_per_sm(FORM))
-direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2* __restrict__ u1,
-                  int npts, const int* __restrict__ mx, const int* __restrict__ my, size_t chunk,
-                  double2* __restrict__ part)
+direct_sum_kernel(DirectGeom g, const DirectTerms* s, const float2* u1, int npts, const int* mx,
+                  const int* my, size_t chunk, double2* part)
 {
     constexpr int P = kDirectPoints;
     static_assert(P % 2 == 0 && P <= 32, "points in pairs, a lane each for the sums");
@@ -316,8 +314,8 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
         for (int k = 0; k < P / 2; ++k) sr[k] = lr[k] = si[k] = li[k] = pair2(0.f);
         for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
             const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
-            const ulonglong2 t0 = __ldg(tp), t1 = __ldg(tp + 1);
-            const float2 u = __ldg(&u1[n]);
+            const ulonglong2 t0 = tp[0], t1 = tp[1];
+            const float2 u = u1[n];
 #pragma unroll
             for (int k = 0; k < P / 2; ++k) {
                 float2 re, im;
@@ -338,7 +336,7 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
                 for (size_t n = b0 + threadIdx.x; n < b1; n += kDirectThreads) {
                     const ulonglong2* tp = reinterpret_cast<const ulonglong2*>(s + n);
                     float2 re, im;
-                    products(std::true_type{}, __ldg(tp), __ldg(tp + 1), __ldg(&u1[n]), 2 * k, re, im);
+                    products(std::true_type{}, tp[0], tp[1], u1[n], 2 * k, re, im);
                     v[0] += re.x;
                     v[1] += im.x;
                     v[2] += re.y;
@@ -382,10 +380,8 @@ direct_sum_kernel(DirectGeom g, const DirectTerms* __restrict__ s, const float2*
 }
 
 // The chunks' sums in order, times the outer factor: a warp per point.
-__global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int* __restrict__ mx,
-                                     const int* __restrict__ my, int chunks,
-                                     const double2* __restrict__ part,
-                                     const unsigned* __restrict__ bad, float2* __restrict__ out)
+__global__ void direct_finish_kernel(DirectGeom g, int form, int npts, const int* mx, const int* my,
+                                     int chunks, const double2* part, const unsigned* bad, float2* out)
 {
     chain_next();
     chain_wait();

@@ -46,8 +46,8 @@ fft_cols_kernel(ColArgs a)
 // e^{+i} along y, band rows [row0, row0 + nrows) stored to rows[s - row0][kx].
 template <int L>
 __global__ void __launch_bounds__(ColCfg<L>::THREADS, ColCfgSel<L>::MIN_BLOCKS)
-fft_cols_adj_kernel(const float2* __restrict__ g, int m2x, int m2y, const float2* __restrict__ cx,
-                    const float2* __restrict__ cy, float2* __restrict__ rows, int row0, int nrows,
+fft_cols_adj_kernel(const float2* g, int m2x, int m2y, const float2* cx, const float2* cy,
+                    float2* rows, int row0, int nrows,
                     const float2* __restrict__ tw)
 {
     using C = ColCfg<L>;
@@ -58,15 +58,15 @@ fft_cols_adj_kernel(const float2* __restrict__ g, int m2x, int m2y, const float2
     const int col = blockIdx.x * C::LPC + c;
     const bool active = col < m2x;
     const int colc = active ? col : 0;
-    const float2 fx = __ldg(&cx[colc]);
+    const float2 fx = cx[colc];
     const int half = m2y / 2;
     auto bin = [&](int i) { return i < half ? i + half : i - (L - half); };
     auto kept = [&](int i) { return active && (i < half || i >= L - half); };
     auto ld = [&](int i) -> float2 {
-        return kept(i) ? __ldg(&g[(size_t)bin(i) * m2x + colc]) : make_float2(0.f, 0.f);
+        return kept(i) ? g[(size_t)bin(i) * m2x + colc] : make_float2(0.f, 0.f);
     };
     auto scale = [&](int i, float2 v) -> float2 {  // conj(fx * cy[k]) * g
-        const float2 f = kept(i) ? __ldg(&cy[bin(i)]) : make_float2(0.f, 0.f);
+        const float2 f = kept(i) ? cy[bin(i)] : make_float2(0.f, 0.f);
         return cmulc(cmulc(v, fx), f);
     };
     auto st = [&](int i, float2 v) {
@@ -80,7 +80,7 @@ fft_cols_adj_kernel(const float2* __restrict__ g, int m2x, int m2y, const float2
 // e^{+i} along x, band columns [col_lo, col_hi) stored to the fine grid.
 template <int L>
 __global__ void __launch_bounds__(RowCfg<L>::THREADS, L == 4096 ? 4 : 1)
-fft_rows_adj_kernel(const float2* __restrict__ rows, int nrows, int m2x, float2* __restrict__ grid,
+fft_rows_adj_kernel(const float2* rows, int nrows, int m2x, float2* grid,
                     int row0, int col_lo, int col_hi, const float2* __restrict__ tw)
 {
     using C = RowCfg<L>;
@@ -95,7 +95,7 @@ fft_rows_adj_kernel(const float2* __restrict__ rows, int nrows, int m2x, float2*
     const int half = m2x / 2;
     auto ld = [&](int i) -> float2 {
         const bool kept = active && (i < half || i >= L - half);
-        return kept ? __ldg(&src[i < half ? i + half : i - (L - half)]) : make_float2(0.f, 0.f);
+        return kept ? src[i < half ? i + half : i - (L - half)] : make_float2(0.f, 0.f);
     };
     auto st = [&](int i, float2 v) {
         if (active && i >= col_lo && i < col_hi) dst[i] = v;

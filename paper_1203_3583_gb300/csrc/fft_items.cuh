@@ -76,7 +76,7 @@ struct ColArgs {
     int row0, nrows;
     int m2x, m2y;
     int col0, col1;      // kept columns [col0, col1) this pass transforms
-    const float2* cx;    // [m2x] deconvolution x chirp
+    const float2* cx;    // [m2x] deconvolution x chirp (complete before the call's first kernel starts)
     const float2* cy;    // [m2y] same, times the global factor
     float2* u2;          // [m2y][m2x]
     const float2* tw;
@@ -142,7 +142,7 @@ __device__ __forceinline__ void cols_body(const ColArgs& a, int blk, float2* sm,
     const float2* rows = a.rows;
     auto ld = [&](int i) -> float2 {
         const int rr = i - row0;
-        return (active && rr >= 0 && rr < nrows) ? __ldg(&rows[row_group_index(rr, colc, nrows)])
+        return (active && rr >= 0 && rr < nrows) ? rows[row_group_index(rr, colc, nrows)]
                                                  : make_float2(0.f, 0.f);
     };
     auto st = [&](int i, float2 v) {

@@ -100,10 +100,8 @@ __global__ void __launch_bounds__(256) features_kernel(const float* q, const Axi
 // lane: 121 us for 16384 tiles; see learned_gradient.)
 constexpr int kMlpTiles = 32;
 
-__global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restrict__ prm,
-                                                          const float* __restrict__ feat, int ntiles,
-                                                          float* __restrict__ hid,
-                                                          float* __restrict__ tab)
+__global__ void __launch_bounds__(256) mlp_forward_kernel(const float* prm, const float* feat,
+                                                          int ntiles, float* hid, float* tab)
 {
     constexpr int O = kLearnTableSize, H = kLearnHidden, F = kLearnFeat, T = kMlpTiles;
     static_assert(O == 64 && H % 4 == 0, "four tiles at a time in 256 threads");
@@ -117,7 +115,7 @@ __global__ void __launch_bounds__(256) mlp_forward_kernel(const float* __restric
     const int o = tid % O;
     float w2[H];
 #pragma unroll
-    for (int i = 0; i < H; ++i) w2[i] = __ldg(&prm[kLpW2 + o * H + i]);
+    for (int i = 0; i < H; ++i) w2[i] = prm[kLpW2 + o * H + i];
     const float b2 = prm[kLpB2 + o], base = prm[kLpBase + o];
     __syncthreads();
     for (int i = tid; i < nt * H; i += 256) {
@@ -159,8 +157,8 @@ __device__ __forceinline__ void cheb_even(float u, float (&T)[kLearnCheb])
     }
 }
 
-__global__ void deconv_build_kernel(const float* __restrict__ prm, const float2* __restrict__ cb,
-                                    float2* __restrict__ c, float* __restrict__ corr, int m, int off)
+__global__ void deconv_build_kernel(const float* prm, const float2* cb, float2* c, float* corr, int m,
+                                    int off)
 {
     chain_next();
     chain_wait();
@@ -224,9 +222,8 @@ __device__ __forceinline__ void block_add(double v, double* part, double* out)
 // squares are carried as FP32 values with their exact rounding errors: FP64
 // sums over 4.2 M points are bound by the FP64 pipe (this and the squared
 // error together took 116 us).
-__global__ void __launch_bounds__(256) ref_norm_kernel(const float2* __restrict__ ref, size_t n,
-                                                       double* red, float* __restrict__ gcorr,
-                                                       int ncorr)
+__global__ void __launch_bounds__(256) ref_norm_kernel(const float2* ref, size_t n, double* red,
+                                                       float* gcorr, int ncorr)
 {
     chain_next();
     chain_wait();
@@ -236,12 +233,12 @@ __global__ void __launch_bounds__(256) ref_norm_kernel(const float2* __restrict_
     float2 sum = make_float2(0.f, 0.f), err = sum;
 #pragma unroll 8
     for (size_t i = i0; i < n; i += step)
-        add_square2(sum, err, __ldg(&ref[i]), make_float2(0.f, 0.f));
+        add_square2(sum, err, ref[i], make_float2(0.f, 0.f));
     double v = ((double)sum.x + (double)sum.y) + ((double)err.x + (double)err.y);
     if (!squares_in_range(sum)) {
         v = 0.0;
         for (size_t i = i0; i < n; i += step) {
-            const float2 b = __ldg(&ref[i]);
+            const float2 b = ref[i];
             v += (double)b.x * b.x + (double)b.y * b.y;
         }
     }
@@ -258,9 +255,8 @@ __global__ void __launch_bounds__(256) ref_norm_kernel(const float2* __restrict_
 constexpr int kLossCols = 128, kLossRows = 32;
 
 __global__ void __launch_bounds__(256)
-loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
-            const float* __restrict__ corr, int m2x, int m2y, double* red, float2* __restrict__ g,
-            float* __restrict__ gcorr)
+loss_kernel(const float2* u2, const float2* ref, const float* corr, int m2x, int m2y, double* red,
+            float2* g, float* gcorr)
 {
     chain_next();
     chain_wait();
@@ -275,11 +271,18 @@ loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
     for (int y = blockIdx.y * kLossRows + warp; y < y1; y += 8) {
         const size_t row = (size_t)y * m2x;
         float across = 0.f;
+        float2 us[kLossCols / 32], rs[kLossCols / 32];  // all loads before the first store
+#pragma unroll
+        for (int j = 0; j < kLossCols / 32; ++j) {
+            const int c = c0 + 32 * j;
+            us[j] = c < m2x ? u2[row + c] : make_float2(0.f, 0.f);
+            rs[j] = c < m2x ? ref[row + c] : make_float2(0.f, 0.f);
+        }
 #pragma unroll
         for (int j = 0; j < kLossCols / 32; ++j) {
             const int c = c0 + 32 * j;
             if (c < m2x) {
-                const float2 a = __ldg(&u2[row + c]), b = __ldg(&ref[row + c]);
+                const float2 a = us[j], b = rs[j];
                 // a - b = d + e exactly
                 const float2 d = csub(a, b), z = csub(d, a);
                 const float2 e = csub(csub(a, csub(d, z)), cadd(b, z));
@@ -302,7 +305,7 @@ loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
         e2 = 0.0;
         for (int y = blockIdx.y * kLossRows + warp; y < y1; y += 8)
             for (int c = c0; c < min(m2x, (int)(blockIdx.x + 1) * kLossCols); c += 32) {
-                const float2 a = __ldg(&u2[(size_t)y * m2x + c]), b = __ldg(&ref[(size_t)y * m2x + c]);
+                const float2 a = u2[(size_t)y * m2x + c], b = ref[(size_t)y * m2x + c];
                 const double dx = (double)a.x - b.x, dy = (double)a.y - b.y;
                 e2 += dx * dx + dy * dy;
             }
@@ -318,8 +321,8 @@ loss_kernel(const float2* __restrict__ u2, const float2* __restrict__ ref,
 }
 
 // dL/dd_j = sum_k dL/dcorr[k] T_2j(u_k): block 0 the x axis, block 1 the y axis
-__global__ void __launch_bounds__(1024) cheb_grad_kernel(const float* __restrict__ gcorr, int m2x,
-                                                         int m2y, float* __restrict__ grad)
+__global__ void __launch_bounds__(1024) cheb_grad_kernel(const float* gcorr, int m2x, int m2y,
+                                                         float* grad)
 {
     chain_next();
     chain_wait();
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int
     // the tile's polynomials as (x, y) coefficient pairs
 #pragma unroll
     for (int e = lane; e < 2 * W * K; e += 32)
-        tsm[wid][2 * (e % (W * K)) + e / (W * K)] = __ldg(&a.tab[(size_t)t * kLearnTableSize + e]);
+        tsm[wid][2 * (e % (W * K)) + e / (W * K)] = a.tab[(size_t)t * kLearnTableSize + e];
     __syncwarp();
     const int nx = (t % a.nstx) * kSrcTile + (lane & 15);
     const int ny0 = (t / a.nstx) * kSrcTile + (lane >> 4) * (kSrcTile / 2);
@@ -406,7 +409,7 @@ __global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int
             const int ny = ny0 + r + 1;
             const size_t n = (size_t)ny * a.n1x + nx;
             next.q = __ldg(&a.q[n]);
-            next.u = __ldg(&a.u1[n]);
+            next.u = a.u1[n];
             next.ey = a.ay[ny];
             next.py = a.py[ny];
         }
@@ -419,7 +422,7 @@ __global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int
             for (int b = 0; b < W; ++b) {
                 const float2* row = a.grid + (size_t)((l0y + b) & my) * a.nfx;
 #pragma unroll
-                for (int i = 0; i < W; ++i) B[b][i] = __ldg(&row[(l0x + i) & mx]);
+                for (int i = 0; i < W; ++i) B[b][i] = row[(l0x + i) & mx];
             }
         } else {
             // (clamped all the same: every address stays inside the grid)
@@ -428,7 +431,7 @@ __global__ void __launch_bounds__(32 * kTgWarps) table_grad_kernel(TGArgs a, int
 #pragma unroll
             for (int b = 0; b < W; ++b)
 #pragma unroll
-                for (int i = 0; i < W; ++i) B[b][i] = __ldg(cell + (size_t)b * a.nfx + i);
+                for (int i = 0; i < W; ++i) B[b][i] = cell[(size_t)b * a.nfx + i];
         }
         const float2 c = sample_value_fast(s, a.inc_d);
         float wx[W], wy[W];
@@ -493,11 +496,9 @@ constexpr int kBackTiles = 8;
 constexpr int kBackBlocks = 304;      // two per SM
 constexpr int kMlpParams = kLpDx;     // table and MLP parameters come first
 
-__global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restrict__ prm,
-                                                           const float* __restrict__ feat,
-                                                           const float* __restrict__ hid,
-                                                           const float* __restrict__ tgrad, int ntiles,
-                                                           float* __restrict__ part)
+__global__ void __launch_bounds__(256) mlp_backward_kernel(const float* prm, const float* feat,
+                                                           const float* hid, const float* tgrad,
+                                                           int ntiles, float* part)
 {
     constexpr int O = kLearnTableSize, H = kLearnHidden, F = kLearnFeat, T = kBackTiles;
     static_assert(T * H == 256 && T * O == 512 && O * H == 8 * 256 && H * F <= 256,
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
     const int tt = tid / H, ti = tid % H;       // its hidden gradient
     float w2[O];
 #pragma unroll
-    for (int k = 0; k < O; ++k) w2[k] = __ldg(&prm[kLpW2 + k * H + ti]);
+    for (int k = 0; k < O; ++k) w2[k] = prm[kLpW2 + k * H + ti];
     float gw2[8], gw1 = 0.f, gb1 = 0.f, gbase = 0.f;
 #pragma unroll
     for (int i = 0; i < 8; ++i) gw2[i] = 0.f;
@@ -521,10 +522,10 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
     float n0, n1, nh, nf;
     auto fetch = [&](int t0) {
         const int nt = min(T, ntiles - t0);
-        n0 = tid < nt * O ? __ldg(&tgrad[(size_t)t0 * O + tid]) : 0.f;
-        n1 = tid + 256 < nt * O ? __ldg(&tgrad[(size_t)t0 * O + tid + 256]) : 0.f;
-        nh = tid < nt * H ? __ldg(&hid[(size_t)t0 * H + tid]) : 0.f;
-        nf = tid < nt * F ? __ldg(&feat[(size_t)t0 * F + tid]) : 0.f;
+        n0 = tid < nt * O ? tgrad[(size_t)t0 * O + tid] : 0.f;
+        n1 = tid + 256 < nt * O ? tgrad[(size_t)t0 * O + tid + 256] : 0.f;
+        nh = tid < nt * H ? hid[(size_t)t0 * H + tid] : 0.f;
+        nf = tid < nt * F ? feat[(size_t)t0 * F + tid] : 0.f;
     };
     fetch(blockIdx.x * T);
     for (int t0 = blockIdx.x * T; t0 < ntiles; t0 += gridDim.x * T) {
@@ -590,8 +591,7 @@ __global__ void __launch_bounds__(256) mlp_backward_kernel(const float* __restri
 
 // The blocks' sums, added in order: a thread per parameter and eighth of the
 // blocks.
-__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict__ part, int blocks,
-                                                         float* __restrict__ grad)
+__global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* part, int blocks, float* grad)
 {
     __shared__ float red[8][32];
     chain_next();
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict
     float v = 0.f;
     if (i < kMlpParams) {
 #pragma unroll 8
-        for (int b = wid; b < blocks; b += 8) v += __ldg(&part[(size_t)b * kMlpParams + i]);
+        for (int b = wid; b < blocks; b += 8) v += part[(size_t)b * kMlpParams + i];
     }
     red[wid][lane] = v;
     __syncthreads();
@@ -612,8 +612,7 @@ __global__ void __launch_bounds__(256) mlp_reduce_kernel(const float* __restrict
 }
 
 
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float c1,
+__global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float c1,
                             float c2, float eps)
 {
     chain_next();
@@ -703,6 +702,9 @@ asfd_status learned_refresh(asfd_plan_s* P, cudaStream_t st)
                              (const float2*)P->cxb, P->cx, P->lcorr, m2x, kLpDx));
     ASFD_CUDA(launch_chained(deconv_build_kernel, dim3((m2y + 255) / 256), 256, 0, st, F(P->lparams),
                              (const float2*)P->cyb, P->cy, P->lcorr + m2x, m2y, kLpDy));
+    // no kernel queued after this starts before the tables are complete (it would
+    // before a chained launch): the column pass reads cx and cy as constants
+    ASFD_CUDA(cudaMemsetAsync(P->lred + 2, 0, sizeof(double), st));
     return ASFD_OK;
 }
 
@@ -725,7 +727,7 @@ asfd_status learned_init(asfd_plan_s* P, cudaStream_t st)
     LA(cyb, sizeof(float2) * P->prm.m2y);
     LA(lcorr, sizeof(float) * mm);
     LA(lcgrad, sizeof(float) * mm);
-    LA(lred, sizeof(double) * 2);
+    LA(lred, sizeof(double) * 3);
     LA(lpart, sizeof(float) * kBackBlocks * kMlpParams);
 #undef LA
     // the ES width-4 deconvolution/chirp tables become the base tables

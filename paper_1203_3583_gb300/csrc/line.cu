@@ -126,7 +126,7 @@ constexpr int kLineOneBlock = 1024;
 // Adds sample j's taps to the line (periodic).
 __device__ __forceinline__ void line_spread_sample(const LineArgs& a, int j)
 {
-    const float2 u = __ldg(&a.u1[j]), ej = __ldg(&a.e[j]);
+    const float2 u = a.u1[j], ej = __ldg(&a.e[j]);
     const float2 c = make_float2(u.x * ej.x - u.y * ej.y, u.x * ej.y + u.y * ej.x);
     const float f = __ldg(&a.bf[j]) - a.half_w;
     const float cf = ceilf(f);

@@ -101,7 +101,7 @@ __device__ __forceinline__ Raw load_raw(const Args& a, int nx, int ny)
     Raw r;
     const size_t n = (size_t)ny * a.n1x + nx;
     r.q = __ldg(&a.q[n]);
-    r.u = __ldg(&a.u1[n]);
+    r.u = a.u1[n];
     r.ex = a.ax[nx];
     r.ey = a.ay[ny];
     r.px = a.px[nx];
@@ -158,7 +158,7 @@ __device__ __forceinline__ void table_weights(const float* tab, float dx, float 
     const float tx = fmaf(2.0f, dx, -1.0f), ty = fmaf(2.0f, dy, -1.0f);
 #pragma unroll
     for (int i = 0; i < W; ++i) {
-        const float4 lo = __ldg(&t4[2 * i]), hi = __ldg(&t4[2 * i + 1]);
+        const float4 lo = t4[2 * i], hi = t4[2 * i + 1];
         float p = hi.w;
         p = fmaf(p, tx, hi.z);
         p = fmaf(p, tx, hi.y);
@@ -167,7 +167,7 @@ __device__ __forceinline__ void table_weights(const float* tab, float dx, float 
         p = fmaf(p, tx, lo.z);
         p = fmaf(p, tx, lo.y);
         wx[i] = fmaf(p, tx, lo.x);
-        const float4 lo2 = __ldg(&t4[2 * (W + i)]), hi2 = __ldg(&t4[2 * (W + i) + 1]);
+        const float4 lo2 = t4[2 * (W + i)], hi2 = t4[2 * (W + i) + 1];
         float q = hi2.w;
         q = fmaf(q, ty, hi2.z);
         q = fmaf(q, ty, hi2.y);

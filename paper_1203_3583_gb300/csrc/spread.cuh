@@ -450,7 +450,7 @@ __device__ __forceinline__ void window_tile(const SpreadArgs& a, int t, float2* 
         float2 ua = make_float2(0.f, 0.f), ub = make_float2(0.f, 0.f);
         if (slot_ok(0, 0)) {
             qa = __ldg(&a.q[(size_t)ny0 * a.n1x + nx0]);
-            ua = __ldg(&a.u1[(size_t)ny0 * a.n1x + nx0]);
+            ua = a.u1[(size_t)ny0 * a.n1x + nx0];
         }
         if (nsamp > 1) {
             int o1 = 0, j1 = 0;
@@ -458,7 +458,7 @@ __device__ __forceinline__ void window_tile(const SpreadArgs& a, int t, float2* 
             if (slot_ok(o1, j1)) {
                 const size_t n = (size_t)(ny0 + j1) * a.n1x + nx0 + o1;
                 qb = __ldg(&a.q[n]);
-                ub = __ldg(&a.u1[n]);
+                ub = a.u1[n];
             }
         }
         AxisEntry ex{};
@@ -469,7 +469,7 @@ __device__ __forceinline__ void window_tile(const SpreadArgs& a, int t, float2* 
             if (s + 2 < nsamp && slot_ok(oc, jc)) {
                 const size_t n = (size_t)(ny0 + jc) * a.n1x + nx0 + oc;
                 qc = __ldg(&a.q[n]);
-                uc = __ldg(&a.u1[n]);
+                uc = a.u1[n];
             }
             const bool v = slot_ok(o, j);
             const int nx = nx0 + o, ny = ny0 + j;
@@ -706,9 +706,8 @@ __device__ __forceinline__ void window_atomic_item(const SpreadArgs& a, int it, 
     auto load_tab = [&](int ty) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (TAB && lane < 8 * W && ty * kSrcTile < a.n1y)
-            v = __ldg(reinterpret_cast<const float4*>(a.table + ((size_t)ty * a.nstx + tcol) *
-                                                                   kLearnTableSize) +
-                      lane % (4 * W));
+            v = reinterpret_cast<const float4*>(a.table + ((size_t)ty * a.nstx + tcol) *
+                                                              kLearnTableSize)[lane % (4 * W)];
         return v;
     };
     float4 tnext = load_tab(ny0 / kSrcTile);
@@ -850,7 +849,7 @@ __device__ __forceinline__ void atomic_tile(const SpreadArgs& a, int tile, float
         const bool hitx = (cx0 < kTileX) || (cx0 + W - 1 > mx);
         const bool hity = (cy0 < kTileY) || (cy0 + W - 1 > my);
         if (!(hitx && hity)) continue;
-        const float2 c = sample_value(__ldg(&a.u1[n]), ex, ey, q, a.inc_d);
+        const float2 c = sample_value(a.u1[n], ex, ey, q, a.inc_d);
 
         float wx[W], wyv[W];
         if constexpr (TAB) {

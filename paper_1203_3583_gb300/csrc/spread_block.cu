@@ -386,14 +386,14 @@ __global__ void __launch_bounds__(32 * kDenseWarps) spread_fold_kernel(SpreadArg
     };
     size_t n = (size_t)ny0 * a.n1x + nx;
     float qn = __ldg(&a.q[n]);
-    float2 un = __ldg(&a.u1[n]);
+    float2 un = a.u1[n];
     for (int ny = ny0; ny <= nyl; ++ny) {
         const float q = qn;
         const float2 u = un;
         n += a.n1x;
         if (ny < nyl) {
             qn = __ldg(&a.q[n]);
-            un = __ldg(&a.u1[n]);
+            un = a.u1[n];
         }
         const AxisEntry ey = a.ay[ny];
         int l0x, l0y;

@@ -226,10 +226,10 @@ __global__ void __launch_bounds__(32 * kItemWarps) spread_item_kernel(ItemArgs i
 constexpr int kGatherRows = 4;
 
 __global__ void __launch_bounds__(128)
-item_gather_kernel(const float2* __restrict__ scratch, const int* __restrict__ xbox,
+item_gather_kernel(const float2* scratch, const int* __restrict__ xbox,
                    const int* __restrict__ ybox, const int* __restrict__ xmap,
                    const int* __restrict__ ymap, int x0, int y0, int bw, int bh, int ncb, int tw,
-                   int th, float2* __restrict__ grid, int nfx)
+                   int th, float2* grid, int nfx)
 {
     chain_next();
     chain_wait();
@@ -242,10 +242,10 @@ item_gather_kernel(const float2* __restrict__ scratch, const int* __restrict__ x
 #pragma unroll
     for (int k = 0; k < kItemMaxOverlap; ++k) tx[k] = k < ncx ? x - __ldg(&xbox[2 * (cb0 + k)]) : 0;
     const size_t tile = (size_t)th * tw;
+    float2 sums[kGatherRows];  // (all loads before the first store)
 #pragma unroll
     for (int r = 0; r < kGatherRows; ++r) {
-        const int by = blockIdx.y * kGatherRows + r;
-        if (by >= bh) break;
+        const int by = min((int)blockIdx.y * kGatherRows + r, bh - 1);
         const int y = y0 + by;
         const int ym = __ldg(&ymap[by]);
         const int rr0 = ym & 0xffffff, ncy = ym >> 24;
@@ -259,14 +259,19 @@ item_gather_kernel(const float2* __restrict__ scratch, const int* __restrict__ x
 #pragma unroll
                 for (int k = 0; k < kItemMaxOverlap; ++k) {
                     if (k < ncx) {
-                        const float2 v = __ldg(t + k * tile + tx[k]);
+                        const float2 v = t[k * tile + tx[k]];
                         s.x += v.x;
                         s.y += v.y;
                     }
                 }
             }
         }
-        grid[(size_t)y * nfx + x] = s;
+        sums[r] = s;
+    }
+#pragma unroll
+    for (int r = 0; r < kGatherRows; ++r) {
+        const int by = blockIdx.y * kGatherRows + r;
+        if (by < bh) grid[(size_t)(y0 + by) * nfx + x] = sums[r];
     }
 }
 
