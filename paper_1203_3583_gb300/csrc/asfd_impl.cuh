@@ -92,7 +92,7 @@ struct asfd_plan_s {
     double* bux = nullptr;          // unreduced alpha x~ + nf/2 per axis (plan only)
     double* buy = nullptr;
     float* q = nullptr;             // [n1y][n1x]  d1 / (z0 - d1)
-    float* q_next = nullptr;        // [n1y][n1x]  the same of a height map being checked (on need)
+    float* q_old = nullptr;         // [n1y][n1x]  the same while another map is checked (on need)
     float2* cx = nullptr;           // [m2x] destination chirp * (-1)^m' / psi_hat
     float2* cy = nullptr;           // [m2y] same, times the global factor
     float2* twx = nullptr;          // [nfx] e^{-2 pi i k/nfx}

@@ -107,11 +107,12 @@ constexpr int kStatRows = 64;       // rows whose coordinates it stages at a tim
 // above.  A thread takes a column over a chunk of rows: its x extremes are
 // those of q, mapped, as the coordinate is monotone in q; the spacing takes the
 // FP64 difference of neighbouring base coordinates and FP32 q terms (~1 cell,
-// good to ~1e-6 cells; the binning adds a one-cell margin).  An update's q
-// goes beside the plan's, so that a rejected map changes nothing.  (Four kernels
+// good to ~1e-6 cells; the binning adds a one-cell margin).  q is formed
+// in place (captured launches hold its address) and an update keeps the old one
+// aside, to put it back if the map is rejected.  (Four kernels
 // with three waits for their results, and loops over 4096 source tiles on the
 // host, left the GPU idle for 0.2 of a 0.41 ms optimisation step at 1024^2.)
-__global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* q,
+__global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* q, float* q_old,
                                                        const AxisEntry* ax, const AxisEntry* ay,
                                                        const double* bux, const double* buy,
                                                        int n1x, int n1y, double z0, float inv_z0,
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* 
     float qlo = 3e38f, qhi = -3e38f, ylo = 3e38f, yhi = -3e38f, mx = 3e38f, my = 3e38f;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *status = 0;
     float qn = in && r0 < r1 ? load(nx, r0) : 0.f;
+    float oldn = q_old && on && r0 < r1 ? q[(size_t)r0 * n1x + nx] : 0.f;
     // the rows' base coordinates, their FP64 differences and slopes in FP32, a
     // batch of rows at a time
     __shared__ float4 rows[kStatRows];
@@ -160,8 +162,12 @@ __global__ void __launch_bounds__(256) d1_stats_kernel(const double* d1, float* 
             const float qq = qn;
             const float qx = __shfl_down_sync(0xffffffffu, qq, 1);
             if (in && ny + 1 < n1y) qn = load(nx, ny + 1);
+            const float old = oldn;
+            if (q_old && on && ny + 1 < r1) oldn = q[(size_t)(ny + 1) * n1x + nx];
             if (on) {
-                q[(size_t)ny * n1x + nx] = qq;
+                const size_t n = (size_t)ny * n1x + nx;
+                if (q_old) q_old[n] = old;
+                q[n] = qq;
                 qlo = fminf(qlo, qq);
                 qhi = fmaxf(qhi, qq);
                 const float4 r = rows[ny - b0];
@@ -661,23 +667,23 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
 {
     const asfd_params& p = P->prm;
     const size_t nsrc = (size_t)p.n1x * p.n1y;
-    // where q of the new map waits to be accepted: in place for a new plan (which
-    // is given up with its map), else in a work buffer, which lies idle between
-    // calls; where none is large enough in a buffer of the plan's own
-    float* q_next = P->q;
+    // where the plan's old q waits until the new map is accepted (a new plan is
+    // given up with its map): a work buffer, which lies idle between calls, or where
+    // none is large enough a buffer of the plan's own
+    float* q_old = nullptr;
     if (!fresh) {
         const size_t bytes = sizeof(float) * nsrc;
         const size_t rows = sizeof(float2) * (size_t)P->nfy * row_buffer_width(p.m2x);
         const size_t grid = sizeof(float2) * (size_t)P->nfx * P->nfy;
         asfd_status s = ASFD_OK;
         if (P->ws) {
-            q_next = reinterpret_cast<float*>(P->stage_u1);  // 8 bytes per sample
+            q_old = reinterpret_cast<float*>(P->stage_u1);  // 8 bytes per sample
         } else if (bytes <= std::max(rows, grid)) {
             s = plan_ensure_work(P, kWorkTransform);
-            q_next = reinterpret_cast<float*>(bytes <= rows ? P->rows : P->grid);
+            q_old = reinterpret_cast<float*>(bytes <= rows ? P->rows : P->grid);
         } else {
-            if (!P->q_next) s = alloc_n(P, &P->q_next, nsrc);
-            q_next = P->q_next;
+            if (!P->q_old) s = alloc_n(P, &P->q_old, nsrc);
+            q_old = P->q_old;
         }
         if (s != ASFD_OK) return s;
     }
@@ -687,11 +693,12 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
     static_assert((65536 + kStatCols - 1) / kStatCols <= kStatBlocks, "n1x <= 65536 fits one row of blocks");
     const int sgx = (p.n1x + kStatCols - 1) / kStatCols;
     const int sgy = std::max(1, std::min(kStatBlocks / sgx, p.n1y));
-    d1_stats_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(d1, q_next, P->ax, P->ay, P->bux, P->buy, p.n1x,
-                                                    p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
+    d1_stats_kernel<<<dim3(sgx, sgy), 256, 0, st>>>(d1, P->q, q_old, P->ax, P->ay, P->bux, P->buy,
+                                                    p.n1x, p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
     ASFD_CUDA(cudaGetLastError());
     std::vector<float> stats((size_t)sgx * sgy * kStatWords);
-    // (to pageable memory: the call returns when the copy has ended)
+    // (to pageable memory: the call returns when the copy, and with it all work
+    // before it, has ended: from here on the new q is in place for every stream)
     ASFD_CUDA(cudaMemcpyAsync(stats.data(), P->stat, sizeof(float) * stats.size(), cudaMemcpyDeviceToHost,
                               st));
     const auto value = [&](int k) {
@@ -699,17 +706,24 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
         for (size_t b = k + kStatWords; b < stats.size(); b += kStatWords) m = std::max(m, stats[b]);
         return m;
     };
+    const auto put_back = [&]() -> asfd_status {
+        if (!q_old) return ASFD_OK;
+        ASFD_CUDA(cudaMemcpyAsync(P->q, q_old, sizeof(float) * nsrc, cudaMemcpyDeviceToDevice, st));
+        ASFD_CUDA(cudaStreamSynchronize(st));
+        return ASFD_OK;
+    };
+    asfd_status cs;
     if (value(kStatBad) != 0.f) {
+        if ((cs = put_back()) != ASFD_OK) return cs;
         cudaMemsetAsync(P->status, (int)kStatusBadD1, 1, st);  // (the word's low byte)
         return fail(ASFD_ERR_ARG, "d1 has a non-finite value or d1 >= z0");
     }
     const float me = value(kStatEps);
-    if (me > 0.1f)
+    if (me > 0.1f) {
+        if ((cs = put_back()) != ASFD_OK) return cs;
         return fail(ASFD_ERR_UNSUPPORTED, "max |d1|/z0 = " + std::to_string(me) +
                                               " exceeds the supported 0.1");
-    // (copied, not swapped: captured launches hold the plan's pointer)
-    if (q_next != P->q)
-        ASFD_CUDA(cudaMemcpyAsync(P->q, q_next, sizeof(float) * nsrc, cudaMemcpyDeviceToDevice, st));
+    }
 
     // 2. the band (fine-grid tiles that footprints reach) and the wrap flags
     const double hw = 0.5 * P->w + 1.0;  // half width plus a one-cell safety margin
@@ -741,7 +755,7 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
     P->band_ty1 = by1 + 1;
     P->max_abs_eps = me;
     P->wraps = wrapx || wrapy;
-    asfd_status cs = plan_build_colored(P, wrapx || wrapy, -value(kStatStepX), -value(kStatStepY), st);
+    cs = plan_build_colored(P, wrapx || wrapy, -value(kStatStepX), -value(kStatStepY), st);
     if (cs != ASFD_OK) return cs;
     P->tile_pairs = 0;
     if (!P->colored && !P->dense) {
@@ -800,9 +814,6 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
         ASFD_CUDA(cudaStreamSynchronize(st));
         P->tile_pairs = (long long)lst.size();
     }
-    // the plan is ready on every stream when this returns (the copy of q has run
-    // while the host chose the launches)
-    ASFD_CUDA(cudaStreamSynchronize(st));
     if (P->learned && P->lfeat) {
         cs = learned_features(P, st);
         if (cs != ASFD_OK) return cs;
