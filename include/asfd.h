@@ -141,8 +141,12 @@ asfd_status asfd_plan_create(asfd_plan* out, const asfd_params* p, const double*
 /* Replace the plan's height map (same sizes) and rebuild the d1-dependent
  * tables and binning.  Synchronises `stream`: the new map is in place, for
  * every stream, when the call returns.  Uses the plan's work buffers (not
- * concurrent with other calls on the plan).  Same errors as asfd_plan_create;
- * the plan is unchanged on failure. */
+ * concurrent with other calls on the plan).  A call captured into a CUDA graph
+ * keeps the launch shape and the band (asfd_plan_info) it was captured with: its
+ * replays transform the new map where that still fits (small changes of the
+ * heights); capture it again where the band or spread_kind has changed, or the
+ * samples' spacing by more than a few per cent.  Same errors as
+ * asfd_plan_create; the plan is unchanged on failure. */
 asfd_status asfd_plan_update_d1(asfd_plan plan, const double* d1_dev, void* stream);
 
 /*

@@ -310,7 +310,8 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
     const int gy0 = ylo, gy1 = ba.ybox[2 * by + 1];
     const int band_x1 = (a.band_tx0 + a.band_ntx) * kTileX;
     const int xb = max(gx0, a.band_tx0 * kTileX), xe = min(gx1, band_x1);
-    const int yb = max(gy0, 0), ye = min(gy1, a.nfy);
+    // (gy0 + th: the boxes of a replayed launch may be those of a later map)
+    const int yb = max(gy0, 0), ye = min(min(gy1, a.nfy), gy0 + th);
     const int across = max(1, (xe - xb + 31) / 32) * 32;          // threads along x
     const int parts = max(1, (int)blockDim.x / across);           // shares of the rows
     const int part = (int)threadIdx.x / across;
@@ -485,63 +486,100 @@ asfd_status plan_build_block(asfd_plan_s* P, const std::vector<double>& cr,
         for (size_t i = 0; i < b.size(); i += 2) m = std::max(m, b[i + 1] - b[i]);
         return m;
     };
-    int dev = 0, sms = 0;
-    ASFD_CUDA(cudaGetDevice(&dev));
-    ASFD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // (beyond 64 samples per kernel width: see ACCURATE)
-    const bool dup = P->min_step_x < 1.0 + 1e-3 || w + 0.01 > 64.0 * P->min_step_x ||
-                     w + P->row_spread_y + 0.01 > 64.0 * P->min_step_y;
+    bool dup = P->min_step_x < 1.0 + 1e-3 || w + 0.01 > 64.0 * P->min_step_x ||
+               w + P->row_spread_y + 0.01 > 64.0 * P->min_step_y;
+    std::vector<int> xb, yb;
+    int warps = P->blk_warps, chunks = P->blk_chunks, rows = P->blk_rows, tw = P->blk_tw, th = P->blk_th;
+    // A captured call replays with the shape it was captured with, on the new map's
+    // boxes: that shape is kept while it serves the map.
+    bool keep = P->captured && rows > 0 && (P->blk_dup || !dup);
+    if (keep) {
+        xb = boxes(cr, p.n1x, HC * chunks);
+        yb = boxes(rr, p.n1y, rows);
+        keep = separate(xb, warps) && separate(yb, 1) && widest(xb) - w + WS <= tw && widest(yb) <= th;
+    }
+    dup = dup || (keep && P->blk_dup);
     const BlkKernel kern = dup ? blk_kernel<true>(w) : blk_kernel<false>(w);
     if (!kern) return ASFD_OK;
     // (process-wide, the same value for every plan)
     ASFD_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kBlkMaxSmem));
-    // columns: 4 warps of one chunk, more warps and then more chunks until
-    // blocks two apart are disjoint
-    int warps = 4, chunks = 1;
-    std::vector<int> xb;
-    for (;;) {
-        xb = boxes(cr, p.n1x, HC * chunks);
-        if (separate(xb, warps)) break;
-        if (warps < kBlkMaxWarps) warps *= 2;
-        else if ((long long)HC * chunks * warps < p.n1x) ++chunks;
-        else return ASFD_OK;
-    }
-    const int tw = widest(xb) - w + WS;
-    const int ncols = (int)xb.size() / 2, nbx = (ncols + warps - 1) / warps;
-    // rows: the fewest for disjoint blocks, then the count that ends soonest
-    // by a model in rows: whole waves of resident blocks per colour (a warp
-    // waits on its own chain of latencies, so a full SM takes no longer than
-    // one block), each of its rows and a fixed part (the empty and the last
-    // window, the merge)
-    double best = 1e300;
-    int rows = 0, th = 0;
-    std::vector<int> yb;
-    for (int r = 8; r < 2 * p.n1y; r += std::max(1, r / 8)) {
-        const std::vector<int> b = boxes(rr, p.n1y, r);
-        if (!separate(b, 1)) continue;
-        const int h = widest(b);
-        const size_t smem = warps * (blk_ring(w) + sizeof(float2) * (size_t)S * tw * h);
-        if (smem > kBlkMaxSmem) break;
-        int per_sm = 0;
-        ASFD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)kern,
-                                                                32 * warps, smem));
-        if (per_sm < 1) break;
-        const int nby = (int)b.size() / 2;
-        double t = 0.0;
-        for (int c = 0; c < 4; ++c) {
-            const long long blocks = (long long)((nbx + 1 - (c & 1)) / 2) * ((nby + 1 - c / 2) / 2);
-            const long long slots = (long long)sms * per_sm;
-            t += (double)((blocks + slots - 1) / slots) * (r * chunks + 2.0 * w + 8.0) + 4.0;
+    if (!keep) {
+        int dev = 0, sms = 0;
+        ASFD_CUDA(cudaGetDevice(&dev));
+        ASFD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        // columns: 4 warps of one chunk, more warps and then more chunks until
+        // blocks two apart are disjoint
+        warps = 4;
+        chunks = 1;
+        for (;;) {
+            xb = boxes(cr, p.n1x, HC * chunks);
+            if (separate(xb, warps)) break;
+            if (warps < kBlkMaxWarps) warps *= 2;
+            else if ((long long)HC * chunks * warps < p.n1x) ++chunks;
+            else return ASFD_OK;
         }
-        if (t < best) {
-            best = t;
-            rows = r;
-            th = h;
-            yb = b;
+        tw = widest(xb) - w + WS;
+        const auto bytes = [&](int tw_, int th_) {
+            return warps * (blk_ring(w) + sizeof(float2) * (size_t)S * tw_ * th_);
+        };
+        const auto resident = [&](size_t smem, int* per_sm) -> asfd_status {
+            ASFD_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, (const void*)kern,
+                                                                    32 * warps, smem));
+            return ASFD_OK;
+        };
+        const int nc = (int)xb.size() / 2, nbx = (nc + warps - 1) / warps;
+        // rows: the fewest for disjoint blocks, then the count that ends soonest
+        // by a model in rows: whole waves of resident blocks per colour (a warp
+        // waits on its own chain of latencies, so a full SM takes no longer than
+        // one block), each of its rows and a fixed part (the empty and the last
+        // window, the merge)
+        double best = 1e300;
+        int best_per_sm = 0;
+        asfd_status s;
+        rows = 0;
+        for (int r = 8; r < 2 * p.n1y; r += std::max(1, r / 8)) {
+            const std::vector<int> b = boxes(rr, p.n1y, r);
+            if (!separate(b, 1)) continue;
+            const int h = widest(b);
+            const size_t smem = bytes(tw, h);
+            if (smem > kBlkMaxSmem) break;
+            int per_sm = 0;
+            if ((s = resident(smem, &per_sm)) != ASFD_OK) return s;
+            if (per_sm < 1) break;
+            const int nby = (int)b.size() / 2;
+            double t = 0.0;
+            for (int c = 0; c < 4; ++c) {
+                const long long blocks = (long long)((nbx + 1 - (c & 1)) / 2) * ((nby + 1 - c / 2) / 2);
+                const long long slots = (long long)sms * per_sm;
+                t += (double)((blocks + slots - 1) / slots) * (r * chunks + 2.0 * w + 8.0) + 4.0;
+            }
+            if (t < best) {
+                best = t;
+                best_per_sm = per_sm;
+                rows = r;
+                th = h;
+                yb = b;
+            }
+        }
+        if (rows == 0) {
+            P->blk_rows = 0;
+            return ASFD_OK;
+        }
+        // room for footprints that move by a cell or two in later maps (above),
+        // where it costs no resident block
+        for (int e = 2; e > 0; --e) {
+            int per_sm = 0;
+            if (bytes(tw + e, th + e) > kBlkMaxSmem) continue;
+            if ((s = resident(bytes(tw + e, th + e), &per_sm)) != ASFD_OK) return s;
+            if (per_sm < best_per_sm) continue;
+            tw += e;
+            th += e;
+            break;
         }
     }
-    if (rows == 0) return ASFD_OK;
+    const int ncols = (int)xb.size() / 2;
     asfd_status s;
     if (!P->blk_xbox) {  // sized for the most groups of any height map
         const size_t n = (size_t)((p.n1x + HC - 1) / HC) + (size_t)((p.n1y + 7) / 8);
@@ -556,7 +594,7 @@ asfd_status plan_build_block(asfd_plan_s* P, const std::vector<double>& cr,
     P->blk_chunks = chunks;
     P->blk_rows = rows;
     P->blk_ncols = ncols;
-    P->blk_nbx = nbx;
+    P->blk_nbx = (ncols + warps - 1) / warps;
     P->blk_nby = (int)yb.size() / 2;
     P->blk_tw = tw;
     P->blk_th = th;

@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(128)
 item_gather_kernel(const float2* scratch, const int* __restrict__ xbox,
                    const int* __restrict__ ybox, const int* __restrict__ xmap,
                    const int* __restrict__ ymap, int x0, int y0, int bw, int bh, int ncb, int tw,
-                   int th, float2* grid, int nfx)
+                   int th, int items, float2* grid, int nfx)
 {
     chain_next();
     chain_wait();
@@ -255,10 +255,12 @@ item_gather_kernel(const float2* scratch, const int* __restrict__ xbox,
             if (j < ncy) {
                 const int rr = rr0 + j;
                 const int ty = y - __ldg(&ybox[2 * rr]);
+                // (outside only where a replayed launch meets a later map's boxes)
+                const bool in = (unsigned)ty < (unsigned)th && rr * ncb + cb0 + ncx <= items;
                 const float2* t = scratch + ((size_t)(rr * ncb + cb0) * th + ty) * tw;
 #pragma unroll
                 for (int k = 0; k < kItemMaxOverlap; ++k) {
-                    if (k < ncx) {
+                    if (k < ncx && in && (unsigned)tx[k] < (unsigned)tw) {
                         const float2 v = t[k * tile + tx[k]];
                         s.x += v.x;
                         s.y += v.y;
@@ -425,7 +427,7 @@ asfd_status launch_spread_itemtile(asfd_plan_s* P, const float2* u1, cudaStream_
     e = launch_chained(item_gather_kernel, dim3((bw + 127) / 128, (bh + kGatherRows - 1) / kGatherRows),
                        128, 0, st, (const float2*)P->rows, (const int*)P->it_xbox,
                        (const int*)P->it_ybox, (const int*)P->it_xmap, (const int*)P->it_ymap, bx0, by0,
-                       bw, bh, P->it_ncb, P->it_tw, P->it_th, P->grid, P->nfx);
+                       bw, bh, P->it_ncb, P->it_tw, P->it_th, P->it_items, P->grid, P->nfx);
     if (e != cudaSuccess) return cuda_fail(e, "item_gather_kernel launch");
     return ASFD_OK;
 }
