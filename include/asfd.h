@@ -413,8 +413,8 @@ const char* asfd_status_string(asfd_status s);
 const char* asfd_last_error(void);
 
 /*
- * Test hooks for the failure paths (no counterpart in the paper; neither
- * call touches the GPU).
+ * Test hooks for the failure paths and the choice of the spread (no
+ * counterpart in the paper; no call touches the GPU).
  *
  * asfd_debug_fail_allocations(n): the next n device allocations made for 2D
  * plans (asfd_plan_create, asfd_plan_update_d1, learned tables, batch
@@ -424,9 +424,17 @@ const char* asfd_last_error(void);
  *
  * asfd_debug_live_buffers(): the device buffers currently held by all 2D
  * plans of the process (a failed asfd_plan_create must leave it unchanged).
+ *
+ * asfd_debug_spread_path(plan, out): which spread the plan uses (spread_kind
+ * names kinds of results and shares some): out[0] = 0 conflict-free tiles,
+ * 1 wrapped windows, 2 the tiles with sliding windows, 3 the default windows,
+ * 4 item tiles, 5 block items; for block items out[1..4] = warps per block,
+ * column chunks per warp, rows per block, 1 where samples may share cells
+ * (else 0).  Returns ASFD_ERR_ARG for NULL.
  */
 void asfd_debug_fail_allocations(int n);
 long long asfd_debug_live_buffers(void);
+asfd_status asfd_debug_spread_path(asfd_plan plan, int out[5]);
 
 /*
  * Sum of several surfaces' fields at one destination (e.g. the polygons of

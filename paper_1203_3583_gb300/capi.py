@@ -119,6 +119,7 @@ SIGNATURES = {
     "asfd_last_error": (ctypes.c_char_p, []),
     "asfd_debug_fail_allocations": (None, [_int]),
     "asfd_debug_live_buffers": (ctypes.c_longlong, []),
+    "asfd_debug_spread_path": (_int, [_vp, ctypes.POINTER(_int)]),
     "asfd_fft_lines": (_int, [_int, _int, _int, _vp, _vp, _vp]),
     "asfd_direct_sum": (_int, [ctypes.POINTER(Params), _vp, _vp, _int, _int, _vp, _vp, _vp, _vp]),
     "asfd_line_plan_create": (_int, [ctypes.POINTER(_vp), ctypes.POINTER(LineParams), _vp, _vp,

@@ -94,6 +94,18 @@ void asfd_debug_fail_allocations(int n) { asfd::g_alloc_budget.store(n < 0 ? -1 
 
 long long asfd_debug_live_buffers(void) { return asfd::g_live_buffers.load(); }
 
+asfd_status asfd_debug_spread_path(asfd_plan P, int out[5])
+{
+    clear_error();
+    if (!P || !out) return fail(ASFD_ERR_ARG, "NULL argument");
+    out[0] = P->itemtile ? 4 : P->blk ? 5 : P->dense ? 3 : P->fold ? 1 : P->windowed ? 2 : 0;
+    out[1] = P->blk ? P->blk_warps : 0;
+    out[2] = P->blk ? P->blk_chunks : 0;
+    out[3] = P->blk ? P->blk_rows : 0;
+    out[4] = P->blk && P->blk_dup ? 1 : 0;
+    return ASFD_OK;
+}
+
 asfd_status asfd_plan_create(asfd_plan* out, const asfd_params* p, const double* d1_dev,
                              void* stream)
 {

@@ -308,7 +308,8 @@ asfd_status plan_build_itemtile(asfd_plan_s* P, cudaStream_t st)
     long long slots = 0;
     asfd_status s = item_slots(P->w, &slots);
     if (s != ASFD_OK) return s;
-    const int rows0 = window_run_rows(p.n1y, ncb, slots);
+    // (the default spread's shorter runs on tiny grids are none for tiles)
+    const int rows0 = std::max(kItemMinRows, window_run_rows(p.n1y, ncb, slots));
     // tables: per column block, per run (sized for the shortest runs tried)
     // and per fine column / row; each allocated once, a refused one retried
     const long long max_runs = (p.n1y + kItemMinRows - 1) / kItemMinRows;
