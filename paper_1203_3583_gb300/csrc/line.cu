@@ -148,10 +148,21 @@ __global__ void __launch_bounds__(256) line_spread_kernel(LineArgs a)
     if (j < a.n) line_spread_sample(a, j);
 }
 
+// Threads of the transform's block, at most: as many as there are samples to
+// spread, or as transform the line; 512 for 8192 points, whose 32 values per
+// thread fit the 128 registers that leaves (64 of a block of 1024: 324 bytes of
+// spills).
+template <int L, bool SPREAD>
+__host__ __device__ constexpr int line_threads()
+{
+    constexpr int tpl = FftShape<L>::TPL < 32 ? 32 : FftShape<L>::TPL;
+    return !SPREAD ? tpl : L == 8192 ? 512 : 1024;
+}
+
 // The block spreads the samples (SPREAD), and its first TPL threads transform
 // the line, leave it zero for the next call and write the destination.
 template <int L, bool SPREAD>
-__global__ void __launch_bounds__(1024) line_transform_kernel(LineArgs a)
+__global__ void __launch_bounds__(line_threads<L, SPREAD>()) line_transform_kernel(LineArgs a)
 {
     extern __shared__ float2 sm[];
     chain_next();
@@ -197,9 +208,9 @@ cudaError_t line_launch(const LineArgs& a, bool spread, cudaStream_t st)
         if (attr != cudaSuccess) return attr;
     }
     if (!spread)
-        return launch_chained(line_transform_kernel<L, false>, dim3(1), TPL < 32 ? 32 : TPL, smem, st,
-                              a);
-    int threads = std::min(1024, (a.n + 31) / 32 * 32);
+        return launch_chained(line_transform_kernel<L, false>, dim3(1), line_threads<L, false>(), smem,
+                              st, a);
+    int threads = std::min(line_threads<L, true>(), (a.n + 31) / 32 * 32);
     threads = std::max(threads, std::max(32, TPL));
     return launch_chained(line_transform_kernel<L, true>, dim3(1), (unsigned)threads, smem, st, a);
 }
