@@ -11,6 +11,7 @@ torch = pytest.importorskip("torch")
 
 from paper_1203_3583_gb300 import capi, workloads as W  # noqa: E402
 from paper_1203_3583_gb300.fresnel import FresnelPlan  # noqa: E402
+from tests.test_gpu_spread_block import GRIDS, case  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -33,3 +34,38 @@ def test_small_repeatable_plans_take_item_tiles(n, alpha):
     g = W.geometry(n, n, p1, p1, m, m, p2, p2, lam, z0)
     with FresnelPlan(g, np.zeros((n, n)), deterministic=True) as plan:
         assert spread_path(plan)[0] == ITEM_TILES
+
+
+# (grid of test_gpu_spread_block, width): the block's shape is checked where it is the point
+BLOCK = [(name, w) for name in GRIDS for w in (8, 9, 12, 13, 16)] + \
+        [(name, 7) for name in ("dense", "denser", "half", "sliver")]
+
+
+@pytest.mark.parametrize("name,width", BLOCK)
+def test_block_items(name, width):
+    """Monotone maps at widths above 7, and repeatable plans whose samples are less
+    than a cell apart: block items, the oracle's field and equal bits in two runs."""
+    g, u1, d1, ref = case(name)
+    with FresnelPlan(g, d1, kernel_width=width, deterministic=width == 7) as plan:
+        path, warps, chunks, rows, dup = spread_path(plan)
+        u = torch.as_tensor(u1, device="cuda")
+        a = plan.execute(u)
+        b = plan.execute(u)
+        torch.cuda.synchronize()
+    assert path == BLOCK_ITEMS
+    assert dup == (1 if GRIDS[name][4] < 1.0 else 0)
+    if name == "denser" and width > 7:  # blocks two apart meet unless warps take chunks in turn
+        assert warps == 8 and chunks > 1
+    assert torch.equal(a, b)
+    err = np.linalg.norm(a.cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err < max(3.0 * 10.0 ** (-(width - 1)), 5e-6), (name, width, err)
+
+
+@pytest.mark.parametrize("width", [7, 8, 16])
+@pytest.mark.parametrize("deterministic", [False, True])
+def test_wrapping_maps_take_wrapped_windows(width, deterministic):
+    lam, z0, p1, m, n = 633e-9, 0.06, 8e-6, 64, 150
+    p2 = 1.3 * lam * z0 / (p1 * 2 * m)
+    g = W.geometry(n, n, p1, p1, m, m, p2, p2, lam, z0)
+    with FresnelPlan(g, np.zeros((n, n)), kernel_width=width, deterministic=deterministic) as plan:
+        assert spread_path(plan)[0] == WRAPPED
