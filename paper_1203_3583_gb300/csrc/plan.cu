@@ -415,6 +415,17 @@ bool pow2_in(int n, int lo, int hi) { return n >= lo && n <= hi && (n & (n - 1))
 // at 0.49, whose band is large: 62.3, 69.3.
 constexpr double kDupSpacing = 0.45;
 
+// Fine cells per sample above which conflict-free tiles spread faster than block
+// items: kSparse per unit of kernel width (fewer than 2 w samples then reach a
+// cell), kSparseWindow for the sliding-window tiles of widths up to 7.  Around the
+// lines either can be the faster by a fifth.  Whole transforms, block items and
+// tiles (us):
+//   w7, 700^2   1.69 cells  85,  82    3.8  108,  60    6.3  135,  83    9  217, 121
+//   w8, 256^2   2.25        59, 103    3.8   79,  71    4.8   87,  58    9  112,  47
+//   w12, 700^2  3.8        115, 230    4.8  144, 191    6.3  155, 146    9  316, 276
+//   w14, 256^2  4.8        128, 281    6.3  156, 200    9    194, 144   16  231, 130
+constexpr double kSparse = 0.5, kSparseWindow = 2.5;
+
 asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double msy, cudaStream_t st);
 
 asfd_status plan_alloc_buffer(asfd_plan_s* P, void** p, size_t bytes) { return alloc(P, p, bytes); }
@@ -894,23 +905,27 @@ asfd_status plan_build_colored(asfd_plan_s* P, bool wraps, double msx, double ms
     for (int nx = 0; nx < p.n1x; ++nx) spread_x = std::max(spread_x, cr[2 * nx + 1] - cr[2 * nx]);
     P->row_spread_y = spread_y;
     P->col_spread_x = spread_x;
-    if (p.kind == ASFD_KERNEL_ES) {
-        // per-item tiles and a gather where they apply (2048^2 w7: 100 us against
-        // 137 us for block items), else block items
-        asfd_status s = plan_build_itemtile(P, st);
-        if (s == ASFD_OK && !P->itemtile) s = plan_build_block(P, cr, rr, st);
-        if (s != ASFD_OK) return s;
-    }
-    const bool placed = P->itemtile || P->blk;
-    if (P->w > kMaxRingWidth) return placed ? ASFD_OK : fold();
+    // the conflict-free tiles apply up to 64 samples between lanes (beyond, with
+    // samples packed far below one cell apart, few lanes find work in a tile)
     const double margin = 0.01;
     const double sxd = std::ceil((P->w + margin) / msx);
     const double hd = std::ceil((P->w + spread_y + margin) / msy);
     // the register-window tiles also need columns w apart across rows
     const double sxw = std::ceil((P->w + spread_x + margin) / msx);
-    // beyond 64 samples between lanes (samples packed far below one cell
-    // apart) few lanes find work in a tile and the atomic windows are faster
-    if (!(sxd <= 64.0) || !(hd <= 64.0)) return placed ? ASFD_OK : fold();
+    const bool tiles = P->w <= kMaxRingWidth && sxd <= 64.0 && hd <= 64.0;
+    if (p.kind == ASFD_KERNEL_ES) {
+        // per-item tiles and a gather where they apply (2048^2 w7: 100 us against
+        // 137 us for block items), else block items
+        asfd_status s = plan_build_itemtile(P, st);
+        // unless samples lie so far apart that the block items' windows start anew
+        // at almost every sample, while the tiles' 32 lanes need few steps: cells
+        // per sample against kSparse (a captured plan keeps the items of its replays)
+        const double line = P->w <= kMaxWindowWidth ? kSparseWindow : kSparse * P->w;
+        const bool sparse = tiles && msx * msy > line && !(P->captured && P->blk_rows > 0);
+        if (s == ASFD_OK && !P->itemtile && !sparse) s = plan_build_block(P, cr, rr, st);
+        if (s != ASFD_OK) return s;
+    }
+    if (!tiles) return P->itemtile || P->blk ? ASFD_OK : fold();
 
     // per band tile: source columns whose x range meets the tile's x range
     // widened by half a kernel and a cell, likewise rows (ranges are

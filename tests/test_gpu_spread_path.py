@@ -9,6 +9,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle  # noqa: E402
 from paper_1203_3583_gb300 import capi, workloads as W  # noqa: E402
 from paper_1203_3583_gb300.fresnel import FresnelPlan  # noqa: E402
 from tests.test_gpu_spread_block import GRIDS, case  # noqa: E402
@@ -69,3 +70,31 @@ def test_wrapping_maps_take_wrapped_windows(width, deterministic):
     g = W.geometry(n, n, p1, p1, m, m, p2, p2, lam, z0)
     with FresnelPlan(g, np.zeros((n, n)), kernel_width=width, deterministic=deterministic) as plan:
         assert spread_path(plan)[0] == WRAPPED
+
+
+CONFLICT_FREE, SLIDING = 0, 2
+
+
+@pytest.mark.parametrize("width,deterministic,sparse", [(4, True, 2.5), (7, True, 2.5), (8, False, 4.0),
+                                                        (12, False, 6.0), (14, False, 7.0)])
+@pytest.mark.parametrize("ratio", [1.0, 2.0])
+def test_sparse_maps_take_conflict_free_tiles(width, deterministic, sparse, ratio):
+    """Fine cells per sample on both sides of the line (their product counts), and the
+    oracle's field there."""
+    lam, z0, p1, n = 633e-9, 0.06, 8e-6, 44
+    rng = np.random.default_rng(width)
+    for cells, paths in ((0.93 * sparse, (ITEM_TILES, BLOCK_ITEMS)),
+                         (1.07 * sparse, (ITEM_TILES, SLIDING if width <= 7 else CONFLICT_FREE))):
+        ax, ay = np.sqrt(cells * ratio), np.sqrt(cells / ratio)
+        m = 128
+        g = W.geometry(n, n, p1, p1, m, m, ax * lam * z0 / (p1 * 2 * m), ay * lam * z0 / (p1 * 2 * m),
+                       lam, z0)
+        d1 = W.surface_smooth_random(g, rng, 8.0, 10e-6)
+        u1 = W.field_random_amp_phase(g, rng)
+        with FresnelPlan(g, d1, kernel_width=width, deterministic=deterministic) as plan:
+            path = spread_path(plan)[0]
+            out = plan.execute(torch.as_tensor(u1, device="cuda")).cpu().numpy()
+        assert path in (paths if width <= 7 else paths[1:]), (cells, path)
+        ref = oracle.eq7(g, u1, d1)
+        err = np.linalg.norm(out - ref) / np.linalg.norm(ref)
+        assert err < max(3.0 * 10.0 ** (-(width - 1)), 5e-6), (cells, path, err)
