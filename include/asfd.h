@@ -168,7 +168,8 @@ asfd_status asfd_plan_update_d1(asfd_plan plan, const double* d1_dev, void* stre
  * caller owns (e.g. a tensor of PyTorch's caching allocator) and must keep
  * alive, and not use otherwise, while calls on the plan can run.  Work
  * buffers the plan had allocated itself are freed.  With a workspace set, no
- * call on the plan allocates device memory.  ws_dev = NULL with bytes = 0
+ * call on the plan allocates device memory, and each transform first clears the
+ * part of the fine grid that it adds into (another plan may have used it).  ws_dev = NULL with bytes = 0
  * detaches the workspace; the plan then allocates its own work buffers again
  * on first use.  Without a workspace a plan allocates its work buffers at the
  * first call that needs them (asfd_execute, asfd_execute_stage,

@@ -19,8 +19,8 @@
 // indices and their sum are then exact modulo 2^64, which is the reduction
 // modulo one turn.  (With FP64 arithmetic per pair -- 2 lanes per clock and
 // SM, where integer multiply-adds have 64 -- and one block per point group 256
-// points of 1024^2 samples took 28.6 ms; now 0.45 ms, at an error against 64
-// bits of 5.1e-8 instead of 6.2e-8.)
+// points of 1024^2 samples took 28.6 ms; now 0.46 ms, at an error against 64
+// bits of 5e-8 instead of 6e-8.)
 //   Eq. 2: 2 (s.x1 + sz d1 + r)/lambda half-turns, amplitude 1/r^2,
 //          r = |(x2 - x1, z0 - d1)|, in FP64 from an FP32 reciprocal square
 //          root and its residual to third order (as good as an FP64 square
@@ -203,7 +203,7 @@ __host__ __device__ constexpr int direct_blocks_per_sm(int form)
 
 // Point groups in x, sample chunks in y: the chunk's sums over its samples of
 // kDirectPoints points, to part[chunk][point].  Bound by the FMA pipe and
-// instruction issue together (69 and 55 % busy: 12 packed operations, 4
+// instruction issue together (60 and 55 % busy: 12 packed operations, 4
 // integer multiply-adds and 10 integer operations a pair), so more resident
 // warps, a sample's loads one iteration ahead and one exact wave of blocks
 // made no difference (0.39-0.42 ms against 0.385 ms at 256 points of 1024^2

@@ -29,12 +29,12 @@
 // What bounds it: a warp's chain of latencies per source row (ring, position,
 // phases), at 8 warps per SM (230 registers at W = 12: 144 are the window).
 // Measured, whole transforms, against the conflict-free tiles and, for maps
-// denser than 64 samples per kernel width, the shared-memory float atomics that
-// these maps took before (us):
-//   2048^2, 1.04 cells per sample   w8 501 -> 217, w12 1465 -> 359, w16 3470 -> 707
-//   600^2 onto 256^2 (0.4 cells)    w7 346 -> 124, w8 817 -> 89, w12 2617 -> 130
-//   1300 x 1258 onto 64^2 (0.03)    w7 199000 -> 818, w12 584000 -> 4980
-//   4096^2, 1.44 cells, w7          1871 -> 1184
+// denser than 64 samples per kernel width and widths above 14, the shared-memory
+// float atomics that these maps took before (us):
+//   2048^2, 1.04 cells per sample   w8 506 -> 218, w12 1407 -> 356, w16 3433 -> 695
+//   600^2 onto 256^2 (0.4 cells)    w7 487 -> 109, w8 1221 -> 93, w12 3774 -> 139
+//   1300 x 1258 onto 64^2 (0.03)    w7 211500 -> 1789, w12 606400 -> 5317
+// Maps whose samples lie cells apart keep the tiles (kSparse in plan.cu).
 // Sharing a column between 4 lanes at W = 12 (half the registers, twice the
 // steps) took 1.45 times as long.
 #include <algorithm>
@@ -351,9 +351,9 @@ __global__ void __launch_bounds__(32 * kBlkMaxWarps) spread_block_kernel(BlkArgs
 // fine grid with float2 atomic adds.  Warp item `it` takes 32 / S columns over
 // dense_rows rows.  Any map is handled: a sample that does not continue its
 // lane's window flushes it.  (Shared-memory tiles with float atomics, a
-// compare-and-swap loop each and one block per 64 x 64 cells, took 1.6 ms for
-// a wrapping 1024^2 onto 512^2 at w12, now 0.14; 388 ms for 1300 x 1258 onto
-// 64^2, now 0.20; 1.1 ms for a folding 1024^2, now 0.72.)
+// compare-and-swap loop each and one block per 64 x 64 cells, took 1093 us for a
+// wrapping 1024^2 onto 512^2 at w12, now 59; 205 ms for 1300 x 1258 onto 64^2, now
+// 0.09; 1178 us for a folding 1024^2, now 304.)
 template <int W>
 __global__ void __launch_bounds__(32 * kDenseWarps) spread_fold_kernel(SpreadArgs a)
 {
