@@ -708,10 +708,10 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
                                                     p.n1x, p.n1y, p.z0, (float)(1.0 / p.z0), P->status, P->stat);
     ASFD_CUDA(cudaGetLastError());
     std::vector<float> stats((size_t)sgx * sgy * kStatWords);
-    // (to pageable memory: the call returns when the copy, and with it all work
-    // before it, has ended: from here on the new q is in place for every stream)
     ASFD_CUDA(cudaMemcpyAsync(stats.data(), P->stat, sizeof(float) * stats.size(), cudaMemcpyDeviceToHost,
                               st));
+    // (the only wait: from here on the new q is in place for every stream)
+    ASFD_CUDA(cudaStreamSynchronize(st));
     const auto value = [&](int k) {
         float m = stats[k];
         for (size_t b = k + kStatWords; b < stats.size(); b += kStatWords) m = std::max(m, stats[b]);
