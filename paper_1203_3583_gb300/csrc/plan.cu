@@ -828,7 +828,8 @@ asfd_status plan_build_d1(asfd_plan_s* P, const double* d1, bool fresh, cudaStre
     if (P->learned && P->lfeat) {
         cs = learned_features(P, st);
         if (cs != ASFD_OK) return cs;
-        return learned_refresh(P, st);
+        if ((cs = learned_refresh(P, st)) != ASFD_OK) return cs;
+        ASFD_CUDA(cudaStreamSynchronize(st));  // (its tables too, for every stream)
     }
     return ASFD_OK;
 }

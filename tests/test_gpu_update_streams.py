@@ -12,8 +12,9 @@ from paper_1203_3583_gb300.fresnel import FresnelPlan  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("deterministic", [False, True])
-def test_nothing_is_left_on_the_stream(deterministic):
+@pytest.mark.parametrize("kw", [dict(), dict(deterministic=True), dict(kind="learned")],
+                         ids=["default", "repeatable", "learned"])
+def test_nothing_is_left_on_the_stream(kw):
     m = 512
     lam, z0, p1 = 633e-9, 0.06, 1e-6
     p2 = 0.05 * lam * z0 / (p1 * 2 * m)
@@ -21,7 +22,7 @@ def test_nothing_is_left_on_the_stream(deterministic):
     d1 = torch.zeros((4096, 16384), dtype=torch.float64, device="cuda")
     other = torch.full_like(d1, 1e-5)
     s = torch.cuda.Stream()
-    with FresnelPlan(g, d1, deterministic=deterministic) as plan:
+    with FresnelPlan(g, d1, **kw) as plan:
         torch.cuda.synchronize()
         for heights in (other, d1, other, d1):
             plan.update_d1(heights, stream=s)
